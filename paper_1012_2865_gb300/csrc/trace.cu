@@ -116,14 +116,14 @@ __device__ __forceinline__ void acc_flush(LaneAcc& a, const TraceArgs& A, const 
   if (a.inst >= 0 && a.inst < bb.nrows) {
     // straight-line reductions (adding zeros costs less than branching)
     double* t = bb.rows + kBlkRow * a.inst;
-    atomicAdd(&t[0], a.emitted);
-    atomicAdd(&t[1], a.absorbed);
-    atomicAdd(&t[2], a.escaped);
+    red_add(&t[0], a.emitted);
+    red_add(&t[1], a.absorbed);
+    red_add(&t[2], a.escaped);
     if (a.resumed != 0.0 || a.halted != 0.0) {
-      atomicAdd(&t[3], a.resumed);
-      atomicAdd(&t[4], a.halted);
+      red_add(&t[3], a.resumed);
+      red_add(&t[4], a.halted);
     }
-    atomicAdd(reinterpret_cast<unsigned long long*>(&t[kAcc]), a.segments);
+    red_add(reinterpret_cast<unsigned long long*>(&t[kAcc]), a.segments);
     if (a.fallbacks | a.fallbacks_tau) {
       atomicAdd(&bb.fb[2 * a.inst], a.fallbacks);
       atomicAdd(&bb.fb[2 * a.inst + 1], a.fallbacks_tau);
@@ -346,15 +346,15 @@ struct Walk64 {
       }
     }
     const double kadd = P * w * dr * phi * fcv;
-    atomicAdd(&K[idx], kadd);
-    if (heat != 0.0) atomicAdd(&G[idx], kadd * heat);
+    red_add(&K[idx], kadd);
+    if (heat != 0.0) red_add(&G[idx], kadd * heat);
     if (dr > 0) nseg++;
     P = P - P * am;
     tau = __dadd_rn(tau, dtau);
     if (tau > A.tau_term) {
       const double kres = P * rw / nh * fcv;
-      atomicAdd(&K[idx], kres);
-      if (heat != 0.0) atomicAdd(&G[idx], kres * heat);
+      red_add(&K[idx], kres);
+      if (heat != 0.0) red_add(&G[idx], kres * heat);
       acc.absorbed += Pstart * unit(A);
       return EV_DONE;
     }
@@ -859,8 +859,8 @@ struct Walk32 {
       }
     }
     const float kadd = P * k32.y * dr * phi * fcv;
-    atomicAdd(&K[idx], kadd);
-    if (k32.w != 0.0f) atomicAdd(&G[idx], kadd * k32.w);
+    red_add(&K[idx], kadd);
+    if (k32.w != 0.0f) red_add(&G[idx], kadd * k32.w);
     if (dr > 0.0f) nseg++;
     P = P * tr;
     {
@@ -895,8 +895,8 @@ struct Walk32 {
       if (term) {
         if (nh > 0.0f) {
           const float kres = P * k32.z / nh * fcv;
-          atomicAdd(&K[idx], kres);
-          if (k32.w != 0.0f) atomicAdd(&G[idx], kres * k32.w);
+          red_add(&K[idx], kres);
+          if (k32.w != 0.0f) red_add(&G[idx], kres * k32.w);
         }
         acc.absorbed += (double)Pstart * unit(A);
         return EV_DONE;
