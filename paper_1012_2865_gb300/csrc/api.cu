@@ -23,8 +23,9 @@ namespace rtg {
 cudaError_t launch_trace_init(unsigned long long* ctl, void* queue, size_t queue_bytes, unsigned long long n_roots,
                               int first_pass, int mode, unsigned long long in_cap, int pass, int passes,
                               cudaStream_t st);
-cudaError_t trace_occupancy(int precision, int fsl, int block, int* blocks_per_sm);
-cudaError_t launch_trace(int precision, int fsl, const TraceArgs& A, int grid, int block, cudaStream_t st);
+cudaError_t trace_occupancy(int precision, int fsl, int variant, int block, int* blocks_per_sm);
+cudaError_t launch_trace(int precision, int fsl, int variant, const TraceArgs& A, int grid, int block,
+                         cudaStream_t st);
 cudaError_t launch_flight_table(const double* old, double* neu, float2* neu32, int n_new, double c_dt,
                                 cudaStream_t st);
 
@@ -224,6 +225,7 @@ struct rt_grid {
   std::vector<SrcIn> src;              // sources as given by the caller
   SourceDev* src_dev = nullptr;
   size_t src_dev_cap = 0;
+  int variant = WALK_ANY;              // FP32 walker of the device source table
   bool src_dirty = true;
   int last_level0 = -1;
   int src_offset = 0;                  // index of the first source in checksums
@@ -519,12 +521,6 @@ int rt_set_source_rates(rt_grid* g, int n, const double* ndot) {
   return RT_OK;
 }
 
-// A source coordinate for which the FP32 walker may treat equal FP32 crossing
-// distances of a 45-degree ray as an exact tie: a multiple of 1/16 no larger
-// than 4096 cells, so every plane offset b - s is exact in FP32 and distinct
-// offsets stay at least 1/16 apart.
-static bool exact_in_f32(double v) { return v == ldexp(floor(ldexp(v, 4)), -4) && fabs(v) <= 4096.0; }
-
 // Source records of grid g for a given initial level (Step 1: Ndot spread
 // over 12 * 4^level0 root packages), attributed to instance slot `inst`.
 // unit[i] / p0[i], when given, override the photons/s carried by P = 1 and
@@ -547,23 +543,18 @@ static void build_sources(const rt_grid* g, int level0, int inst, std::vector<So
     S.rw = S.unit / vol;
     S.inst = inst;
     S.local = g->src_offset + (int)i;
-    int exact = 1;
-    float s32[3], slo[3], sab[3];
-    for (int a = 0; a < 3; ++a) {
-      s32[a] = (float)S.s[a];
-      slo[a] = (float)(S.s[a] - (double)s32[a]);
-      const bool pair_exact = (double)s32[a] + (double)slo[a] == S.s[a];
-      sab[a] = pair_exact ? 0.0f : (float)(ldexp(fabs(S.s[a]), -46));
-      exact &= exact_in_f32(S.s[a]) ? 1 : 0;
-    }
-    S.exact32 = exact && g->nx <= 4096 && g->ny <= 4096 && g->nz <= 4096;
+    fill_position32(S, g->nx, g->ny, g->nz, S.p0);
     // the FP32 walker deposits Gamma in eV/s (rt_get_rates converts to erg/s)
     S.k32 = make_float4((float)S.sdx, (float)S.w, (float)S.rw, (float)(H.e_ph - kEIon[H.type]));
-    S.s32 = make_float4(s32[0], s32[1], s32[2], S.exact32 ? 1.0f : 0.0f);
-    S.slo32 = make_float4(slo[0], slo[1], slo[2], (float)(S.sdx - (double)(float)S.sdx));
-    S.sabs32 = make_float4(sab[0], sab[1], sab[2], (float)S.p0);
     v.push_back(S);
   }
+}
+
+// Whether the FP32 walker can take the exact variant for a launch over v.
+static int walk_variant(const std::vector<SourceDev>& v) {
+  for (const SourceDev& S : v)
+    if (!S.exact32) return WALK_ANY;
+  return WALK_EXACT;
 }
 
 // Build the per-source device table of a single grid for a given initial
@@ -600,6 +591,7 @@ static int prepare_sources(rt_grid* g, int level0, bool fsl) {
   if (!v.empty())
     CUDA_TRY(cudaMemcpyAsync(g->src_dev, v.data(), v.size() * sizeof(SourceDev), cudaMemcpyHostToDevice, g->stream));
   CUDA_TRY(cudaStreamSynchronize(g->stream));  // v goes out of scope
+  g->variant = walk_variant(v);
   g->src_dirty = false;
   g->last_level0 = level0;
   g->src_fsl = fsl;
@@ -650,6 +642,7 @@ static void fill_common_args(TraceArgs& A, const rt_trace_params* p) {
   A.tau_term = -log(p->f_term);
   A.tau_term32 = (float)A.tau_term;
   A.tau_term32lo = (float)(A.tau_term - (double)A.tau_term32);
+  A.tau_near = A.tau_term32 * (1.0f - 1.0f / 4096.0f);
   A.timeout_ns = (long long)((p->timeout_s > 0 ? p->timeout_s : 2.0) * 1e9);
   A.segs_per_iter = p->segs_per_iter > 0 ? p->segs_per_iter : 8;
   A.checksums = (p->flags & RT_TRACE_CHECKSUMS) != 0;
@@ -668,7 +661,7 @@ static void fill_common_args(TraceArgs& A, const rt_trace_params* p) {
 // flight (fsl) are shared out over the passes on the device; `mode` and
 // `in_cap` say what the first pass takes over from the previous trace.
 static int launch_passes(TraceArgs A, size_t queue_bytes, const SourceDev* src, int nsrc, int passes, int precision,
-                         int fsl, int mode, unsigned long long in_cap, int blocks, cudaEvent_t ev0, cudaEvent_t ev1,
+                         int fsl, int variant, int mode, unsigned long long in_cap, int blocks, cudaEvent_t ev0, cudaEvent_t ev1,
                          cudaStream_t st, bool stall = false) {
   if ((unsigned long long)nsrc >= kMaxQueueSources)
     return fail(RT_ERR_INVALID_ARG, "trace: %d sources in one launch (at most %u)", nsrc, kMaxQueueSources - 1u);
@@ -688,7 +681,7 @@ static int launch_passes(TraceArgs A, size_t queue_bytes, const SourceDev* src, 
     A.nsrc = nsrc;
     A.src_first = s0;
     A.n_roots = n;
-    LAUNCH_TRY(launch_trace(precision, fsl, A, blocks, 256, st));
+    LAUNCH_TRY(launch_trace(precision, fsl, variant, A, blocks, 256, st));
   }
   CUDA_TRY(cudaEventRecord(ev1, st));
   return RT_OK;
@@ -842,12 +835,12 @@ static int enqueue_trace(rt_grid* g, const rt_trace_params* p, int passes, bool 
   }
   const int block = 256;  // the trace kernel is compiled for 256-thread blocks
   int per_sm = 0;
-  CUDA_TRY(trace_occupancy(g->precision, fsl ? 1 : 0, block, &per_sm));
+  CUDA_TRY(trace_occupancy(g->precision, fsl ? 1 : 0, g->variant, block, &per_sm));
   if (per_sm < 1) per_sm = 1;
   if (p->blocks_per_sm > 0 && p->blocks_per_sm < per_sm) per_sm = p->blocks_per_sm;
   if ((rc = g->ts.bind_rows(A, per_sm * g->ctx->num_sms, 1))) return rc;
-  if ((rc = launch_passes(A, g->ts.cap * g->ts.rec_bytes, g->src_dev, nsrc, passes, g->precision, fsl ? 1 : 0, mode,
-                          in_cap, per_sm * g->ctx->num_sms, g->ev0, g->ev1, st, (p->flags & RT_TRACE_SELFTEST_STALL) != 0)))
+  if ((rc = launch_passes(A, g->ts.cap * g->ts.rec_bytes, g->src_dev, nsrc, passes, g->precision, fsl ? 1 : 0,
+                          g->variant, mode, in_cap, per_sm * g->ctx->num_sms, g->ev0, g->ev1, st, (p->flags & RT_TRACE_SELFTEST_STALL) != 0)))
     return rc;
   commit_flight(g, fsl);
   g->traced = true;
@@ -1532,6 +1525,7 @@ struct rt_batch {
   size_t inst_cap = 0;
   SourceDev* src_dev = nullptr;
   size_t src_cap = 0;
+  int variant = WALK_ANY;       // FP32 walker of the source table
   int nsrc = 0;
   unsigned long long n_roots = 0;
   long long max_cells = 0;
@@ -1609,6 +1603,7 @@ static int batch_rebuild(rt_batch* b, int level0) {
     CUDA_TRY(cudaMemcpyAsync(b->src_dev, src.data(), src.size() * sizeof(SourceDev), cudaMemcpyHostToDevice, b->stream));
   CUDA_TRY(cudaStreamSynchronize(b->stream));
   b->nsrc = (int)src.size();
+  b->variant = walk_variant(src);
   b->n_roots = (12ULL << (2 * level0)) * (unsigned long long)src.size();
   b->max_diag = diag;
   b->dirty = false;
@@ -1649,11 +1644,12 @@ static int batch_enqueue(rt_batch* b, const rt_trace_params* p, int passes) {
     if ((rc = ensure_dir_table(b->ctx, want, &A.dir_tab, &A.dir_levels))) return rc;
   }
   int per_sm = 0;
-  CUDA_TRY(trace_occupancy(b->precision, 0, 256, &per_sm));
+  CUDA_TRY(trace_occupancy(b->precision, 0, b->variant, 256, &per_sm));
   if (per_sm < 1) per_sm = 1;
   if (p->blocks_per_sm > 0 && p->blocks_per_sm < per_sm) per_sm = p->blocks_per_sm;
   if ((rc = b->ts.bind_rows(A, per_sm * b->ctx->num_sms, ninst))) return rc;
-  if ((rc = launch_passes(A, b->ts.cap * b->ts.rec_bytes, b->src_dev, b->nsrc, passes, b->precision, 0, FLIGHT_OFF, 0,
+  if ((rc = launch_passes(A, b->ts.cap * b->ts.rec_bytes, b->src_dev, b->nsrc, passes, b->precision, 0,
+                          b->variant, FLIGHT_OFF, 0,
                           per_sm * b->ctx->num_sms,
                           b->ev0, b->ev1, st)))
     return rc;
@@ -1990,7 +1986,7 @@ int rt_batch_autotune(rt_batch* b, rt_trace_params* p) {
   if ((rc = rt_batch_trace(b, &q, 1))) return rc;  // sizes the queue, warms up
   const int spi[] = {4, 8, 16, 32, 64};
   int per_sm_max = 0;
-  CUDA_TRY(trace_occupancy(b->precision, 0, 256, &per_sm_max));
+  CUDA_TRY(trace_occupancy(b->precision, 0, b->variant, 256, &per_sm_max));
   float best = 1e30f;
   rt_trace_params bestp = q;
   for (int bps = 1; bps <= (per_sm_max > 0 ? per_sm_max : 1); ++bps) {

@@ -33,8 +33,9 @@ namespace rtg {
 cudaError_t launch_trace_init(unsigned long long* ctl, void* queue, size_t queue_bytes, unsigned long long n_roots,
                               int first_pass, int mode, unsigned long long in_cap, int pass, int passes,
                               cudaStream_t st);
-cudaError_t trace_occupancy(int precision, int fsl, int block, int* blocks_per_sm);
-cudaError_t launch_trace(int precision, int fsl, const TraceArgs& A, int grid, int block, cudaStream_t st);
+cudaError_t trace_occupancy(int precision, int fsl, int variant, int block, int* blocks_per_sm);
+cudaError_t launch_trace(int precision, int fsl, int variant, const TraceArgs& A, int grid, int block,
+                         cudaStream_t st);
 cudaError_t launch_direction_table(int level, float4* tab, cudaStream_t st);
 }  // namespace rtg
 
@@ -103,8 +104,6 @@ int na_setup(int dev, unsigned char** base, int* sms) {
   *sms = g_na_sms[dev];
   return RT_OK;
 }
-
-bool na_exact(double v) { return v == ldexp(floor(ldexp(v, 4)), -4) && fabs(v) <= 4096.0; }
 
 // The FP32 walker deposits Gamma in eV/s (an FP32 erg/s deposit of a faintly
 // lit cell would fall below the FP32 normal range); the caller's array is
@@ -196,19 +195,8 @@ int rt_trace_noalloc(const rt_noalloc_grid* g, int nsrc, const double* pos_cm, c
       S.rw = S.unit / vol;
       S.inst = 0;
       S.local = i;
-      int exact = 1;
-      float s32[3], slo[3], sab[3];
-      for (int a = 0; a < 3; ++a) {
-        s32[a] = (float)S.s[a];
-        slo[a] = (float)(S.s[a] - (double)s32[a]);
-        sab[a] = ((double)s32[a] + (double)slo[a] == S.s[a]) ? 0.0f : (float)ldexp(fabs(S.s[a]), -46);
-        exact &= na_exact(S.s[a]) ? 1 : 0;
-      }
-      S.exact32 = exact && g->nx <= 4096 && g->ny <= 4096 && g->nz <= 4096;
+      fill_position32(S, g->nx, g->ny, g->nz, 0.0);
       S.k32 = make_float4((float)S.sdx, (float)S.w, (float)S.rw, (float)(e_ph_eV[i] - kEHI));  // heat in eV
-      S.s32 = make_float4(s32[0], s32[1], s32[2], S.exact32 ? 1.0f : 0.0f);
-      S.slo32 = make_float4(slo[0], slo[1], slo[2], (float)(S.sdx - (double)(float)S.sdx));
-      S.sabs32 = make_float4(sab[0], sab[1], sab[2], 0.0f);
     }
     if ((e = cudaMemcpyAsync(src + i0, chunk, m * sizeof(SourceDev), cudaMemcpyHostToDevice, st)) != cudaSuccess ||
         (e = cudaStreamSynchronize(st)) != cudaSuccess)
@@ -240,6 +228,7 @@ int rt_trace_noalloc(const rt_noalloc_grid* g, int nsrc, const double* pos_cm, c
     A.tau_term = -log(p->f_term);
     A.tau_term32 = (float)A.tau_term;
     A.tau_term32lo = (float)(A.tau_term - (double)A.tau_term32);
+    A.tau_near = A.tau_term32 * (1.0f - 1.0f / 4096.0f);
     A.queue = base + kNaQueueOff;
     A.cap = p->queue_capacity > 0 ? (unsigned long long)p->queue_capacity : (unsigned long long)RT_NOALLOC_MAX_RECORDS;
     A.ctl = ctl;
@@ -253,13 +242,13 @@ int rt_trace_noalloc(const rt_noalloc_grid* g, int nsrc, const double* pos_cm, c
       A.theta32[l] = (float)A.theta[l];
     }
     int per_sm = 0;
-    if ((e = trace_occupancy(RT_FP32_MIXED, 0, 256, &per_sm)) != cudaSuccess) return na_fail(RT_ERR_CUDA, "occupancy", e);
+    if ((e = trace_occupancy(RT_FP32_MIXED, 0, WALK_ANY_PLAIN, 256, &per_sm)) != cudaSuccess) return na_fail(RT_ERR_CUDA, "occupancy", e);
     if (per_sm < 1) per_sm = 1;
     if (p->blocks_per_sm > 0 && p->blocks_per_sm < per_sm) per_sm = p->blocks_per_sm;
     if (per_sm * sms > kNaMaxBlocks) return na_fail(RT_ERR_INVALID_ARG, "more trace blocks than the budget rows hold");
     A.blk = (double*)(base + kNaBlkOff);
     A.blk_rows = 1;
-    if ((e = launch_trace(RT_FP32_MIXED, 0, A, per_sm * sms, 256, st)) != cudaSuccess)
+    if ((e = launch_trace(RT_FP32_MIXED, 0, WALK_ANY_PLAIN, A, per_sm * sms, 256, st)) != cudaSuccess)
       return na_fail(RT_ERR_CUDA, "trace launch", e);
     long long blocks = ((long long)ncell + 255) / 256;
     if (blocks > 8LL * sms) blocks = 8LL * sms;

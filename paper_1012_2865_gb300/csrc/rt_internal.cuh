@@ -2,6 +2,7 @@
 // library's kernels (trace.cu, chem.cu) and its host code (api.cu).
 #pragma once
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 #include "rt.h"
@@ -59,6 +60,8 @@ struct __align__(16) SourceDev {
   float4 s32;     // position as FP32 pair, high part; .w = 1 if exact32
   float4 slo32;   // low part (s - s32); .w = sdx - k32.x
   float4 sabs32;  // 2^-46 |s| where the pair does not hold s exactly, else 0; .w = p0
+  float4 sb32;    // s - sa as FP32 pairs (sb32, sblo32), sa the integer nearest s
+  float4 sblo32;
   // FP64 view
   double s[3];    // position in cell units (pos_cm / dx)
   double sdx;     // sigma * dx: optical depth per unit n_HI per cell length
@@ -73,7 +76,41 @@ struct __align__(16) SourceDev {
   int local;      // index of the source within its grid (checksum)
   int exact32;    // position on a 1/16-cell lattice within 4096 cells (see api.cu)
   int type;       // photon type of its packages (0 H I, 1 He I, 2 He II)
+  int sa[3];
 };
+
+// A source coordinate for which the FP32 walker's plane distances b - s are
+// exact in FP32 (and equal distances of a 45-degree ray are an exact tie): a
+// multiple of 1/16 no larger than 4096 cells, so that distinct distances stay
+// at least 1/16 apart.
+inline bool exact_in_f32(double v) { return v == ldexp(floor(ldexp(v, 4)), -4) && fabs(v) <= 4096.0; }
+
+// The FP32 view of a source's position from S.s (and S.exact32).
+inline void fill_position32(SourceDev& S, int nx, int ny, int nz, double p0) {
+  int exact = 1;
+  float hi[3], lo[3], ab[3], bh[3], bl[3];
+  for (int a = 0; a < 3; ++a) {
+    hi[a] = (float)S.s[a];
+    lo[a] = (float)(S.s[a] - (double)hi[a]);
+    const bool held = (double)hi[a] + (double)lo[a] == S.s[a];
+    ab[a] = held ? 0.0f : (float)(ldexp(fabs(S.s[a]), -46));
+    const double sa = rint(S.s[a]), sb = S.s[a] - sa;  // exact difference
+    S.sa[a] = (int)sa;
+    bh[a] = (float)sb;
+    bl[a] = (float)(sb - (double)bh[a]);
+    exact &= exact_in_f32(S.s[a]) ? 1 : 0;
+  }
+  S.exact32 = exact && nx <= 4096 && ny <= 4096 && nz <= 4096;
+  S.s32 = make_float4(hi[0], hi[1], hi[2], S.exact32 ? 1.0f : 0.0f);
+  S.slo32 = make_float4(lo[0], lo[1], lo[2], (float)(S.sdx - (double)(float)S.sdx));
+  S.sabs32 = make_float4(ab[0], ab[1], ab[2], (float)p0);
+  S.sb32 = make_float4(bh[0], bh[1], bh[2], 0.0f);
+  S.sblo32 = make_float4(bl[0], bl[1], bl[2], 0.0f);
+}
+
+// Instantiations of the FP32 walker: every source of the launch exact32, any
+// source, and any source with n_HI as plain FP32 instead of pairs.
+enum WalkVariant { WALK_EXACT = 0, WALK_ANY = 1, WALK_ANY_PLAIN = 2 };
 
 // InstDev.flags: the FP32-mixed grid stores n_HI as float2 pairs (n_HI
 // rounded to FP32, and the remainder), so the walker sums optical depth to
@@ -180,6 +217,7 @@ struct TraceArgs {
   int dir_levels;             // -1: no table
   double tau_term;
   float tau_term32, tau_term32lo;  // tau_term as an FP32 pair
+  float tau_near;                  // above it the FP32 walker tests the termination in full
   void* queue;
   unsigned long long cap;
   unsigned long long* ctl;

@@ -52,6 +52,7 @@ static_assert(kBlkGrids <= kShInst, "a grid with a budget row has its counters i
 constexpr int kBlock = 256;  // threads per block of the trace kernel
 
 enum Event { EV_NONE = 0, EV_SPLIT = 1, EV_DONE = 2, EV_HALT = 3 };
+enum Start { NO_START = 0, START_CHILD, START_ROOT, START_RESUMED };
 constexpr int kAcc = 5;  // budget sums per grid: emitted, absorbed, escaped, resumed, halted
 
 // Photon budget of one lane for the grid it is working on; lives in shared
@@ -80,9 +81,11 @@ struct LaneAcc {
   unsigned long long segments;
   unsigned int fallbacks, fallbacks_tau;
   int inst;
+  // of the lane's package (FP32 walker): P, optical depth and its error bound
+  // at the start; read only when the package ends, so kept out of registers
+  float Pstart, tau0, tau_err;
   // 72 bytes = 18 banks: the 8-byte accesses of a half-warp to one field
   // fall on 16 different bank pairs (a 64-byte stride puts them on two)
-  unsigned int pad[3];
 };
 static_assert(sizeof(LaneAcc) == 72, "conflict-free stride of the per-lane sums");
 
@@ -230,28 +233,26 @@ struct Walk64 {
     Pstart = P;
     steps = 0;
   }
-  // Steps 3a-3b: direction and cell at radius r.  Returns false if the
-  // package starts outside the box.
-  __device__ __forceinline__ bool start(const TraceArgs& A) {
+  // Steps 3a-3b: direction and cell at radius r, false outside the box.  A
+  // package continued from the previous trace (given) is in the cell it
+  // halted in.
+  template <bool FSL>
+  __device__ __forceinline__ bool start(const TraceArgs& A, LaneAcc&, bool given, uint32_t cell) {
     bind(A);
-    c0 = cell_of64(__dadd_rn(s0, __dmul_rn(r, n0)), n0);
-    c1 = cell_of64(__dadd_rn(s1, __dmul_rn(r, n1)), n1);
-    c2 = cell_of64(__dadd_rn(s2, __dmul_rn(r, n2)), n2);
-    if (!inside()) return false;
+    if (FSL && given) {
+      c0 = (int)(cell % (uint32_t)nx);
+      c1 = (int)((cell / (uint32_t)nx) % (uint32_t)ny);
+      c2 = (int)(cell / ((uint32_t)nx * (uint32_t)ny));
+    } else {
+      c0 = cell_of64(__dadd_rn(s0, __dmul_rn(r, n0)), n0);
+      c1 = cell_of64(__dadd_rn(s1, __dmul_rn(r, n1)), n1);
+      c2 = cell_of64(__dadd_rn(s2, __dmul_rn(r, n2)), n2);
+      if (!inside()) return false;
+    }
     t0 = next_t64(c0, s0, n0);
     t1 = next_t64(c1, s1, n1);
     t2 = next_t64(c2, s2, n2);
     return true;
-  }
-  // A package continued from the previous trace: the cell it halted in.
-  __device__ __forceinline__ void resume(const TraceArgs& A, uint32_t cell) {
-    bind(A);
-    c0 = (int)(cell % (uint32_t)nx);
-    c1 = (int)((cell / (uint32_t)nx) % (uint32_t)ny);
-    c2 = (int)(cell / ((uint32_t)nx * (uint32_t)ny));
-    t0 = next_t64(c0, s0, n0);
-    t1 = next_t64(c1, s1, n1);
-    t2 = next_t64(c2, s2, n2);
   }
   __device__ __forceinline__ void set_rlim(const TraceArgs& A) {
     if ((int)age < A.n_ages) rlim = A.rlim64[age];
@@ -384,6 +385,9 @@ struct Walk64 {
     }
     return EV_NONE;
   }
+  __device__ __forceinline__ void seal(const TraceArgs&, const LaneAcc&) {}
+  __device__ __forceinline__ void begin_visit() {}
+  __device__ __forceinline__ int end_visit(const TraceArgs&, LaneAcc&, int, int ev) { return ev; }
   // Budget of the parent's run when it splits (children carry P/4 each).
   __device__ __forceinline__ void on_split(const TraceArgs& A, LaneAcc& acc) const {
     acc.absorbed += (Pstart - P) * unit(A);
@@ -441,25 +445,37 @@ __device__ __noinline__ double retrace_tau64(const TraceArgs& A, uint32_t src, i
 // ---------------------------------------------------------------------------
 // FP32-mixed walker.
 //
-// All per-segment arithmetic is FP32.  Crossing distances t_i, the radius r
-// and segment lengths are carried as unevaluated FP32 pairs (hi + lo,
-// "double-float"), built from the pixel direction stored as an FP32 pair
-// (FP64 direction rounded twice) and from the source position as an FP32
+// All per-segment arithmetic is FP32.  Crossing distances t_i, the radius r,
+// segment lengths and the optical depth are carried as unevaluated FP32 pairs
+// (hi + lo, "double-float"), built from the pixel direction stored as an FP32
+// pair (FP64 direction rounded twice) and from the source position as an FP32
 // pair, so each t carries ~44 correct bits while every instruction is FP32.
-// Optical depth, attenuation and the k_ph / Gamma deposits are plain FP32.
+// Attenuation and the k_ph / Gamma deposits are plain FP32.
+//
+// The walker is bound by its dependent instructions and the warps' issue
+// slots (four warps per scheduler at 128 registers), so a segment's common
+// case is kept short: planes are counted along each axis instead of located
+// from cell indices (Axis), one comparison with a radius set at the package's
+// start covers split, box exit and halt, one more the termination, and the
+// decisions in full (decide, terminates) run only for a segment that fails
+// either comparison or whose two nearest planes lie within 2^-20 of each
+// other.  Source constants sit in registers; what only a package's end needs
+// sits in shared memory.  With the decisions in full at every segment the
+// trace of the 128^3 Stroemgren snapshot took 0.41 ms, now 0.30 ms; 24 sources in an
+// ionised 128^3 grid 13.2 -> 9.6 ms; 1000 in a clumpy 256^3 grid 3.9 -> 3.3 ms.
 //
 // Each decision that shapes the ray tree -- which cell plane is crossed next,
 // whether the package splits, whether it terminates -- is taken from the
 // FP32 values only when an error bound proves it equals the FP64 decision:
 //   |t_pair - t_FP64| <= 2^-40 t + 2^-46 |s| / |n|   (per axis),
-//   |tau_FP32 - tau_FP64| <= tau_err (accumulated per segment).
+//   |tau_pair - tau_FP64| <= tau_bound (per package).
 // Inside a band the decision is re-taken in FP64: the crossing distances of
 // the current cell from the FP64 direction, or the FP64 optical depth of the
 // package's lineage.  Per-level counts therefore equal the FP64 path's.
 // ---------------------------------------------------------------------------
 constexpr float kEps32 = 5.9604645e-8f;   // 2^-24
 constexpr float kBandT = 9.094947e-13f;   // 2^-40
-constexpr float kClose = 4.76837158e-7f;  // 2^-21: high parts farther apart are ordered
+constexpr float kNear = 9.53674316e-7f;   // 2^-20: high parts farther apart are ordered
 
 // Direction of (level, pix) as FP32 pairs: from the device table when the
 // level is tabulated, else from the FP64 evaluation.  Returns the
@@ -507,31 +523,102 @@ __device__ __noinline__ int decide64(const TraceArgs& A, uint32_t src, int level
   return out;
 }
 
+// One axis of a ray.  Planes crossed by the axis are met at the distances
+//   t = |plane - s| / |n|,  |plane - s| = d for a source on the 1/16-cell
+// lattice (EXACT: d is an exact FP32 number and grows by exactly 1 per
+// plane), else k + off |n| with k an integer and off the source's offset from
+// the nearest integer, times 1 / |n|.  So the next plane of an axis costs
+// four (EXACT) or ten FP32 instructions and no table or source record.  t is
+// a pair whose low part may reach 2^-22 of the high part (it is not
+// renormalised; every use allows for that).
+constexpr float kFar = 1e30f;  // crossing distance of an axis that the ray never crosses
+template <bool EXACT>
+struct Axis {
+  F2 iv;       // 1 / |n| (0 for a vanishing component)
+  F2 t;        // distance to the next plane
+  F2 off;      // general: offset term of t
+  float d;     // EXACT
+  int k;       // general
+  int stride;  // change of the cell index at a plane (its sign is the direction's)
+  __device__ __forceinline__ void plane() {
+    const float f = EXACT ? d : (float)k;
+    const float p = __fmul_rn(f, iv.hi);
+    float e = fmaf(f, iv.hi, -p);
+    e = fmaf(f, iv.lo, e);
+    if (EXACT) {
+      t = F2{p, e};
+    } else {
+      // k = 0, or |k| >= 1 and |off| <= iv / 2: the first sum's error is exact
+      const float h = __fadd_rn(p, off.hi);
+      const float z = __fadd_rn(__fsub_rn(p, h), off.hi);
+      t = F2{h, __fadd_rn(__fadd_rn(e, z), off.lo)};
+    }
+  }
+  __device__ __forceinline__ void next() {
+    if (EXACT) d += 1.0f;
+    else ++k;
+    plane();
+  }
+  // Cell c of an axis with direction n, source coordinate s (EXACT) or
+  // sa + sb (general), dim cells and index stride `step`.
+  __device__ __forceinline__ void init(int c, F2 n, float s, int sa, F2 sb, int step) {
+    const bool neg = n.hi < 0.0f;
+    iv = n.hi != 0.0f ? f2_recip(n) : F2{0.0f, 0.0f};
+    if (neg) iv = F2{-iv.hi, -iv.lo};
+    stride = n.hi > 0.0f ? step : (neg ? -step : 0);
+    off = F2{0.0f, 0.0f};
+    if (EXACT) {
+      d = neg ? s - (float)c : (float)(c + 1) - s;
+    } else {
+      k = neg ? sa - c : c + 1 - sa;
+      if (!neg) sb = F2{-sb.hi, -sb.lo};
+      off = n.hi != 0.0f ? f2_mul(sb, iv) : sb;
+    }
+    if (n.hi != 0.0f) plane();
+    else t = F2{kFar, 0.0f};
+  }
+  // the cell that init was given, advanced by the planes crossed since
+  __device__ __forceinline__ int cell(float s, int sa) const {
+    if (EXACT) return stride < 0 ? (int)(s - d) : (int)(s + d) - 1;
+    return stride < 0 ? sa - k : sa + k - 1;
+  }
+  // distance along the axis of the point at radius rm from the middle of the cell
+  __device__ __forceinline__ float off_middle(float rm, float s, int sa) const {
+    float n = iv.hi != 0.0f ? __frcp_rn(iv.hi) : 0.0f;
+    if (stride < 0) n = -n;
+    return fabsf(fmaf(n, rm, s) - ((float)cell(s, sa) + 0.5f));
+  }
+};
+
+// EXACT: every source of the launch lies on the 1/16-cell lattice.  PAIR:
+// n_HI is stored as FP32 pairs.
+template <bool EXACT, bool PAIR>
 struct Walk32 {
   using Rec = Rec32;  // packages in flight between traces; records of FSL traces
   template <bool FSL> using Q = typename std::conditional<FSL, Rec32, QRec32>::type;  // queue record
   uint32_t src, pix;
   uint32_t age;         // traces since emission (finite speed of light)
   F2 rlim;              // halting radius of this age
-  uint32_t level;       // bits 0-3 level, bit 8: 45-degree ray of an exact source,
-                        // bit 9: n_HI stored as FP32 pairs
+  uint32_t level;       // bits 0-3 level, bit 8: 45-degree ray of an exact source
   F2 r;
-  float P, tau, tau_lo, Pstart, tau_err;
-  F2 iv0, iv1, iv2;     // 1 / n_i (0 for a vanishing component)
-  F2 t0, t1, t2;        // distance to the next plane on each axis
-  int c0, c1, c2;
-  int nx, ny, nz, steps;
+  float P, tau, tau_lo;
+  float tau_err;        // error bound of tau (in records and while a package starts or ends)
+  Axis<EXACT> a0, a1, a2;
+  int idx;              // cell index
+  int steps;            // segments of the package in earlier queue visits
   unsigned nseg;
   float nh, nh_lo;      // n_HI of the current cell (pair), loaded one step ahead
+  float lim;            // below it no crossing splits, leaves the box or halts
+  float sk, q;          // sum of kappa over the package's segments; error of tau per unit of it
+  float sdx, sdx_lo, w, heat;
   const float* nhi;
   float* K;
   float* G;
 
   __device__ __forceinline__ int lvl() const { return (int)(level & 15u); }
-  __device__ __forceinline__ int cell_index() const { return c0 + nx * (c1 + ny * c2); }
   __device__ __forceinline__ bool diag_exact() const { return (level & 256u) != 0; }
-  __device__ __forceinline__ void load_nh(int idx) {
-    if (level & 512u) {
+  __device__ __forceinline__ void load_nh() {
+    if (PAIR) {
       const float2 v = __ldg(reinterpret_cast<const float2*>(nhi) + idx);
       nh = v.x;
       nh_lo = v.y;
@@ -547,46 +634,35 @@ struct Walk32 {
   }
   __device__ __forceinline__ int inst(const TraceArgs& A) const { return A.src[src].inst; }
   __device__ __forceinline__ double unit(const TraceArgs& A) const { return A.src[src].unit; }
-  __device__ __forceinline__ bool inside() const {
-    return c0 >= 0 && c0 < nx && c1 >= 0 && c1 < ny && c2 >= 0 && c2 < nz;
-  }
-  // distance from the source to the next plane of cell c along an axis
-  __device__ __forceinline__ static F2 next_t(int c, float s_hi, float s_lo, F2 iv) {
-    if (iv.hi == 0.0f) return {__int_as_float(0x7f800000), 0.0f};
-    const float b = (float)(iv.hi > 0.0f ? c + 1 : c);
-    const F2 d0 = two_sum(b, -s_hi);
-    const F2 d = fast_two_sum(d0.hi, __fsub_rn(d0.lo, s_lo));
-    return f2_mul(d, iv);
-  }
   // cell of coordinate u along an axis (tie rule: n > 0 floor, n < 0 ceil - 1)
   __device__ __forceinline__ static int cell_of(F2 u, float n) {
     const int f = f2_floor(u);
     if (n < 0.0f && (float)f == u.hi && u.lo == 0.0f) return f - 1;
     return f;
   }
-  __device__ __forceinline__ float band(const TraceArgs& A, F2 t, int axis) const {
-    const float4 sa = __ldg(&A.src[src].sabs32);
-    const float ab = axis == 0 ? sa.x * fabsf(iv0.hi) : (axis == 1 ? sa.y * fabsf(iv1.hi) : sa.z * fabsf(iv2.hi));
-    return fmaf(t.hi, kBandT, ab);
-  }
 
-  // Geometry of a package at radius r: direction pairs, first cell (the
-  // cell index `cell` when given, else the cell holding the point at r),
-  // next crossings.  False when that cell is outside the box.
-  template <bool GIVEN = false>
-  __device__ __forceinline__ bool start_geom(const TraceArgs& A, uint32_t cell = 0) {
+  // A package at radius r: the absorber and accumulators of its photon type
+  // (Sec. 3.2), its direction, first cell (the cell index `cell` when given:
+  // a package continued from the previous trace; else the cell holding the
+  // point at r), next crossings and limits.  False when that cell is outside
+  // the box.
+  template <bool FSL>
+  __device__ __forceinline__ bool start(const TraceArgs& A, LaneAcc& acc, bool given, uint32_t cell) {
     const SourceDev& S = A.src[src];
+    const InstDev& I = A.inst[S.inst];
     const float4 sh = __ldg(&S.s32);
     const float4 sl = __ldg(&S.slo32);
-    const InstDev& I = A.inst[S.inst];
-    nx = I.nx; ny = I.ny; nz = I.nz;
+    acc.Pstart = P;
+    acc.tau0 = tau;
+    acc.tau_err = tau_err;
+    steps = 0;
+    sk = 0.0f;
     F2 n[3];
     const int diag = dir_pair(A, lvl(), pix, n);
-    level = (level & (15u | 512u)) | ((diag && sh.w != 0.0f) ? 256u : 0u);
-    iv0 = n[0].hi != 0.0f ? f2_recip(n[0]) : F2{0.0f, 0.0f};
-    iv1 = n[1].hi != 0.0f ? f2_recip(n[1]) : F2{0.0f, 0.0f};
-    iv2 = n[2].hi != 0.0f ? f2_recip(n[2]) : F2{0.0f, 0.0f};
-    if (GIVEN) {
+    level = (level & 15u) | ((diag && sh.w != 0.0f) ? 256u : 0u);
+    const int nx = I.nx, ny = I.ny, nz = I.nz;
+    int c0, c1, c2;
+    if (FSL && given) {
       c0 = (int)(cell % (uint32_t)nx);
       c1 = (int)((cell / (uint32_t)nx) % (uint32_t)ny);
       c2 = (int)(cell / ((uint32_t)nx * (uint32_t)ny));
@@ -594,36 +670,52 @@ struct Walk32 {
       c0 = cell_of(f2_add(F2{sh.x, sl.x}, f2_mul(r, n[0])), n[0].hi);
       c1 = cell_of(f2_add(F2{sh.y, sl.y}, f2_mul(r, n[1])), n[1].hi);
       c2 = cell_of(f2_add(F2{sh.z, sl.z}, f2_mul(r, n[2])), n[2].hi);
-      if (!inside()) return false;
+      if (c0 < 0 || c0 >= nx || c1 < 0 || c1 >= ny || c2 < 0 || c2 >= nz) return false;
     }
-    t0 = next_t(c0, sh.x, sl.x, iv0);
-    t1 = next_t(c1, sh.y, sl.y, iv1);
-    t2 = next_t(c2, sh.z, sl.z, iv2);
-    return true;
-  }
-  __device__ __forceinline__ void bind(const TraceArgs& A) {
-    const SourceDev& S = A.src[src];
-    const InstDev& I = A.inst[S.inst];
-    // the absorber and accumulators of the package's photon type (Sec. 3.2)
+    idx = c0 + nx * (c1 + ny * c2);
     const int t = S.type;
     nhi = (const float*)(t == 0 ? I.nhi : I.nhe[t - 1]);
+    load_nh();
+    if (EXACT) {
+      a0.init(c0, n[0], sh.x, 0, F2{0.0f, 0.0f}, 1);
+      a1.init(c1, n[1], sh.y, 0, F2{0.0f, 0.0f}, nx);
+      a2.init(c2, n[2], sh.z, 0, F2{0.0f, 0.0f}, nx * ny);
+    } else {
+      const float4 bh = __ldg(&S.sb32), bl = __ldg(&S.sblo32);
+      a0.init(c0, n[0], sh.x, S.sa[0], F2{bh.x, bl.x}, 1);
+      a1.init(c1, n[1], sh.y, S.sa[1], F2{bh.y, bl.y}, nx);
+      a2.init(c2, n[2], sh.z, S.sa[2], F2{bh.z, bl.z}, nx * ny);
+    }
     K = (float*)(t == 0 ? I.K : I.Khe[t - 1]);
     G = (float*)(t == 0 ? I.G : I.Ghe[t - 1]);
-    level = (level & ~512u) | ((I.flags & kInstNhiPair) ? 512u : 0u);
-    Pstart = P;
-    steps = 0;
-  }
-  __device__ __forceinline__ bool start(const TraceArgs& A) {
-    bind(A);
-    if (!start_geom(A)) return false;
-    load_nh(cell_index());
+    const float4 k32 = __ldg(&S.k32);  // sdx, w, rw, heat
+    sdx = k32.x; sdx_lo = sl.w; w = k32.y; heat = k32.w;
+    // Radii before and after which the next crossing cannot / must need the
+    // full decision: the exit plane of each axis (its distance from the
+    // source in FP32, widened by the rounding of s and of the product), the
+    // split radius and the halting radius.
+    float lo = kFar, hi = kFar;
+    exit_of(a0, n[0].hi < 0.0f ? sh.x : (float)nx - sh.x, (float)nx, lo, hi);
+    exit_of(a1, n[1].hi < 0.0f ? sh.y : (float)ny - sh.y, (float)ny, lo, hi);
+    exit_of(a2, n[2].hi < 0.0f ? sh.z : (float)nz - sh.z, (float)nz, lo, hi);
+    const int l = lvl();
+    if (l < A.max_level) {
+      lo = fminf(lo, A.rsplit32[l]);
+      hi = fminf(hi, A.rsplit32[l]);
+    }
+    if (FSL) lo = fminf(lo, rlim.hi);
+    lim = fmaf(lo, -kNear, lo);
+    const float4 sa = __ldg(&S.sabs32);
+    q = fmaf(hi, 4.1f * kBandT, 1e-30f) +
+        4.1f * fmaxf(sa.x * a0.iv.hi, fmaxf(sa.y * a1.iv.hi, sa.z * a2.iv.hi));
     return true;
   }
-  // A package continued from the previous trace: the cell it halted in.
-  __device__ __forceinline__ void resume(const TraceArgs& A, uint32_t cell) {
-    bind(A);
-    start_geom<true>(A, cell);
-    load_nh(cell_index());
+  __device__ __forceinline__ static void exit_of(const Axis<EXACT>& a, float d, float dim, float& lo, float& hi) {
+    const float m = dim * (8.0f * kEps32);
+    if (a.iv.hi > 0.0f) {
+      lo = fminf(lo, (d - m) * a.iv.hi);
+      hi = fminf(hi, (d + m) * a.iv.hi);
+    }
   }
   __device__ __forceinline__ void set_rlim(const TraceArgs& A) {
     if ((int)age < A.n_ages) {
@@ -635,10 +727,34 @@ struct Walk32 {
     }
   }
 
-  __device__ __forceinline__ void load(const Rec& q) {
-    r = {q.r, q.r_lo}; P = q.P; tau = q.tau; tau_lo = q.tau_lo; tau_err = q.tau_err; src = q.src; pix = q.pix;
-    level = q.tag & 15u;
-    age = q.age;
+  __device__ __forceinline__ void load(const Rec& q_) {
+    r = {q_.r, q_.r_lo}; P = q_.P; tau = q_.tau; tau_lo = q_.tau_lo; tau_err = q_.tau_err; src = q_.src; pix = q_.pix;
+    level = q_.tag & 15u;
+    age = q_.age;
+  }
+  // Bound on |tau (pair) - tau (FP64 evaluation)| at radius rmax.  Each
+  // crossing's pair lies within 2^-40 t + 2^-46 |s| / |n| of the FP64 one and
+  // shifts the boundary between two cells, so tau by at most that times the
+  // two kappas (twice that, with margin); the pair products add 2^-37 dtau
+  // (2^-22 dtau where n_HI is plain FP32), and the pair sum 2^-44 tau a
+  // segment plus the rounding of its low part, which is renormalised once per
+  // queue visit and so stays below segs_per_iter 2^-24 tau.
+  __device__ __forceinline__ float tau_bound(const TraceArgs& A, const LaneAcc& acc, float rmax) const {
+    const float4 sa = __ldg(&A.src[src].sabs32);
+    const float ab = fmaxf(sa.x * a0.iv.hi, fmaxf(sa.y * a1.iv.hi, sa.z * a2.iv.hi));
+    const float e_dtau = PAIR ? 8.0f * kBandT : 4.0f * kEps32;
+    const float spi = (float)A.segs_per_iter;
+    return acc.tau_err + fmaf(tau, kEps32, tau - acc.tau0) * e_dtau + sk * (fmaf(rmax, 4.0f * kBandT, 1e-30f) + 4.0f * ab) +
+           ((float)steps + spi) * tau * (kBandT / 16.0f + spi * (kEps32 * kEps32));
+  }
+  // The package's radius and optical depth as normalised pairs with the error
+  // bound, for its children or the store of packages in flight.
+  __device__ __forceinline__ void seal(const TraceArgs& A, const LaneAcc& acc) {
+    r = fast_two_sum(r.hi, r.lo);
+    const F2 t2 = fast_two_sum(tau, tau_lo);
+    tau = t2.hi;
+    tau_lo = t2.lo;
+    tau_err = tau_bound(A, acc, r.hi);
   }
   // Record of child cpix (level + 1, P/4, same radius, age, optical depth and
   // its error bound); the level sits in the tag's low bits until publication.
@@ -648,13 +764,13 @@ struct Walk32 {
     c.src = src; c.pix = cpix; c.tag = (uint32_t)(lvl() + 1); c.age = age;
     return c;
   }
-  __device__ __forceinline__ static uint32_t cell_of_record(const Rec& q) { return q.cell; }
+  __device__ __forceinline__ static uint32_t cell_of_record(const Rec& q_) { return q_.cell; }
   // A halted package as the next trace continues it (one trace older).
-  __device__ __forceinline__ void store_halted(Rec* q) const {
-    reinterpret_cast<float4*>(&q->r)[0] = make_float4(r.hi, r.lo, P, tau);
-    reinterpret_cast<uint4*>(&q->tau_lo)[0] =
+  __device__ __forceinline__ void store_halted(Rec* q_) const {
+    reinterpret_cast<float4*>(&q_->r)[0] = make_float4(r.hi, r.lo, P, tau);
+    reinterpret_cast<uint4*>(&q_->tau_lo)[0] =
         make_uint4(__float_as_uint(tau_lo), __float_as_uint(tau_err), src, pix);
-    reinterpret_cast<uint4*>(&q->tag)[0] = make_uint4((uint32_t)lvl(), age + 1, (uint32_t)cell_index(), 0u);
+    reinterpret_cast<uint4*>(&q_->tag)[0] = make_uint4((uint32_t)lvl(), age + 1, (uint32_t)idx, 0u);
   }
   // Publish a record in the global queue: payload first, then the tag with
   // release semantics.  FSL records (48 B) carry the age and the tag
@@ -724,114 +840,130 @@ struct Walk32 {
     level = (uint32_t)(lvl() + 1); pix = 4u * pix; P = P * 0.25f;
   }
 
-  // The next crossing as the FP64 evaluation takes it: bits 0-2 the planes
-  // crossed, bit 3 a split first, bits 4-5 the axis of the smallest pair,
-  // bit 6 (FSL) the crossing lies beyond the halting radius; rn_out receives
-  // the crossing distance.  Orders the pairs cannot prove are re-taken in
-  // FP64 (decide64) and counted in fb.
+  // The next crossing as the FP64 evaluation takes it, where the fast test of
+  // step() cannot tell: bits 0-2 the planes crossed, bit 3 a split first, bit
+  // 6 (FSL) the crossing lies beyond the halting radius, bit 7 the crossing
+  // leaves the box; rn receives the crossing distance.  Orders that the pairs
+  // cannot prove are re-taken in FP64 (decide64) and counted in fb.
   template <bool FSL>
-  __device__ __forceinline__ int decide(const TraceArgs& A, F2& rn_out, unsigned& fb) const {
-    // next crossing: the smallest pair, and whether the order is provable
+  __device__ __forceinline__ int decide(const TraceArgs& A, F2& rn, unsigned& fb) const {
+    const SourceDev& S = A.src[src];
     int imin = 0;
-    F2 rn = t0;
-    if (f2_less(t1, rn)) { rn = t1; imin = 1; }
-    if (f2_less(t2, rn)) { rn = t2; imin = 2; }
+    rn = a0.t;
+    if (f2_diff(a1.t, rn) < 0.0f) { rn = a1.t; imin = 1; }
+    if (f2_diff(a2.t, rn) < 0.0f) { rn = a2.t; imin = 2; }
+    const float4 sab = __ldg(&S.sabs32);
+    const float b0 = fmaf(a0.t.hi, kBandT, sab.x * a0.iv.hi), b1 = fmaf(a1.t.hi, kBandT, sab.y * a1.iv.hi),
+                b2 = fmaf(a2.t.hi, kBandT, sab.z * a2.iv.hi);
+    const float emin = imin == 0 ? b0 : (imin == 1 ? b1 : b2);
     bool m0 = imin == 0, m1 = imin == 1, m2 = imin == 2;
     bool unsure = false;
-    const float close = fmaf(rn.hi, kClose, rn.hi) + 1e-30f;
-    const bool c_0 = imin != 0 && iv0.hi != 0.0f && t0.hi <= close;
-    const bool c_1 = imin != 1 && iv1.hi != 0.0f && t1.hi <= close;
-    const bool c_2 = imin != 2 && iv2.hi != 0.0f && t2.hi <= close;
+    const bool xy_tie = diag_exact() && f2_eq(a0.t, a1.t);
+    if (!m0 && f2_diff(a0.t, rn) <= b0 + emin) { if (imin == 1 && xy_tie) m0 = true; else unsure = true; }
+    if (!m1 && f2_diff(a1.t, rn) <= b1 + emin) { if (imin == 0 && xy_tie) m1 = true; else unsure = true; }
+    if (!m2 && f2_diff(a2.t, rn) <= b2 + emin) unsure = true;
     const int l = lvl();
-    const float R = A.rsplit32[l];
-    const bool can_split = l < A.max_level;
-    const bool split_close = can_split && !(rn.hi > fmaf(R, kClose, R)) && !(rn.hi < fmaf(R, -kClose, R));
-    bool split = can_split && rn.hi > R;
-    // Step 3j: the crossing against the halting radius, decided like the split
-    bool halt = FSL && rn.hi > rlim.hi;
-    const bool halt_close = FSL && !(rn.hi > fmaf(rlim.hi, kClose, rlim.hi)) &&
-                            !(rn.hi < fmaf(rlim.hi, -kClose, rlim.hi));
-    if (c_0 || c_1 || c_2 || split_close || halt_close) {
-      // a close pair: compare exactly, re-take the decision in FP64 if unprovable
-      const float emin = band(A, rn, imin);
-      const bool xy_tie = diag_exact() && f2_eq(t0, t1);
-      if (c_0 && f2_diff(t0, rn) <= band(A, t0, 0) + emin) { if (imin == 1 && xy_tie) m0 = true; else unsure = true; }
-      if (c_1 && f2_diff(t1, rn) <= band(A, t1, 1) + emin) { if (imin == 0 && xy_tie) m1 = true; else unsure = true; }
-      if (c_2 && f2_diff(t2, rn) <= band(A, t2, 2) + emin) unsure = true;
-      if (split_close) {
-        const float d = f2_diff(rn, F2{R, A.rsplit32lo[l]});
-        const float bnd = emin + R * kBandT;
-        if (d > bnd) split = true;
-        else if (-d > bnd) split = false;
-        else unsure = true;
-      }
-      if (halt_close) {
-        const float d = f2_diff(rn, rlim);
-        const float bnd = emin + rlim.hi * kBandT;
-        if (d > bnd) halt = true;
-        else if (-d > bnd) halt = false;
-        else unsure = true;
-      }
-      if (unsure) {
-        const double rlim64 = !FSL ? __longlong_as_double(0x7ff0000000000000LL)
-                                   : ((int)age < A.n_ages ? A.rlim64[age] : 0.0);
-        const int d64 = decide64(A, src, l, pix, c0, c1, c2, rlim64);
-        split = (d64 & 8) != 0;
-        halt = (d64 & 64) != 0;
-        m0 = (d64 & 1) != 0;
-        m1 = (d64 & 2) != 0;
-        m2 = (d64 & 4) != 0;
-        ++fb;
-      }
+    bool split = false, halt = false;
+    if (l < A.max_level) {
+      const float R = A.rsplit32[l];
+      const float d = f2_diff(rn, F2{R, A.rsplit32lo[l]});
+      split = d > 0.0f;
+      if (fabsf(d) <= emin + R * kBandT) unsure = true;
     }
-    rn_out = rn;
-    return (m0 ? 1 : 0) | (m1 ? 2 : 0) | (m2 ? 4 : 0) | (split ? 8 : 0) | (imin << 4) | (halt ? 64 : 0);
-  }
-  // Cross the planes of `m` (bits 0-2) at distance rn.
-  // The first crossed axis is selected rather than branched on, so the lanes
-  // of a warp (crossing different axes) evaluate one next_t together; a
-  // second or third axis crossed at the same point (edges, corners) is rare.
-  __device__ __forceinline__ void advance(const TraceArgs& A, int m, F2 rn) {
-    const int mm = m & 7;
-    if (mm) {
-      const float4 sh = __ldg(&A.src[src].s32);
-      const float4 sl = __ldg(&A.src[src].slo32);
-      const int a = (mm & 1) ? 0 : ((mm & 2) ? 1 : 2);
-      const F2 iv = a == 0 ? iv0 : (a == 1 ? iv1 : iv2);
-      const int c = (a == 0 ? c0 : (a == 1 ? c1 : c2)) + (iv.hi > 0.0f ? 1 : -1);
-      const F2 t = next_t(c, a == 0 ? sh.x : (a == 1 ? sh.y : sh.z), a == 0 ? sl.x : (a == 1 ? sl.y : sl.z), iv);
-      if (a == 0) { c0 = c; t0 = t; }
-      else if (a == 1) { c1 = c; t1 = t; }
-      else { c2 = c; t2 = t; }
-      const int rest = mm & ~(1 << a);
-      if (rest) {
-        if (rest & 2) { c1 += iv1.hi > 0.0f ? 1 : -1; t1 = next_t(c1, sh.y, sl.y, iv1); }
-        if (rest & 4) { c2 += iv2.hi > 0.0f ? 1 : -1; t2 = next_t(c2, sh.z, sl.z, iv2); }
-      }
+    if (FSL) {  // Step 3j: the crossing against the halting radius, decided like the split
+      const float d = f2_diff(rn, rlim);
+      halt = d > 0.0f;
+      if (fabsf(d) <= emin + rlim.hi * kBandT) unsure = true;
     }
-    r = rn;
+    const float4 sh = __ldg(&S.s32);
+    const int c0 = a0.cell(sh.x, S.sa[0]), c1 = a1.cell(sh.y, S.sa[1]), c2 = a2.cell(sh.z, S.sa[2]);
+    if (unsure) {
+      const double rlim64 = !FSL ? __longlong_as_double(0x7ff0000000000000LL)
+                                 : ((int)age < A.n_ages ? A.rlim64[age] : 0.0);
+      const int d64 = decide64(A, src, l, pix, c0, c1, c2, rlim64);
+      split = (d64 & 8) != 0;
+      halt = (d64 & 64) != 0;
+      m0 = (d64 & 1) != 0;
+      m1 = (d64 & 2) != 0;
+      m2 = (d64 & 4) != 0;
+      ++fb;
+    }
+    const InstDev& I = A.inst[S.inst];
+    const bool out = (m0 && (a0.stride < 0 ? c0 == 0 : c0 + 1 == I.nx)) ||
+                     (m1 && (a1.stride < 0 ? c1 == 0 : c1 + 1 == I.ny)) ||
+                     (m2 && (a2.stride < 0 ? c2 == 0 : c2 + 1 == I.nz));
+    return (m0 ? 1 : 0) | (m1 ? 2 : 0) | (m2 ? 4 : 0) | (split ? 8 : 0) | (halt ? 64 : 0) | (out ? 128 : 0);
   }
 
+  // tau is at or near the termination: whether the package ends here (Step 3i).
+  template <bool FSL>
+  __device__ __forceinline__ bool terminates(const TraceArgs& A, LaneAcc& acc, float rn, bool halt) const {
+    const float d = f2_diff(F2{tau, tau_lo}, F2{A.tau_term32, A.tau_term32lo});
+    const float bnd = tau_bound(A, acc, rn) + tau * (4.0f * kBandT) + 1e-30f;
+    if (d > bnd) return true;
+    if (-d > bnd) return false;
+    // too close to call: the lineage's optical depth in FP64 (a lineage
+    // emitted in an earlier trace crossed other media, and a cut segment
+    // is not the cell's: there the pair's own decision stands)
+    acc.fallbacks_tau++;
+    double t64 = __longlong_as_double(0x7ff8000000000000LL);
+    if (!FSL || (age == 0 && !halt)) {
+      const SourceDev& S = A.src[src];
+      const float4 sh = __ldg(&S.s32);
+      t64 = retrace_tau64(A, src, lvl(), pix, a0.cell(sh.x, S.sa[0]), a1.cell(sh.y, S.sa[1]), a2.cell(sh.z, S.sa[2]));
+    }
+    return isnan(t64) ? (d > 0.0f) : (t64 > A.tau_term);
+  }
+
+  // One segment.  Returns EV_SPLIT before traversing a cell whose exit radius
+  // exceeds R_split, EV_DONE when the package is absorbed or leaves the box,
+  // EV_HALT (FSL) when it has travelled to its halting radius.
   template <bool FSL>
   __device__ __forceinline__ int step(const TraceArgs& A, LaneAcc& acc) {
+    // The next plane: the smallest high part, provably the nearest when no
+    // other is within 2^-20 of it (each is within 2^-22 of its distance).
     F2 rn;
-    unsigned fb = 0;
-    const int m = decide<FSL>(A, rn, fb);
-    acc.fallbacks += fb;
-    const int l = lvl();
-    if (m & 8) return EV_SPLIT;
+    rn.hi = fminf(a0.t.hi, fminf(a1.t.hi, a2.t.hi));
+    const float close = fmaf(rn.hi, kNear, rn.hi);
+    bool m0 = a0.t.hi <= close, m1 = a1.t.hi <= close, m2 = a2.t.hi <= close;
+    rn.lo = m0 ? a0.t.lo : (m1 ? a1.t.lo : a2.t.lo);
+    const bool rare = rn.hi >= lim || (m0 && m1) || (m2 && (m0 || m1));
+    int m = 0;
+    if (rare) {
+      unsigned fb = 0;
+      m = decide<FSL>(A, rn, fb);
+      acc.fallbacks += fb;
+      if (m & 8) return EV_SPLIT;
+      m0 = (m & 1) != 0;
+      m1 = (m & 2) != 0;
+      m2 = (m & 4) != 0;
+    }
     const bool halt = FSL && (m & 64);  // Step 3j: the segment ends at rlim
-    // segment length, kappa = sigma dx n_HI and dtau as FP32 pairs: the
-    // optical depth (pair) follows the FP64 sum to ~2^-44 where n_HI is a pair
-    F2 dr2 = f2_sub(halt ? rlim : rn, r);
-    if (dr2.hi < 0.0f) dr2 = F2{0.0f, 0.0f};
-    const float dr = dr2.hi;
-    const int idx = cell_index();
-    const float4 k32 = __ldg(&A.src[src].k32);  // sdx, w, rw, heat
-    const F2 kap2 = f2_mul(F2{k32.x, __ldg(&A.src[src].slo32.w)}, F2{nh, nh_lo});
-    const F2 dtau2 = f2_mul(kap2, dr2);
-    const float kap = kap2.hi;
-    const float dtau = dtau2.hi;
+    // segment length as a pair (both ends are pairs; |end| >= |r| or the
+    // difference of the high parts is exact)
+    const F2 end = halt ? rlim : rn;
+    const float dh = __fsub_rn(end.hi, r.hi);
+    const float dl = __fadd_rn(__fsub_rn(__fsub_rn(end.hi, dh), r.hi), __fsub_rn(end.lo, r.lo));
+    float dr = __fadd_rn(dh, dl);
+    float drl = __fadd_rn(__fsub_rn(dh, dr), dl);
+    if (dr > 0.0f) {
+      nseg++;
+    } else {
+      dr = 0.0f;
+      drl = 0.0f;
+    }
+    // kappa = sigma dx n_HI and dtau = kappa dr as pairs: the optical depth
+    // follows the FP64 sum to ~2^-44 where n_HI is a pair
+    const float kap = __fmul_rn(sdx, nh);
+    float kl = fmaf(sdx, nh, -kap);
+    if (PAIR) kl = fmaf(sdx, nh_lo, kl);
+    kl = fmaf(sdx_lo, nh, kl);
+    const float dp = __fmul_rn(kap, dr);
+    float de = fmaf(kap, dr, -dp);
+    de = fmaf(kap, drl, de);
+    de = fmaf(kl, dr, de);
+    const float dtau = __fadd_rn(dp, de);
+    const float dtl = __fadd_rn(__fsub_rn(dp, dtau), de);
     // transmitted fraction tr = e^-tau; phi = (1 - e^-tau)/tau from its Taylor
     // series below tau = 1/4 (7 terms: the first dropped term, tau^7 / 8!, is
     // below 1.6e-9 there, under FP32 rounding), else from tr.
@@ -844,91 +976,82 @@ struct Walk32 {
     // error (~1e-4 relative) is far inside the tolerance on k_ph
     float fcv = 1.0f;
     if (A.fc) {
-      const float L = r.hi * A.theta32[l];
+      const float rh = __fadd_rn(r.hi, r.lo);
+      const float L = rh * A.theta32[lvl()];
       if (L > 0.0f) {
         const float4 sh = __ldg(&A.src[src].s32);
-        const float rm = fmaf(0.5f, dr, r.hi);
-        const float n0 = iv0.hi != 0.0f ? __frcp_rn(iv0.hi) : 0.0f;
-        const float n1 = iv1.hi != 0.0f ? __frcp_rn(iv1.hi) : 0.0f;
-        const float n2 = iv2.hi != 0.0f ? __frcp_rn(iv2.hi) : 0.0f;
-        const float d = fmaxf(fabsf(fmaf(n0, rm, sh.x) - ((float)c0 + 0.5f)),
-                              fmaxf(fabsf(fmaf(n1, rm, sh.y) - ((float)c1 + 0.5f)),
-                                    fabsf(fmaf(n2, rm, sh.z) - ((float)c2 + 0.5f))));
+        const int* sa = A.src[src].sa;
+        const float rm = fmaf(0.5f, dr, rh);
+        const float d = fmaxf(a0.off_middle(rm, sh.x, sa[0]), fmaxf(a1.off_middle(rm, sh.y, sa[1]), a2.off_middle(rm, sh.z, sa[2])));
         const float f = 0.5f + (0.5f - d) / L;
         fcv = fminf(1.0f, f * f);
       }
     }
-    const float kadd = P * k32.y * dr * phi * fcv;
+    const float kadd = P * w * dr * phi * fcv;
     red_add(&K[idx], kadd);
-    if (k32.w != 0.0f) red_add(&G[idx], kadd * k32.w);
-    if (dr > 0.0f) nseg++;
+    if (heat != 0.0f) red_add(&G[idx], kadd * heat);
     P = P * tr;
     {
-      const F2 t2 = f2_add(F2{tau, tau_lo}, dtau2);
-      tau = t2.hi;
-      tau_lo = t2.lo;
+      // the larger summand first: the sum's rounding error is exact
+      const float s = __fadd_rn(tau, dtau);
+      const float e = __fsub_rn(fminf(tau, dtau), __fsub_rn(s, fmaxf(tau, dtau)));
+      tau_lo = __fadd_rn(tau_lo, __fadd_rn(e, dtl));
+      tau = s;
     }
-    // |tau - tau_FP64| grows by kappa times the pair errors of rn and r (each
-    // within 2^-40 rn + 2^-46 |s|/|n| on its axis; twice that, with margin),
-    // the rounding of the pair products (2^-37 dtau; 2^-22 dtau where n_HI is
-    // plain FP32) and of the pair sum (2^-44 tau)
-    {
-      const float4 sa = __ldg(&A.src[src].sabs32);
-      const float ab = fmaxf(sa.x * fabsf(iv0.hi), fmaxf(sa.y * fabsf(iv1.hi), sa.z * fabsf(iv2.hi)));
-      const float e_dtau = (level & 512u) ? 8.0f * kBandT : 4.0f * kEps32;
-      tau_err = tau_err + dtau * e_dtau + kap * (fmaf(rn.hi, 4.0f * kBandT, 1e-30f) + 4.0f * ab) +
-                tau * (kBandT / 16.0f);
-    }
-    {
-      const float d = f2_diff(F2{tau, tau_lo}, F2{A.tau_term32, A.tau_term32lo});
-      const float bnd = tau_err + tau * (4.0f * kBandT) + 1e-30f;
-      bool term = d > bnd;
-      if (!term && !(-d > bnd)) {
-        // too close to call: the lineage's optical depth in FP64 (a lineage
-        // emitted in an earlier trace crossed other media, and a cut segment
-        // is not the cell's: there the pair's own decision stands)
-        const double t64 = (!FSL || (age == 0 && !halt)) ? retrace_tau64(A, src, l, pix, c0, c1, c2)
-                                                         : __longlong_as_double(0x7ff8000000000000LL);
-        acc.fallbacks_tau++;
-        term = isnan(t64) ? (d > 0.0f) : (t64 > A.tau_term);
-      }
-      if (term) {
+    sk += kap;
+    if (fmaf(sk, q, tau) > A.tau_near) {
+      if (terminates<FSL>(A, acc, rn.hi, halt)) {
         if (nh > 0.0f) {
-          const float kres = P * k32.z / nh * fcv;
+          const float kres = P * __ldg(&A.src[src].k32.z) / nh * fcv;
           red_add(&K[idx], kres);
-          if (k32.w != 0.0f) red_add(&G[idx], kres * k32.w);
+          if (heat != 0.0f) red_add(&G[idx], kres * heat);
         }
-        acc.absorbed += (double)Pstart * unit(A);
+        acc.absorbed += (double)acc.Pstart * unit(A);
         return EV_DONE;
       }
     }
     if (halt) {
       r = rlim;
       const double u = unit(A);
-      acc.absorbed += ((double)Pstart - (double)P) * u;
+      acc.absorbed += ((double)acc.Pstart - (double)P) * u;
       acc.halted += (double)P * u;
       return EV_HALT;
     }
-    advance(A, m, rn);
-    if (!inside()) {
-      const double u = unit(A);
-      acc.absorbed += ((double)Pstart - (double)P) * u;
-      acc.escaped += (double)P * u;
+    if (m & 128) {
+      leave(A, acc);
       return EV_DONE;
     }
-    // the next cell is known before its density is needed: start the load now
-    load_nh(cell_index());
-    if (++steps > A.max_steps) {
-      set_status(A.ctl, RT_ERR_STATE);
-      const double u = unit(A);
-      acc.absorbed += ((double)Pstart - (double)P) * u;
-      acc.escaped += (double)P * u;
-      return EV_DONE;
-    }
+    // cross the plane; the next cell's density is loaded a step ahead
+    r = rn;
+    if (m0) { a0.next(); idx += a0.stride; }
+    if (m1) { a1.next(); idx += a1.stride; }
+    if (m2) { a2.next(); idx += a2.stride; }
+    load_nh();
     return EV_NONE;
   }
+  __device__ __forceinline__ void leave(const TraceArgs& A, LaneAcc& acc) const {
+    const double u = unit(A);
+    acc.absorbed += ((double)acc.Pstart - (double)P) * u;
+    acc.escaped += (double)P * u;
+  }
+  // Around the segments of a queue visit: the pair sum renormalised before,
+  // the bound on a package's segments tested after.
+  __device__ __forceinline__ void begin_visit() {
+    const F2 t2 = fast_two_sum(tau, tau_lo);
+    tau = t2.hi;
+    tau_lo = t2.lo;
+  }
+  __device__ __forceinline__ int end_visit(const TraceArgs& A, LaneAcc& acc, int n, int ev) {
+    steps += n;
+    if (ev == EV_NONE && steps > A.max_steps) {
+      set_status(A.ctl, RT_ERR_STATE);
+      leave(A, acc);
+      return EV_DONE;
+    }
+    return ev;
+  }
   __device__ __forceinline__ void on_split(const TraceArgs& A, LaneAcc& acc) const {
-    acc.absorbed += ((double)Pstart - (double)P) * unit(A);
+    acc.absorbed += ((double)acc.Pstart - (double)P) * unit(A);
   }
   __device__ __forceinline__ void on_start_outside(const TraceArgs& A, LaneAcc& acc) const {
     acc.escaped += (double)P * unit(A);
@@ -976,128 +1099,23 @@ __global__ void __launch_bounds__(kBlock, MinBlocks) trace_kernel(TraceArgs A) {
   W w;
   w.nseg = 0;
   bool active = false;
+  int ev = EV_NONE;
   long long ticket = -1;
   long long seen_out = -1;
   uint64_t seen_ns = global_ns();
   unsigned backoff = 256;  // ns; idle warps back off exponentially up to 4 us
 
   for (;;) {
-    // (1) idle lanes without a ticket take one (one atomic per warp)
-    const bool want = !active && ticket < 0;
-    const unsigned wm = __ballot_sync(kFull, want);
-    if (wm) {
-      const int leader = __ffs(wm) - 1;
-      unsigned long long base = 0;
-      if (lane == leader) base = atomicAdd(&A.ctl[CTL_HEAD], (unsigned long long)__popc(wm));
-      base = __shfl_sync(kFull, base, leader);
-      if (want) ticket = (long long)(base + __popc(wm & lt_mask));
-    }
-    // (2) turn tickets into packages
-    int ev = EV_NONE;
-    if (!active && ticket >= 0) {
-      const unsigned long long tk = (unsigned long long)ticket;
-      bool got = false, resumed = false;
-      uint32_t cell = 0;
-      if (tk < A.n_roots) {
-        const uint32_t ls = (uint32_t)(tk / A.npix0);
-        const uint32_t p = (uint32_t)(tk - (unsigned long long)ls * A.npix0);
-        const uint32_t gsrc = (uint32_t)A.src_first + ls;
-        w.load(W::root_rec(gsrc, (uint32_t)A.level0, p));
-        got = true;
-        const SourceDev& S = A.src[gsrc];
-        acc_switch(acc, w.nseg, S.inst, A, BB);
-        if (FSL) acc.emitted += w.emit(S) * S.unit;
-        else acc.emitted += S.unit;
-        LC.add(A, S.inst, S.local, A.level0, p, 1);
-      } else if (FSL && tk < qbase) {
-        // a package halted by the previous trace continues from its cell
-        const Rec* in = (const Rec*)A.res_in + (res_a + (tk - A.n_roots));
-        const Rec q = *in;
-        w.load(q);
-        cell = W::cell_of_record(q);
-        got = resumed = true;
-      } else {
-        const unsigned long long slot = tk - qbase;
-        if (slot < A.cap) {
-          Rec q;
-          if (W::template poll<FSL>(&queue[slot], epoch, q)) {
-            w.load(q);
-            got = true;
-          }
-        }
-      }
-      if (got) {
-        ticket = -1;
-        active = true;
-        acc_switch(acc, w.nseg, w.inst(A), A, BB);
-        if (FSL) w.set_rlim(A);
-        if (FSL && resumed) {
-          acc.resumed += (double)w.P * w.unit(A);
-          w.resume(A, cell);
-        } else if (!w.start(A)) {
-          w.on_start_outside(A, acc);
-          ev = EV_DONE;
-        }
-      }
-    }
-    // (3) a warp with nothing to trace checks for the end of the trace
-    const unsigned am = __ballot_sync(kFull, active && ev == EV_NONE);
-    if (am == 0 && __ballot_sync(kFull, ev == EV_DONE) == 0) {
-      long long outst = 0;
-      if (lane == 0) outst = (long long)ld_relaxed_u64(&A.ctl[CTL_OUTSTANDING]);
-      outst = __shfl_sync(kFull, outst, 0);
-      if (outst <= 0) break;
-      const uint64_t now = global_ns();
-      if (outst != seen_out) {
-        seen_out = outst;
-        seen_ns = now;
-      } else if ((long long)(now - seen_ns) > A.timeout_ns) {
-        if (lane == 0) set_status(A.ctl, RT_ERR_TIMEOUT);
-        break;
-      }
-      __nanosleep(backoff);
-      backoff = backoff < 4096 ? 2 * backoff : 4096;
-      continue;
-    }
-    backoff = 256;
-    seen_out = -1;  // the no-progress clock runs over one idle stretch only
-    // (4) trace a few segments
-    if (active && ev == EV_NONE) {
-      for (int it = 0; it < A.segs_per_iter; ++it) {
-        ev = w.template step<FSL>(A, acc);
-        if (ev != EV_NONE) break;
-      }
-    }
-    // The lanes left the loop at different steps: reconverge them here, before
-    // the warp-wide steps below.  (Without this barrier the same kernel ran
-    // 7-11 % slower on every workload measured.)
-    __syncwarp();
-    // (4b) halted packages go to the output store (one atomic per warp);
-    //      from here on they are finished packages
-    if (FSL) {
-      const unsigned hm = __ballot_sync(kFull, ev == EV_HALT);
-      if (hm) {
-        const int leader = __ffs(hm) - 1;
-        unsigned long long base = 0;
-        if (lane == leader) base = atomicAdd(&A.ctl[CTL_HALTED], (unsigned long long)__popc(hm));
-        base = __shfl_sync(kFull, base, leader);
-        if (ev == EV_HALT) {
-          const unsigned long long slot = base + __popc(hm & lt_mask);
-          if (slot < A.halt_cap) w.store_halted((Rec*)A.halt_out + slot);
-          else set_status(A.ctl, RT_ERR_QUEUE_OVERFLOW);
-          ev = EV_DONE;
-        }
-      }
-    }
-    // (5) a split keeps child 0 and hands children 1-3 first to lanes of this
-    //     warp that are free (no package and no ticket: in practice the
-    //     lanes whose package ended in this round; a lane holding a ticket
-    //     must stay free to take up the record that the ticket names), the
-    //     rest to the queue (slots reserved together); finished packages
-    //     leave the outstanding count.
+    // (1) What the last queue visit ended.  A split keeps child 0 and hands
+    //     children 1-3 first to lanes of this warp that are free (no package
+    //     and no ticket: in practice the lanes whose package ended in this
+    //     round; a lane holding a ticket must stay free to take up the record
+    //     that the ticket names), the rest to the queue (slots reserved
+    //     together); finished packages leave the outstanding count.
     //     One atomic per warp carries both: +3 per split, -1 per finished
     //     package.  Child j = 3 i + k - 1 of the i-th splitting lane goes to
     //     the j-th free lane when there is one, else to slot base + j - nin.
+    Start fresh = NO_START;  // a package starts in this lane now
     const bool split = (ev == EV_SPLIT);
     const unsigned sm = __ballot_sync(kFull, split);
     const unsigned dm = __ballot_sync(kFull, ev == EV_DONE);
@@ -1128,7 +1146,6 @@ __global__ void __launch_bounds__(kBlock, MinBlocks) trace_kernel(TraceArgs A) {
         active = false;
         ev = EV_NONE;
       }
-      bool fresh = false;  // a package starts in this lane now
       if (!FSL && nin) {
         const unsigned q = __popc(fm & lt_mask);
         const bool recv = ((fm >> lane) & 1u) && q < nin;
@@ -1138,9 +1155,7 @@ __global__ void __launch_bounds__(kBlock, MinBlocks) trace_kernel(TraceArgs A) {
           c.pix += q % 3u + 1u;
           w.load(c);
           active = true;
-          fresh = true;
-          acc_switch(acc, w.nseg, w.inst(A), A, BB);
-          if (FSL) w.set_rlim(A);
+          fresh = START_CHILD;
         }
       }
       if (split) {
@@ -1162,23 +1177,120 @@ __global__ void __launch_bounds__(kBlock, MinBlocks) trace_kernel(TraceArgs A) {
           atomicAdd(&A.ctl[CTL_OUTSTANDING], (unsigned long long)(-(long long)dropped));
         }
         w.become_child0();
-        fresh = true;
+        ev = EV_NONE;
+        fresh = START_CHILD;
       }
-      if (fresh) {
-        if (w.start(A)) ev = EV_NONE;
-        else {
-          w.on_start_outside(A, acc);
+    }
+    // (2) idle lanes without a ticket take one (one atomic per warp)
+    const bool want = !active && ticket < 0;
+    const unsigned wm = __ballot_sync(kFull, want);
+    if (wm) {
+      const int leader = __ffs(wm) - 1;
+      unsigned long long base = 0;
+      if (lane == leader) base = atomicAdd(&A.ctl[CTL_HEAD], (unsigned long long)__popc(wm));
+      base = __shfl_sync(kFull, base, leader);
+      if (want) ticket = (long long)(base + __popc(wm & lt_mask));
+    }
+    // (3) turn tickets into packages
+    uint32_t cell = 0;
+    if (!active && ticket >= 0) {
+      const unsigned long long tk = (unsigned long long)ticket;
+      if (tk < A.n_roots) {
+        const uint32_t ls = (uint32_t)(tk / A.npix0);
+        const uint32_t p = (uint32_t)(tk - (unsigned long long)ls * A.npix0);
+        w.load(W::root_rec((uint32_t)A.src_first + ls, (uint32_t)A.level0, p));
+        fresh = START_ROOT;
+      } else if (FSL && tk < qbase) {
+        // a package halted by the previous trace continues from its cell
+        const Rec q = *((const Rec*)A.res_in + (res_a + (tk - A.n_roots)));
+        w.load(q);
+        cell = W::cell_of_record(q);
+        fresh = START_RESUMED;
+      } else {
+        const unsigned long long slot = tk - qbase;
+        if (slot < A.cap) {
+          Rec q;
+          if (W::template poll<FSL>(&queue[slot], epoch, q)) {
+            w.load(q);
+            fresh = START_CHILD;
+          }
+        }
+      }
+      if (fresh != NO_START) {
+        ticket = -1;
+        active = true;
+      }
+    }
+    // (4) start the new packages, wherever they came from (one that starts
+    //     outside the box is finished at the next (1))
+    __syncwarp();
+    if (fresh != NO_START) {
+      const SourceDev& S = A.src[w.src];
+      acc_switch(acc, w.nseg, S.inst, A, BB);
+      if (FSL) w.set_rlim(A);
+      if (fresh == START_ROOT) {
+        if (FSL) acc.emitted += w.emit(S) * S.unit;
+        else acc.emitted += S.unit;
+        LC.add(A, S.inst, S.local, A.level0, w.pix, 1);
+      }
+      if (FSL && fresh == START_RESUMED) acc.resumed += (double)w.P * S.unit;
+      if (!w.template start<FSL>(A, acc, FSL && fresh == START_RESUMED, cell)) {
+        w.on_start_outside(A, acc);
+        ev = EV_DONE;
+      }
+    }
+    // (5) a warp with nothing to trace checks for the end of the trace
+    const unsigned am = __ballot_sync(kFull, active);
+    if (am == 0) {
+      long long outst = 0;
+      if (lane == 0) outst = (long long)ld_relaxed_u64(&A.ctl[CTL_OUTSTANDING]);
+      outst = __shfl_sync(kFull, outst, 0);
+      if (outst <= 0) break;
+      const uint64_t now = global_ns();
+      if (outst != seen_out) {
+        seen_out = outst;
+        seen_ns = now;
+      } else if ((long long)(now - seen_ns) > A.timeout_ns) {
+        if (lane == 0) set_status(A.ctl, RT_ERR_TIMEOUT);
+        break;
+      }
+      __nanosleep(backoff);
+      backoff = backoff < 4096 ? 2 * backoff : 4096;
+      continue;
+    }
+    backoff = 256;
+    seen_out = -1;  // the no-progress clock runs over one idle stretch only
+    // (6) trace a few segments
+    if (active && ev == EV_NONE) {
+      w.begin_visit();
+      int it = 0;
+      for (; it < A.segs_per_iter; ++it) {
+        ev = w.template step<FSL>(A, acc);
+        if (ev != EV_NONE) break;
+      }
+      ev = w.end_visit(A, acc, it, ev);
+      if (ev == EV_SPLIT || ev == EV_HALT) w.seal(A, acc);
+    }
+    // The lanes left the loop at different steps: reconverge them here, before
+    // the warp-wide steps.  (Without this barrier the same kernel ran
+    // 7-11 % slower on every workload measured.)
+    __syncwarp();
+    // (7) halted packages go to the output store (one atomic per warp);
+    //     from here on they are finished packages
+    if (FSL) {
+      const unsigned hm = __ballot_sync(kFull, ev == EV_HALT);
+      if (hm) {
+        const int leader = __ffs(hm) - 1;
+        unsigned long long base = 0;
+        if (lane == leader) base = atomicAdd(&A.ctl[CTL_HALTED], (unsigned long long)__popc(hm));
+        base = __shfl_sync(kFull, base, leader);
+        if (ev == EV_HALT) {
+          const unsigned long long slot = base + __popc(hm & lt_mask);
+          if (slot < A.halt_cap) w.store_halted((Rec*)A.halt_out + slot);
+          else set_status(A.ctl, RT_ERR_QUEUE_OVERFLOW);
           ev = EV_DONE;
         }
       }
-    }
-    // (6) a child 0 that starts outside the box is finished too
-    const bool done = (ev == EV_DONE);
-    const unsigned dm2 = __ballot_sync(kFull, done);
-    if (dm2) {
-      if (lane == __ffs(dm2) - 1)
-        atomicAdd(&A.ctl[CTL_OUTSTANDING], (unsigned long long)(-(long long)__popc(dm2)));
-      if (done) active = false;
     }
   }
   acc.segments += w.nseg;
@@ -1335,27 +1447,36 @@ cudaError_t launch_flight_table(const double* old, double* neu, float2* neu32, i
 constexpr int kMinBlocks64 = 2;
 constexpr int kMinBlocks32 = TRACE_MIN_BLOCKS;
 
-cudaError_t trace_occupancy(int precision, int fsl, int block, int* blocks_per_sm) {
-  if (block != kBlock) return cudaErrorInvalidValue;
+using TraceKernel = void (*)(TraceArgs);
+// The instantiation for a launch; null for a combination that has none.
+// fsl: finite speed of light (A.rlim*, res_in, halt_out set).
+static TraceKernel trace_instance(int precision, int fsl, int variant) {
   if (precision == RT_FP64)
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        blocks_per_sm,
-        fsl ? trace_kernel<Walk64, kMinBlocks64, true> : trace_kernel<Walk64, kMinBlocks64, false>, block, 0);
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-      blocks_per_sm, fsl ? trace_kernel<Walk32, kMinBlocks32, true> : trace_kernel<Walk32, kMinBlocks32, false>,
-      block, 0);
+    return fsl ? trace_kernel<Walk64, kMinBlocks64, true> : trace_kernel<Walk64, kMinBlocks64, false>;
+  switch (variant) {
+    case WALK_EXACT:
+      return fsl ? trace_kernel<Walk32<true, true>, kMinBlocks32, true>
+                 : trace_kernel<Walk32<true, true>, kMinBlocks32, false>;
+    case WALK_ANY:
+      return fsl ? trace_kernel<Walk32<false, true>, kMinBlocks32, true>
+                 : trace_kernel<Walk32<false, true>, kMinBlocks32, false>;
+    case WALK_ANY_PLAIN:
+      if (!fsl) return trace_kernel<Walk32<false, false>, kMinBlocks32, false>;
+  }
+  return nullptr;
 }
 
-// fsl: the finite-speed-of-light instantiation (A.rlim*, res_in, halt_out set)
-cudaError_t launch_trace(int precision, int fsl, const TraceArgs& A, int grid, int block, cudaStream_t st) {
-  if (block != kBlock) return cudaErrorInvalidValue;
-  if (precision == RT_FP64) {
-    if (fsl) trace_kernel<Walk64, kMinBlocks64, true><<<grid, block, 0, st>>>(A);
-    else trace_kernel<Walk64, kMinBlocks64, false><<<grid, block, 0, st>>>(A);
-  } else {
-    if (fsl) trace_kernel<Walk32, kMinBlocks32, true><<<grid, block, 0, st>>>(A);
-    else trace_kernel<Walk32, kMinBlocks32, false><<<grid, block, 0, st>>>(A);
-  }
+cudaError_t trace_occupancy(int precision, int fsl, int variant, int block, int* blocks_per_sm) {
+  const TraceKernel k = trace_instance(precision, fsl, variant);
+  if (!k || block != kBlock) return cudaErrorInvalidValue;
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, block, 0);
+}
+
+cudaError_t launch_trace(int precision, int fsl, int variant, const TraceArgs& A, int grid, int block,
+                         cudaStream_t st) {
+  const TraceKernel k = trace_instance(precision, fsl, variant);
+  if (!k || block != kBlock) return cudaErrorInvalidValue;
+  k<<<grid, block, 0, st>>>(A);
   return cudaGetLastError();
 }
 

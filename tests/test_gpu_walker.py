@@ -1,0 +1,49 @@
+"""Edges of the FP32 walker's plane arithmetic against the FP64 oracle: its two
+forms (every source on the 1/16-cell lattice, or any position), sources on and
+within rounding of cell planes and box faces, axes longer than the lattice
+form takes, and both forms' optical depths up to the termination.
+
+Counts per level and the created-set checksum must be bit-exact; k_ph, Gamma
+and the budget within the bounds of tests/parity.py.
+"""
+import numpy as np
+import pytest
+
+import parity
+from paper_1012_2865_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+LATTICE = [(0.0, 0.0, 0.0), (8.0, 5.0, 3.0), (4.5, 7.5, 2.5), (3.0625, 9.9375, 6.5), (16.0, 11.0, 7.0)]
+BESIDE = [(8.0 + 1e-12, 5.0 - 1e-9, 3.0 + 1e-7), (1e-13, 11.0 - 1e-9, 3.5), (16.0 - 1e-12, 5.5, 1e-9),
+          (7.3, 5.000001, 2.9999999), (8.0, 5.0, 3.3)]
+
+
+def _grid(dims, cells, xlo, seed=3):
+    rng = np.random.default_rng(seed)
+    box = synth.box_cm(dims[0], 6.6 * dims[0] / 32)
+    dx = box / dims[0]
+    n = len(cells)
+    n_H = 2e-3 if dims == (1, 1, 1) else synth.lognormal_density(None, mean=2e-3, seed=seed, dims=dims)
+    return synth._grid(dims, box, n_H,
+                       rng.uniform(xlo, 1.0, int(np.prod(dims))) if xlo > 0 else 1e-4, np.asarray(cells) * dx,
+                       np.full(n, 1e49), rng.uniform(13.6, 29.6, n), np.full(n, synth.SIGMA_HI))
+
+
+@pytest.mark.parametrize("xlo", [0.9, 0.0])  # rays that are absorbed; rays that leave the box
+@pytest.mark.parametrize("cells", [LATTICE, BESIDE, LATTICE + BESIDE], ids=["lattice", "beside", "both"])
+def test_sources_on_and_beside_planes(cells, xlo):
+    g = _grid((16, 11, 7), cells, xlo)
+    _, b, r = parity.run_gpu(g, "fp32_mixed")
+    parity.assert_trace_parity(g, b, r, parity.run_oracle(g), "fp32_mixed")
+
+
+@pytest.mark.parametrize("dims,cells", [
+    ((1, 1, 1), [(0.5, 0.5, 0.5), (0.1, 0.7, 0.9)]),
+    ((5000, 2, 3), [(2500.5, 0.5, 1.5), (4096.5, 1.0, 2.0), (0.3, 1.9, 0.1)]),
+    ((2, 4097, 1), [(1.0, 4096.5, 0.5), (0.25, 17.0, 0.5)]),
+], ids=["one-cell", "5000", "4097"])
+def test_short_and_long_axes(dims, cells):
+    g = _grid(dims, cells, 0.0)
+    _, b, r = parity.run_gpu(g, "fp32_mixed")
+    parity.assert_trace_parity(g, b, r, parity.run_oracle(g), "fp32_mixed")
