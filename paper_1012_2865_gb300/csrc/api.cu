@@ -23,7 +23,7 @@ namespace rtg {
 cudaError_t launch_trace_init(unsigned long long* ctl, void* queue, size_t queue_bytes, unsigned long long n_roots,
                               int first_pass, int mode, unsigned long long in_cap, int pass, int passes,
                               cudaStream_t st);
-cudaError_t trace_occupancy(int precision, int fsl, int variant, int block, int* blocks_per_sm);
+cudaError_t trace_occupancy(int precision, int fsl, int fc, int variant, int block, int* blocks_per_sm);
 cudaError_t launch_trace(int precision, int fsl, int variant, const TraceArgs& A, int grid, int block,
                          cudaStream_t st);
 cudaError_t launch_flight_table(const double* old, double* neu, float2* neu32, int n_new, double c_dt,
@@ -33,8 +33,11 @@ cudaError_t launch_chem(int precision, long long ncell, const double* nH, double
                         const void* K, void* nhi, double h, int nsub, double alpha, cudaStream_t st);
 cudaError_t launch_refresh(int precision, long long ncell, const double* nH, const double* xHI,
                            void* nhi, cudaStream_t st);
-cudaError_t launch_convert(long long n, const void* src, int src_dtype, void* dst, int dst_dtype,
-                           cudaStream_t st, double scale = 1.0);
+cudaError_t launch_convert(long long n, const void* src, int src_dtype, void* dst, cudaStream_t st);
+cudaError_t launch_read_rates(int precision, long long n, const void* K, const void* G, const double* x, void* ok,
+                              void* og, void* ox, int dtype, double scale, cudaStream_t st);
+cudaError_t launch_write_rates(long long n, const void* k, const void* g, int dtype, void* kg, double scale,
+                               cudaStream_t st);
 cudaError_t launch_complement(long long n, const double* x, double* out, cudaStream_t st);
 cudaError_t launch_commit_state(int precision, long long n, unsigned long long* ctl, const double* sn,
                                const double* sx, const double* sz, double* nH, double* xHI, double* xHII, void* nhi,
@@ -209,8 +212,8 @@ struct rt_grid {
   double* nH = nullptr;
   double* xHI = nullptr;
   double* xHII = nullptr;
-  void* nhi = nullptr;  // FP64 or FP32
-  void* K = nullptr;
+  void* nhi = nullptr;  // FP64, or FP32 pairs
+  void* K = nullptr;    // FP64, or (k_ph, Gamma) FP32 pairs (then G is null)
   void* G = nullptr;
   double* acc = nullptr;               // kAccWords doubles
   unsigned long long* cnt = nullptr;   // kCntWords
@@ -273,14 +276,15 @@ struct rt_grid {
   }
 };
 
-static size_t elem_bytes(int precision) { return precision == RT_FP64 ? 8 : 4; }
+// Bytes of every per-cell array of a grid: FP64, or two FP32 words (n_HI pairs;
+// k_ph and Gamma together).
+static size_t cell_bytes(const rt_grid* g) { return (size_t)g->ncell * 8; }
 
 // The trace kernel's view of a grid (slot `inst` of a launch).
 static InstDev inst_of(const rt_grid* g) {
   InstDev I;
   memset(&I, 0, sizeof I);
   I.nx = g->nx; I.ny = g->ny; I.nz = g->nz;
-  I.flags = g->precision == RT_FP32_MIXED ? kInstNhiPair : 0;
   I.nhi = g->nhi; I.nH = g->nH; I.xHI = g->xHI; I.xHII = g->xHII; I.K = g->K; I.G = g->G;
   I.acc = g->acc; I.cnt = g->cnt;
   for (int t = 0; t < 2; ++t) {
@@ -378,7 +382,7 @@ int rt_create_grid(rt_ctx* ctx, const rt_grid_desc* d, void* stream, rt_grid** o
   g->dx = d->box_len_cm / d->nx;
   g->precision = d->precision;
   g->stream = (cudaStream_t)stream;
-  const size_t n8 = (size_t)ncell * 8, ne = (size_t)ncell * elem_bytes(d->precision);
+  const size_t n8 = cell_bytes(g);
   int rc = RT_OK;
 #define ALLOC(p, b)                                        \
   do {                                                     \
@@ -391,9 +395,9 @@ int rt_create_grid(rt_ctx* ctx, const rt_grid_desc* d, void* stream, rt_grid** o
   ALLOC(g->nH, n8);
   ALLOC(g->xHI, n8);
   ALLOC(g->xHII, n8);
-  ALLOC(g->nhi, d->precision == RT_FP32_MIXED ? 2 * ne : ne);  // mixed: (hi, lo) pairs
-  ALLOC(g->K, ne);
-  ALLOC(g->G, ne);
+  ALLOC(g->nhi, n8);
+  ALLOC(g->K, n8);
+  if (d->precision == RT_FP64) ALLOC(g->G, n8);
   ALLOC(g->acc, kAccWords * sizeof(double));
   ALLOC(g->cnt, kCntWords * sizeof(unsigned long long));
   ALLOC(g->inst_dev, sizeof(InstDev));
@@ -418,8 +422,8 @@ int rt_create_grid(rt_ctx* ctx, const rt_grid_desc* d, void* stream, rt_grid** o
   if (e != cudaSuccess) { delete g; return fail(RT_ERR_CUDA, "refresh: %s", cudaGetErrorString(e)); }
   g_launches.fetch_add(1);
   e = cudaMemsetAsync(g->ts.ctl, 0, CTL_N * sizeof(unsigned long long), st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(g->K, 0, ne, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(g->G, 0, ne, st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(g->K, 0, n8, st);
+  if (e == cudaSuccess && g->G) e = cudaMemsetAsync(g->G, 0, n8, st);
   const InstDev I = inst_of(g);
   if (e == cudaSuccess) e = cudaMemcpyAsync(g->inst_dev, &I, sizeof I, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMallocHost(&g->host_rb, 4096);
@@ -789,12 +793,11 @@ static int enqueue_trace(rt_grid* g, const rt_trace_params* p, int passes, bool 
   int rc = prepare_sources(g, p->level0, fsl);
   if (rc) return rc;
   cudaStream_t st = g->stream;
-  const size_t ne = (size_t)g->ncell * elem_bytes(g->precision);
   // Step 2: k_ph, Gamma and the budget words in one launch
-  LAUNCH_TRY(launch_zero_fields(g->K, g->G, ne, g->acc, kAccWords, g->cnt, kCntWords, st));
+  LAUNCH_TRY(launch_zero_fields(g->K, g->G, cell_bytes(g), g->acc, kAccWords, g->cnt, kCntWords, st));
   for (int t = 0; t < 2 && g->he; ++t) {
-    CUDA_TRY(cudaMemsetAsync(g->Khe[t], 0, ne, st));
-    CUDA_TRY(cudaMemsetAsync(g->Ghe[t], 0, ne, st));
+    CUDA_TRY(cudaMemsetAsync(g->Khe[t], 0, cell_bytes(g), st));
+    if (g->Ghe[t]) CUDA_TRY(cudaMemsetAsync(g->Ghe[t], 0, cell_bytes(g), st));
   }
   const int nsrc = (int)g->src.size();
   if (nsrc == 0) {
@@ -835,7 +838,7 @@ static int enqueue_trace(rt_grid* g, const rt_trace_params* p, int passes, bool 
   }
   const int block = 256;  // the trace kernel is compiled for 256-thread blocks
   int per_sm = 0;
-  CUDA_TRY(trace_occupancy(g->precision, fsl ? 1 : 0, g->variant, block, &per_sm));
+  CUDA_TRY(trace_occupancy(g->precision, fsl ? 1 : 0, A.fc, g->variant, block, &per_sm));
   if (per_sm < 1) per_sm = 1;
   if (p->blocks_per_sm > 0 && p->blocks_per_sm < per_sm) per_sm = p->blocks_per_sm;
   if ((rc = g->ts.bind_rows(A, per_sm * g->ctx->num_sms, 1))) return rc;
@@ -1122,18 +1125,6 @@ int rt_set_state_async(rt_grid* g, const double* n_H, const double* x_HI, const 
   return RT_OK;
 }
 
-// One field into a snapshot or a caller's device buffer: a device-to-device
-// copy when neither the element type nor the scale changes, else the
-// conversion kernel.
-static int copy_or_convert(long long n, const void* src, int sdt, void* dst, int ddt, double scale, cudaStream_t st) {
-  if (sdt == ddt && scale == 1.0) {
-    CUDA_TRY(cudaMemcpyAsync(dst, src, (size_t)n * (sdt == RT_DTYPE_F64 ? 8 : 4), cudaMemcpyDeviceToDevice, st));
-    return RT_OK;
-  }
-  LAUNCH_TRY(launch_convert(n, src, sdt, dst, ddt, st, scale));
-  return RT_OK;
-}
-
 int rt_get_rates_async(rt_grid* g, void* kph, void* gamma, void* x_HI, int dtype, int mem_kind) {
   NvtxRange nr("rt_get_rates_async");
   if (!g) return fail(RT_ERR_INVALID_ARG, "rt_get_rates_async: grid is NULL");
@@ -1143,30 +1134,26 @@ int rt_get_rates_async(rt_grid* g, void* kph, void* gamma, void* x_HI, int dtype
     return fail(RT_ERR_INVALID_ARG, "rt_get_rates_async: mem_kind %d", mem_kind);
   if (g->batch) return fail(RT_ERR_STATE, "rt_get_rates_async: the grid is in a batch (use rt_get_rates)");
   CUDA_TRY(cudaSetDevice(g->ctx->device));
-  const int kd = g->precision == RT_FP64 ? RT_DTYPE_F64 : RT_DTYPE_F32;
-  const void* src[3] = {g->K, g->G, g->xHI};
-  const int sdt[3] = {kd, kd, RT_DTYPE_F64};
-  const double scale[3] = {1.0, gamma_scale(g), 1.0};
   void* dst[3] = {kph, gamma, x_HI};
+  if (!kph && !gamma && !x_HI) return RT_OK;
   const long long n = g->ncell;
   cudaStream_t st = g->stream;
   if (mem_kind == RT_MEM_DEVICE) {
-    for (int f = 0; f < 3; ++f)
-      if (dst[f]) {
-        int rc = copy_or_convert(n, src[f], sdt[f], dst[f], dtype, scale[f], st);
-        if (rc) return rc;
-      }
+    LAUNCH_TRY(launch_read_rates(g->precision, n, g->K, g->G, g->xHI, kph, gamma, x_HI, dtype, gamma_scale(g), st));
     return RT_OK;
   }
   int rc = ensure_async(g, false, true);
   if (rc) return rc;
   const size_t eb = dtype == RT_DTYPE_F64 ? 8 : 4, region = (size_t)n * 8;
   // a field's staging region is free once its previous read-back has left it
+  void* stage[3] = {nullptr, nullptr, nullptr};
   for (int f = 0; f < 3; ++f) {
     if (!dst[f]) continue;
     CUDA_TRY(cudaStreamWaitEvent(st, g->ev_dl[f], 0));
-    if ((rc = copy_or_convert(n, src[f], sdt[f], g->dn_stage + f * region, dtype, scale[f], st))) return rc;
+    stage[f] = g->dn_stage + f * region;
   }
+  LAUNCH_TRY(launch_read_rates(g->precision, n, g->K, g->G, g->xHI, stage[0], stage[1], stage[2], dtype, gamma_scale(g),
+                               st));
   CUDA_TRY(cudaEventRecord(g->ev_snap, st));
   CUDA_TRY(cudaStreamWaitEvent(g->dn, g->ev_snap, 0));
   for (int f = 0; f < 3; ++f) {
@@ -1184,29 +1171,42 @@ int rt_wait_rates(rt_grid* g) {
   return RT_OK;
 }
 
-static int copy_field(rt_grid* g, const void* src, int src_dtype, void* dst, int dtype, int mem_kind,
-                      double scale = 1.0) {
-  if (!dst) return RT_OK;
+// k_ph and Gamma (of rate arrays K, G) and x_HI (of xHI) into the caller's
+// buffers, each where one is given: fields of a type the caller wants as they
+// are go straight to the host, the others through one kernel.
+static int read_fields(rt_grid* g, const void* K, const void* G, const double* xHI, void* kph, void* gamma, void* x,
+                       int dtype, int mem_kind) {
   const long long n = g->ncell;
-  const size_t eb = dtype == RT_DTYPE_F64 ? 8 : 4;
+  const size_t nb = (size_t)n * (dtype == RT_DTYPE_F64 ? 8 : 4);
   cudaStream_t st = g->stream;
+  if (!kph && !gamma && !x) return RT_OK;
   if (mem_kind == RT_MEM_DEVICE) {
-    LAUNCH_TRY(launch_convert(n, src, src_dtype, dst, dtype, st, scale));
+    LAUNCH_TRY(launch_read_rates(g->precision, n, K, G, xHI, kph, gamma, x, dtype, gamma_scale(g), st));
     return RT_OK;
   }
-  if (src_dtype == dtype && scale == 1.0) {  // same type: straight to the host
-    CUDA_TRY(cudaMemcpyAsync(dst, src, (size_t)n * eb, cudaMemcpyDeviceToHost, st));
-    return RT_OK;
+  if (dtype == RT_DTYPE_F64) {
+    if (x) CUDA_TRY(cudaMemcpyAsync(x, xHI, nb, cudaMemcpyDeviceToHost, st));
+    x = nullptr;
+    if (g->precision == RT_FP64) {
+      if (kph) CUDA_TRY(cudaMemcpyAsync(kph, K, nb, cudaMemcpyDeviceToHost, st));
+      if (gamma) CUDA_TRY(cudaMemcpyAsync(gamma, G, nb, cudaMemcpyDeviceToHost, st));
+      kph = gamma = nullptr;
+    }
   }
-  void* tmp = nullptr;
-  CUDA_TRY(cudaMallocAsync(&tmp, (size_t)n * eb, st));
-  cudaError_t e = launch_convert(n, src, src_dtype, tmp, dtype, st, scale);
-  if (e == cudaSuccess) {
-    g_launches.fetch_add(1);
-    e = cudaMemcpyAsync(dst, tmp, (size_t)n * eb, cudaMemcpyDeviceToHost, st);
-  }
+  void* dst[3] = {kph, gamma, x};
+  const int nf = (kph ? 1 : 0) + (gamma ? 1 : 0) + (x ? 1 : 0);
+  if (nf == 0) return RT_OK;
+  char* tmp = nullptr;
+  CUDA_TRY(cudaMallocAsync((void**)&tmp, nf * nb, st));
+  void* stage[3] = {nullptr, nullptr, nullptr};
+  for (int f = 0, k = 0; f < 3; ++f)
+    if (dst[f]) stage[f] = tmp + nb * k++;
+  cudaError_t e = launch_read_rates(g->precision, n, K, G, xHI, stage[0], stage[1], stage[2], dtype, gamma_scale(g), st);
+  if (e == cudaSuccess) g_launches.fetch_add(1);
+  for (int f = 0; f < 3 && e == cudaSuccess; ++f)
+    if (dst[f]) e = cudaMemcpyAsync(dst[f], stage[f], nb, cudaMemcpyDeviceToHost, st);
   cudaFreeAsync(tmp, st);
-  if (e != cudaSuccess) return fail(RT_ERR_CUDA, "copy_field: %s", cudaGetErrorString(e));
+  if (e != cudaSuccess) return fail(RT_ERR_CUDA, "reading fields: %s", cudaGetErrorString(e));
   return RT_OK;
 }
 
@@ -1218,7 +1218,7 @@ int rt_set_absorbers(rt_grid* g, const double* n_HeI, const double* n_HeII, int 
   CUDA_TRY(cudaSetDevice(g->ctx->device));
   cudaStream_t st = g->stream;
   const long long n = g->ncell;
-  const size_t n8 = (size_t)n * 8, ne = (size_t)n * elem_bytes(g->precision);
+  const size_t n8 = cell_bytes(g);
   // staged and checked before the grid's arrays change
   double* stage = nullptr;
   CUDA_TRY(cudaMallocAsync((void**)&stage, 2 * n8, st));
@@ -1250,12 +1250,12 @@ int rt_set_absorbers(rt_grid* g, const double* n_HeI, const double* n_HeII, int 
       e = cudaMalloc((void**)&g->nhe64[t], n8);
       if (e == cudaSuccess) {
         if (g->precision == RT_FP64) g->nhe[t] = g->nhe64[t];
-        else e = cudaMalloc(&g->nhe[t], 2 * ne);  // FP32 pairs
+        else e = cudaMalloc(&g->nhe[t], n8);  // FP32 pairs
       }
-      if (e == cudaSuccess) e = cudaMalloc(&g->Khe[t], ne);
-      if (e == cudaSuccess) e = cudaMalloc(&g->Ghe[t], ne);
-      if (e == cudaSuccess) e = cudaMemsetAsync(g->Khe[t], 0, ne, st);
-      if (e == cudaSuccess) e = cudaMemsetAsync(g->Ghe[t], 0, ne, st);
+      if (e == cudaSuccess) e = cudaMalloc(&g->Khe[t], cell_bytes(g));
+      if (e == cudaSuccess && g->precision == RT_FP64) e = cudaMalloc(&g->Ghe[t], cell_bytes(g));
+      if (e == cudaSuccess) e = cudaMemsetAsync(g->Khe[t], 0, cell_bytes(g), st);
+      if (e == cudaSuccess && g->Ghe[t]) e = cudaMemsetAsync(g->Ghe[t], 0, cell_bytes(g), st);
       if (e != cudaSuccess) {
         cudaFreeAsync(stage, st);
         cudaStreamSynchronize(st);
@@ -1307,11 +1307,7 @@ int rt_get_rates(rt_grid* g, void* kph, void* gamma, void* x_HI, int dtype, int 
   if (dtype != RT_DTYPE_F64 && dtype != RT_DTYPE_F32) return fail(RT_ERR_INVALID_ARG, "rt_get_rates: dtype %d", dtype);
   if (mem_kind != RT_MEM_HOST && mem_kind != RT_MEM_DEVICE) return fail(RT_ERR_INVALID_ARG, "rt_get_rates: mem_kind %d", mem_kind);
   CUDA_TRY(cudaSetDevice(g->ctx->device));
-  const int kd = g->precision == RT_FP64 ? RT_DTYPE_F64 : RT_DTYPE_F32;
-  int rc;
-  if ((rc = copy_field(g, g->K, kd, kph, dtype, mem_kind))) return rc;
-  if ((rc = copy_field(g, g->G, kd, gamma, dtype, mem_kind, gamma_scale(g)))) return rc;
-  if ((rc = copy_field(g, g->xHI, RT_DTYPE_F64, x_HI, dtype, mem_kind))) return rc;
+  if (int rc = read_fields(g, g->K, g->G, g->xHI, kph, gamma, x_HI, dtype, mem_kind)) return rc;
   CUDA_TRY(cudaStreamSynchronize(g->stream));
   return RT_OK;
 }
@@ -1326,10 +1322,7 @@ int rt_get_rates_typed(rt_grid* g, int type, void* kph, void* gamma, int dtype, 
   if (mem_kind != RT_MEM_HOST && mem_kind != RT_MEM_DEVICE)
     return fail(RT_ERR_INVALID_ARG, "rt_get_rates_typed: mem_kind %d", mem_kind);
   CUDA_TRY(cudaSetDevice(g->ctx->device));
-  const int kd = g->precision == RT_FP64 ? RT_DTYPE_F64 : RT_DTYPE_F32;
-  int rc;
-  if ((rc = copy_field(g, g->Khe[type - 1], kd, kph, dtype, mem_kind))) return rc;
-  if ((rc = copy_field(g, g->Ghe[type - 1], kd, gamma, dtype, mem_kind, gamma_scale(g)))) return rc;
+  if (int rc = read_fields(g, g->Khe[type - 1], g->Ghe[type - 1], nullptr, kph, gamma, nullptr, dtype, mem_kind)) return rc;
   CUDA_TRY(cudaStreamSynchronize(g->stream));
   return RT_OK;
 }
@@ -1341,25 +1334,27 @@ int rt_set_rates(rt_grid* g, const void* kph, const void* gamma, int dtype, int 
   if (mem_kind != RT_MEM_HOST && mem_kind != RT_MEM_DEVICE) return fail(RT_ERR_INVALID_ARG, "rt_set_rates: mem_kind %d", mem_kind);
   CUDA_TRY(cudaSetDevice(g->ctx->device));
   const long long n = g->ncell;
-  const size_t eb = dtype == RT_DTYPE_F64 ? 8 : 4;
-  const int kd = g->precision == RT_FP64 ? RT_DTYPE_F64 : RT_DTYPE_F32;
+  const size_t nb = (size_t)n * (dtype == RT_DTYPE_F64 ? 8 : 4);
   cudaStream_t st = g->stream;
-  const void* src[2] = {kph, gamma};
-  void* dst[2] = {g->K, g->G};
-  const double scale[2] = {1.0, 1.0 / gamma_scale(g)};
-  for (int f = 0; f < 2; ++f) {
-    if (mem_kind == RT_MEM_DEVICE) {
-      LAUNCH_TRY(launch_convert(n, src[f], dtype, dst[f], kd, st, scale[f]));
-      continue;
-    }
-    void* tmp = nullptr;
-    CUDA_TRY(cudaMallocAsync(&tmp, (size_t)n * eb, st));
-    cudaError_t e = cudaMemcpyAsync(tmp, src[f], (size_t)n * eb, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = launch_convert(n, tmp, dtype, dst[f], kd, st, scale[f]);
-    if (e == cudaSuccess) g_launches.fetch_add(1);
-    cudaFreeAsync(tmp, st);
-    if (e != cudaSuccess) return fail(RT_ERR_CUDA, "rt_set_rates: %s", cudaGetErrorString(e));
+  char* tmp = nullptr;  // host arrays are staged
+  cudaError_t e = cudaSuccess;
+  if (mem_kind == RT_MEM_HOST) {
+    CUDA_TRY(cudaMallocAsync((void**)&tmp, 2 * nb, st));
+    e = cudaMemcpyAsync(tmp, kph, nb, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(tmp + nb, gamma, nb, cudaMemcpyHostToDevice, st);
+    kph = tmp;
+    gamma = tmp + nb;
   }
+  if (g->precision == RT_FP32_MIXED) {
+    if (e == cudaSuccess) e = launch_write_rates(n, kph, gamma, dtype, g->K, 1.0 / gamma_scale(g), st);
+    if (e == cudaSuccess) g_launches.fetch_add(1);
+  } else {
+    if (e == cudaSuccess) e = launch_convert(n, kph, dtype, g->K, st);
+    if (e == cudaSuccess) e = launch_convert(n, gamma, dtype, g->G, st);
+    if (e == cudaSuccess) g_launches.fetch_add(2);
+  }
+  if (tmp) cudaFreeAsync(tmp, st);
+  if (e != cudaSuccess) return fail(RT_ERR_CUDA, "rt_set_rates: %s", cudaGetErrorString(e));
   if (mem_kind == RT_MEM_HOST) CUDA_TRY(cudaStreamSynchronize(st));
   return RT_OK;
 }
@@ -1460,8 +1455,7 @@ int rt_get_ionised(rt_grid* g, void* x_HII, int dtype, int mem_kind) {
   if (dtype != RT_DTYPE_F64 && dtype != RT_DTYPE_F32) return fail(RT_ERR_INVALID_ARG, "rt_get_ionised: dtype %d", dtype);
   if (mem_kind != RT_MEM_HOST && mem_kind != RT_MEM_DEVICE) return fail(RT_ERR_INVALID_ARG, "rt_get_ionised: mem_kind %d", mem_kind);
   CUDA_TRY(cudaSetDevice(g->ctx->device));
-  int rc = copy_field(g, g->xHII, RT_DTYPE_F64, x_HII, dtype, mem_kind);
-  if (rc) return rc;
+  if (int rc = read_fields(g, nullptr, nullptr, g->xHII, nullptr, nullptr, x_HII, dtype, mem_kind)) return rc;
   CUDA_TRY(cudaStreamSynchronize(g->stream));
   return RT_OK;
 }
@@ -1644,7 +1638,7 @@ static int batch_enqueue(rt_batch* b, const rt_trace_params* p, int passes) {
     if ((rc = ensure_dir_table(b->ctx, want, &A.dir_tab, &A.dir_levels))) return rc;
   }
   int per_sm = 0;
-  CUDA_TRY(trace_occupancy(b->precision, 0, b->variant, 256, &per_sm));
+  CUDA_TRY(trace_occupancy(b->precision, 0, A.fc, b->variant, 256, &per_sm));
   if (per_sm < 1) per_sm = 1;
   if (p->blocks_per_sm > 0 && p->blocks_per_sm < per_sm) per_sm = p->blocks_per_sm;
   if ((rc = b->ts.bind_rows(A, per_sm * b->ctx->num_sms, ninst))) return rc;
@@ -1986,7 +1980,7 @@ int rt_batch_autotune(rt_batch* b, rt_trace_params* p) {
   if ((rc = rt_batch_trace(b, &q, 1))) return rc;  // sizes the queue, warms up
   const int spi[] = {4, 8, 16, 32, 64};
   int per_sm_max = 0;
-  CUDA_TRY(trace_occupancy(b->precision, 0, b->variant, 256, &per_sm_max));
+  CUDA_TRY(trace_occupancy(b->precision, 0, (p->flags & RT_TRACE_FC) != 0, b->variant, 256, &per_sm_max));
   float best = 1e30f;
   rt_trace_params bestp = q;
   for (int bps = 1; bps <= (per_sm_max > 0 ? per_sm_max : 1); ++bps) {

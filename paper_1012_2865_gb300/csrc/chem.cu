@@ -130,13 +130,13 @@ __global__ void chem_kernel(long long ncell, const double* __restrict__ nH, doub
 // (f2.cuh), since the FP64 pipe, a small fraction of the FP32 one, otherwise
 // bounds the kernel.
 __global__ void chem_mixed_kernel(long long ncell, const double* __restrict__ nH, double* __restrict__ xHI,
-                                  double* __restrict__ xHII, const float* __restrict__ K,
+                                  double* __restrict__ xHII, const float2* __restrict__ K,
                                   float2* __restrict__ nhi, float4 hh, int nsub) {
   const F2 ha = {hh.x, hh.y}, h2 = {hh.z, hh.w};
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < ncell;
        c += (long long)gridDim.x * blockDim.x) {
     double x = xHI[c], z = xHII[c];
-    const float kc = K[c];
+    const float kc = K[c].x;
     if (kc == 0.0f && is_neutral(x, z)) continue;
     const F2 nx = chem_cell_mixed(x, z, nH[c], kc, ha, h2, nsub);
     xHI[c] = x;
@@ -181,11 +181,50 @@ __global__ void check_density_kernel(long long n, const double* __restrict__ a, 
   }
 }
 
-template <typename ST, typename DT>
-__global__ void convert_kernel(long long n, const ST* __restrict__ src, DT* __restrict__ dst, double scale) {
+template <typename ST>
+__global__ void convert_kernel(long long n, const ST* __restrict__ src, double* __restrict__ dst) {
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n;
        c += (long long)gridDim.x * blockDim.x)
-    dst[c] = scale == 1.0 ? (DT)src[c] : (DT)((double)src[c] * scale);
+    dst[c] = (double)src[c];
+}
+
+// Gamma of an FP32-mixed grid, eV/s, in erg/s as FP32: the product with scale
+// as an FP32 pair, rounded (the FP64 pipe is a small fraction of the FP32 one);
+// results near or below the FP32 normal range through FP64.
+__device__ __forceinline__ float scale32(float v, double scale, float sh, float sl) {
+  const float p = __fmul_rn(v, sh);
+  if (fabsf(p) < 1e-30f) return v == 0.0f ? 0.0f : (float)((double)v * scale);
+  return __fadd_rn(p, fmaf(v, sl, fmaf(v, sh, -p)));
+}
+// k_ph, Gamma (times scale) and x_HI for the caller, each where its output is
+// given.  MIXED: kg holds (k_ph, Gamma) pairs, else K and G are FP64 arrays.
+template <bool MIXED, typename DT>
+__global__ void read_rates_kernel(long long n, const void* __restrict__ K, const double* __restrict__ G,
+                                  const double* __restrict__ x, DT* __restrict__ ok, DT* __restrict__ og,
+                                  DT* __restrict__ ox, double scale) {
+  const float sh = (float)scale, sl = (float)(scale - (double)sh);
+  for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n;
+       c += (long long)gridDim.x * blockDim.x) {
+    if (MIXED) {
+      if (ok || og) {
+        const float2 v = ((const float2*)K)[c];
+        if (ok) ok[c] = (DT)v.x;
+        if (og) og[c] = sizeof(DT) == 4 ? (DT)scale32(v.y, scale, sh, sl) : (DT)((double)v.y * scale);
+      }
+    } else {
+      if (ok) ok[c] = (DT)((const double*)K)[c];
+      if (og) og[c] = (DT)(scale == 1.0 ? G[c] : G[c] * scale);
+    }
+    if (ox) ox[c] = (DT)x[c];
+  }
+}
+// The caller's k_ph and Gamma (times scale) into an FP32-mixed grid.
+template <typename ST>
+__global__ void write_rates_kernel(long long n, const ST* __restrict__ k, const ST* __restrict__ g,
+                                   float2* __restrict__ kg, double scale) {
+  for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n;
+       c += (long long)gridDim.x * blockDim.x)
+    kg[c] = make_float2((float)k[c], (float)((double)g[c] * scale));
 }
 
 __global__ void complement_kernel(long long n, const double* __restrict__ x, double* __restrict__ out) {
@@ -382,12 +421,12 @@ __global__ void check_refresh_kernel(long long n, unsigned long long* __restrict
 // dt_max when dt_max is finite (so cells outside the front hold exactly 1).
 template <typename KT>
 __global__ void cell_timestep_kernel(long long n, const double* __restrict__ nH, const double* __restrict__ xHI,
-                                     const KT* __restrict__ K, double sdx, double tau_front, float eps, float alpha,
+                                     const KT* __restrict__ K, int kstride, double sdx, double tau_front, float eps, float alpha,
                                      float dt_max, float unit, float* __restrict__ dtc) {
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n; c += (long long)gridDim.x * blockDim.x) {
     const double nh64 = nH[c], x64 = xHI[c];
     const float nh = (float)nh64, x = (float)x64;
-    const float rate = fabsf((float)K[c] + nh * (1.0f - x) * alpha);
+    const float rate = fabsf((float)K[c * kstride] + nh * (1.0f - x) * alpha);
     float dt = dt_max;
     if (sdx * nh64 * x64 > tau_front && rate > 0.0f) dt = fminf(dt_max, eps / rate);
     dtc[c] = dt == dt_max ? dt_max / unit : dt / unit;
@@ -434,10 +473,10 @@ cudaError_t launch_timestep(long long n, int nx, int ny, int nz, const double* n
   if (g > 152 * 8) g = 152 * 8;
   if (g < 1) g = 1;
   if (fp64_rates)
-    cell_timestep_kernel<double><<<(int)g, block, 0, st>>>(n, nH, xHI, (const double*)K, sdx, tau_front, eps, alpha,
+    cell_timestep_kernel<double><<<(int)g, block, 0, st>>>(n, nH, xHI, (const double*)K, 1, sdx, tau_front, eps, alpha,
                                                           dt_max, unit, dtc);
   else
-    cell_timestep_kernel<float><<<(int)g, block, 0, st>>>(n, nH, xHI, (const float*)K, sdx, tau_front, eps, alpha,
+    cell_timestep_kernel<float><<<(int)g, block, 0, st>>>(n, nH, xHI, (const float*)K, 2, sdx, tau_front, eps, alpha,
                                                          dt_max, unit, dtc);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
@@ -466,7 +505,7 @@ cudaError_t launch_chem(int precision, long long ncell, const double* nH, double
     chem_kernel<double, double><<<grid, block, 0, st>>>(ncell, nH, xHI, xHII, (const double*)K,
                                                          (double*)nhi, h, nsub, alpha);
   else
-    chem_mixed_kernel<<<grid, block, 0, st>>>(ncell, nH, xHI, xHII, (const float*)K, (float2*)nhi,
+    chem_mixed_kernel<<<grid, block, 0, st>>>(ncell, nH, xHI, xHII, (const float2*)K, (float2*)nhi,
                                               step_pairs(h, alpha), nsub);
   return cudaGetLastError();
 }
@@ -493,21 +532,20 @@ cudaError_t launch_check_density(long long n, const double* a, unsigned long lon
   return cudaGetLastError();
 }
 
-// Adds delta to one device word (the trace self-test's phantom package).
-// Step 2 of a trace in one launch: k_ph and Gamma (two arrays of nbytes
-// each, 16-byte aligned) and the budget words (acc, cnt) to zero.
+// Step 2 of a trace in one launch: the rate arrays (nbytes each, 16-byte
+// aligned; b may be null) and the budget words (acc, cnt) to zero.
 __global__ void zero_fields_kernel(uint4* __restrict__ a, uint4* __restrict__ b, size_t n16, size_t nbytes,
                                    unsigned long long* __restrict__ acc, int nacc, unsigned long long* __restrict__ cnt,
                                    int ncnt) {
   const uint4 z = make_uint4(0u, 0u, 0u, 0u);
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n16; i += (size_t)gridDim.x * blockDim.x) {
     a[i] = z;
-    b[i] = z;
+    if (b) b[i] = z;
   }
   if (blockIdx.x == 0) {
     for (size_t t = 16 * n16 + threadIdx.x; t < nbytes; t += blockDim.x) {
       ((unsigned char*)a)[t] = 0;
-      ((unsigned char*)b)[t] = 0;
+      if (b) ((unsigned char*)b)[t] = 0;
     }
     for (int t = threadIdx.x; t < nacc; t += blockDim.x) acc[t] = 0ULL;
     for (int t = threadIdx.x; t < ncnt; t += blockDim.x) cnt[t] = 0ULL;
@@ -526,6 +564,7 @@ cudaError_t launch_zero_fields(void* a, void* b, size_t nbytes, void* acc, int n
   return cudaGetLastError();
 }
 
+// Adds delta to one device word (the trace self-test's phantom package).
 __global__ void add_word_kernel(unsigned long long* w, unsigned long long delta) {
   if (threadIdx.x == 0 && blockIdx.x == 0) *w += delta;
 }
@@ -595,29 +634,30 @@ cudaError_t launch_complement(long long n, const double* x, double* out, cudaStr
 // grid (its descriptor in `inst`), blocks of a row stride over its cells.
 // ---------------------------------------------------------------------------
 
-// Step 2 for every grid: zero k_ph, Gamma (element size esz), the budget
-// sums and the counters.
+// Step 2 for every grid: zero the rates (esz bytes of k_ph and of Gamma per
+// cell, together in one array where G is null), the budget sums and the
+// counters.
+__device__ __forceinline__ void zero_rates(void* K, void* G, size_t bytes) {
+  const uint4 z = make_uint4(0u, 0u, 0u, 0u);
+  uint4* const a = (uint4*)K;
+  uint4* const b = (uint4*)G;
+  const size_t n16 = bytes / 16;
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n16; i += (size_t)gridDim.x * blockDim.x) {
+    a[i] = z;
+    if (b) b[i] = z;
+  }
+  if (blockIdx.x == 0)
+    for (size_t t = 16 * n16 + 4 * threadIdx.x; t < bytes; t += 4 * blockDim.x) {
+      *(unsigned int*)((char*)K + t) = 0u;
+      if (G) *(unsigned int*)((char*)G + t) = 0u;
+    }
+}
 __global__ void batch_zero_kernel(const InstDev* __restrict__ inst, int esz) {
   const InstDev I = inst[blockIdx.y];
-  const long long n = (long long)I.nx * I.ny * I.nz;
-  const long long words = n * esz / 4;
-  unsigned int* K = (unsigned int*)I.K;
-  unsigned int* G = (unsigned int*)I.G;
-  for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < words;
-       c += (long long)gridDim.x * blockDim.x) {
-    K[c] = 0u;
-    G[c] = 0u;
-  }
-  for (int t = 0; t < 2; ++t) {  // helium photon types, where the grid has them
-    if (!I.Khe[t]) continue;
-    unsigned int* Kt = (unsigned int*)I.Khe[t];
-    unsigned int* Gt = (unsigned int*)I.Ghe[t];
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < words;
-         c += (long long)gridDim.x * blockDim.x) {
-      Kt[c] = 0u;
-      Gt[c] = 0u;
-    }
-  }
+  const size_t bytes = (size_t)I.nx * I.ny * I.nz * esz;
+  zero_rates(I.K, I.G, I.G ? bytes : 2 * bytes);
+  for (int t = 0; t < 2; ++t)  // helium photon types, where the grid has them
+    if (I.Khe[t]) zero_rates(I.Khe[t], I.Ghe[t], I.Ghe[t] ? bytes : 2 * bytes);
   if (blockIdx.x == 0) {
     for (int i = threadIdx.x; i < 8; i += blockDim.x) I.acc[i] = 0.0;
     for (int i = threadIdx.x; i < kCntWords; i += blockDim.x) I.cnt[i] = 0ULL;
@@ -633,7 +673,7 @@ __global__ void batch_chem_kernel(const InstDev* __restrict__ inst, double h, in
        c += (long long)gridDim.x * blockDim.x) {
     double x = I.xHI[c], z = I.xHII[c];
     if (MIXED) {
-      const float kc = ((const float*)I.K)[c];
+      const float kc = ((const float2*)I.K)[c].x;
       if (kc == 0.0f && is_neutral(x, z)) continue;
       const F2 nx = chem_cell_mixed(x, z, I.nH[c], kc, ha, h2, nsub);
       ((double*)I.xHI)[c] = x;
@@ -681,19 +721,42 @@ cudaError_t launch_batch_chem(const InstDev* inst, int ninst, int precision, lon
   return cudaGetLastError();
 }
 
-// src_dtype / dst_dtype: RT_DTYPE_F64 or RT_DTYPE_F32; dst = src * scale
-// (the product in FP64)
-cudaError_t launch_convert(long long n, const void* src, int src_dtype, void* dst, int dst_dtype,
-                           cudaStream_t st, double scale) {
+// Outputs of element type dtype; null ones are left out.
+cudaError_t launch_read_rates(int precision, long long n, const void* K, const void* G, const double* x, void* ok,
+                              void* og, void* ox, int dtype, double scale, cudaStream_t st) {
   const int block = 256, grid = grid_for(n, block);
-  if (src_dtype == RT_DTYPE_F64 && dst_dtype == RT_DTYPE_F64)
-    convert_kernel<double, double><<<grid, block, 0, st>>>(n, (const double*)src, (double*)dst, scale);
-  else if (src_dtype == RT_DTYPE_F64 && dst_dtype == RT_DTYPE_F32)
-    convert_kernel<double, float><<<grid, block, 0, st>>>(n, (const double*)src, (float*)dst, scale);
-  else if (src_dtype == RT_DTYPE_F32 && dst_dtype == RT_DTYPE_F64)
-    convert_kernel<float, double><<<grid, block, 0, st>>>(n, (const float*)src, (double*)dst, scale);
+  const double* g = (const double*)G;
+  if (precision == RT_FP64) {
+    if (dtype == RT_DTYPE_F64)
+      read_rates_kernel<false, double><<<grid, block, 0, st>>>(n, K, g, x, (double*)ok, (double*)og, (double*)ox, scale);
+    else
+      read_rates_kernel<false, float><<<grid, block, 0, st>>>(n, K, g, x, (float*)ok, (float*)og, (float*)ox, scale);
+  } else {
+    if (dtype == RT_DTYPE_F64)
+      read_rates_kernel<true, double><<<grid, block, 0, st>>>(n, K, g, x, (double*)ok, (double*)og, (double*)ox, scale);
+    else
+      read_rates_kernel<true, float><<<grid, block, 0, st>>>(n, K, g, x, (float*)ok, (float*)og, (float*)ox, scale);
+  }
+  return cudaGetLastError();
+}
+
+cudaError_t launch_write_rates(long long n, const void* k, const void* g, int dtype, void* kg, double scale,
+                               cudaStream_t st) {
+  const int block = 256, grid = grid_for(n, block);
+  if (dtype == RT_DTYPE_F64)
+    write_rates_kernel<double><<<grid, block, 0, st>>>(n, (const double*)k, (const double*)g, (float2*)kg, scale);
   else
-    convert_kernel<float, float><<<grid, block, 0, st>>>(n, (const float*)src, (float*)dst, scale);
+    write_rates_kernel<float><<<grid, block, 0, st>>>(n, (const float*)k, (const float*)g, (float2*)kg, scale);
+  return cudaGetLastError();
+}
+
+// src of element type src_dtype into an FP64 array
+cudaError_t launch_convert(long long n, const void* src, int src_dtype, void* dst, cudaStream_t st) {
+  const int block = 256, grid = grid_for(n, block);
+  if (src_dtype == RT_DTYPE_F64)
+    convert_kernel<double><<<grid, block, 0, st>>>(n, (const double*)src, (double*)dst);
+  else
+    convert_kernel<float><<<grid, block, 0, st>>>(n, (const float*)src, (double*)dst);
   return cudaGetLastError();
 }
 

@@ -33,7 +33,7 @@ namespace rtg {
 cudaError_t launch_trace_init(unsigned long long* ctl, void* queue, size_t queue_bytes, unsigned long long n_roots,
                               int first_pass, int mode, unsigned long long in_cap, int pass, int passes,
                               cudaStream_t st);
-cudaError_t trace_occupancy(int precision, int fsl, int variant, int block, int* blocks_per_sm);
+cudaError_t trace_occupancy(int precision, int fsl, int fc, int variant, int block, int* blocks_per_sm);
 cudaError_t launch_trace(int precision, int fsl, int variant, const TraceArgs& A, int grid, int block,
                          cudaStream_t st);
 cudaError_t launch_direction_table(int level, float4* tab, cudaStream_t st);
@@ -242,7 +242,7 @@ int rt_trace_noalloc(const rt_noalloc_grid* g, int nsrc, const double* pos_cm, c
       A.theta32[l] = (float)A.theta[l];
     }
     int per_sm = 0;
-    if ((e = trace_occupancy(RT_FP32_MIXED, 0, WALK_ANY_PLAIN, 256, &per_sm)) != cudaSuccess) return na_fail(RT_ERR_CUDA, "occupancy", e);
+    if ((e = trace_occupancy(RT_FP32_MIXED, 0, A.fc, WALK_ANY_PLAIN, 256, &per_sm)) != cudaSuccess) return na_fail(RT_ERR_CUDA, "occupancy", e);
     if (per_sm < 1) per_sm = 1;
     if (p->blocks_per_sm > 0 && p->blocks_per_sm < per_sm) per_sm = p->blocks_per_sm;
     if (per_sm * sms > kNaMaxBlocks) return na_fail(RT_ERR_INVALID_ARG, "more trace blocks than the budget rows hold");

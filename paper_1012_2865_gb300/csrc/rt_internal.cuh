@@ -112,21 +112,18 @@ inline void fill_position32(SourceDev& S, int nx, int ny, int nz, double p0) {
 // source, and any source with n_HI as plain FP32 instead of pairs.
 enum WalkVariant { WALK_EXACT = 0, WALK_ANY = 1, WALK_ANY_PLAIN = 2 };
 
-// InstDev.flags: the FP32-mixed grid stores n_HI as float2 pairs (n_HI
-// rounded to FP32, and the remainder), so the walker sums optical depth to
-// ~2^-44 of the FP64 evaluation.
-constexpr int kInstNhiPair = 1;
-
-// One grid (instance) as the trace kernel sees it.
+// One grid (instance) as the trace kernel sees it.  An FP32-mixed grid stores
+// n_HI as float2 pairs (n_HI rounded to FP32, and the remainder), so the
+// walker sums optical depth to ~2^-44 of the FP64 evaluation, and k_ph and
+// Gamma interleaved (float2 per cell) in K, with G null.
 struct InstDev {
   int nx, ny, nz;
-  int flags;                // kInstNhiPair: nhi holds (hi, lo) FP32 pairs
   const void* nhi;          // absorber density n_HI (double, float or float2), x fastest
   const double* nH;         // hydrogen density, FP64 (decisions re-taken in FP64)
   const double* xHI;        // neutral fraction, FP64
   double* xHII;             // ionised fraction, FP64 (chemistry)
-  void* K;                  // k_ph accumulator (double or float)
-  void* G;                  // Gamma accumulator (double or float)
+  void* K;                  // k_ph accumulator (double, float2 with Gamma, or float)
+  void* G;                  // Gamma accumulator (double or float; null where K holds it)
   double* acc;              // [0] emitted [1] absorbed [2] escaped [3] resumed [4] halted (photons/s)
   unsigned long long* cnt;  // [0,15) counts, [15,30) hashes, [30] segments, [31], [32] fallbacks
   // helium photon types 1, 2 (null until the grid has helium absorbers):
@@ -285,6 +282,10 @@ __device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long
 // in an ionised 128^3 grid 15.4 -> 13.4 ms, a 24-grid batch 4.38 -> 3.82 ms.
 __device__ __forceinline__ void red_add(float* p, float v) {
   asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" ::"l"(__cvta_generic_to_global(p)), "f"(v));
+}
+// two neighbouring words (8-byte aligned)
+__device__ __forceinline__ void red_add2(float* p, float a, float b) {
+  asm volatile("red.relaxed.gpu.global.add.v2.f32 [%0], {%1, %2};" ::"l"(__cvta_generic_to_global(p)), "f"(a), "f"(b));
 }
 __device__ __forceinline__ void red_add(double* p, double v) {
   asm volatile("red.relaxed.gpu.global.add.f64 [%0], %1;" ::"l"(__cvta_generic_to_global(p)), "d"(v));

@@ -51,7 +51,10 @@ constexpr int kShInst = 64;  // grids whose level counters and fallback counts a
 static_assert(kBlkGrids <= kShInst, "a grid with a budget row has its counters in shared memory");
 constexpr int kBlock = 256;  // threads per block of the trace kernel
 
-enum Event { EV_NONE = 0, EV_SPLIT = 1, EV_DONE = 2, EV_HALT = 3 };
+// What ends a lane's part of a queue visit.  EV_RARE: the next segment needs
+// the full decision; EV_TERM: the optical depth is at or near the termination
+// (the FP32 walker leaves both to a stage after the visit's segments).
+enum Event { EV_NONE = 0, EV_SPLIT, EV_DONE, EV_HALT, EV_RARE, EV_TERM };
 enum Start { NO_START = 0, START_CHILD, START_ROOT, START_RESUMED };
 constexpr int kAcc = 5;  // budget sums per grid: emitted, absorbed, escaped, resumed, halted
 
@@ -81,13 +84,17 @@ struct LaneAcc {
   unsigned long long segments;
   unsigned int fallbacks, fallbacks_tau;
   int inst;
-  // of the lane's package (FP32 walker): P, optical depth and its error bound
-  // at the start; read only when the package ends, so kept out of registers
-  float Pstart, tau0, tau_err;
-  // 72 bytes = 18 banks: the 8-byte accesses of a half-warp to one field
+  // of the lane's package (FP32 walker), read only between queue visits and so
+  // kept out of registers: P, optical depth and its error bound at the start,
+  // the radius of the next full decision, segments so far, and the planes
+  // that a segment left at EV_TERM crosses
+  float Pstart, tau0, tau_err, lim;
+  int steps, mask;
+  float cover;  // covering factor of the last segment (where traced with one)
+  // 88 bytes = 22 banks: the 8-byte accesses of a half-warp to one field
   // fall on 16 different bank pairs (a 64-byte stride puts them on two)
 };
-static_assert(sizeof(LaneAcc) == 72, "conflict-free stride of the per-lane sums");
+static_assert(sizeof(LaneAcc) == 88, "conflict-free stride of the per-lane sums");
 
 // A block's budget sums per grid for the first kBlkGrids grids of the
 // launch: its rows of TraceArgs.blk (global memory, kBlkRow words per grid)
@@ -151,6 +158,14 @@ __device__ __forceinline__ void acc_switch(LaneAcc& a, unsigned& nseg, int inst,
     a.inst = inst;
   }
 }
+
+// A warp's state while it has nothing to trace: the outstanding count last
+// seen, when it was first seen, and how long to sleep (ns; doubles up to 4 us).
+struct IdleWarp {
+  long long seen_out;
+  uint64_t seen_ns;
+  unsigned backoff;
+};
 
 struct LevelCounters {
   unsigned int* cnt;        // [kShInst][kLevels]
@@ -385,9 +400,8 @@ struct Walk64 {
     }
     return EV_NONE;
   }
-  __device__ __forceinline__ void seal(const TraceArgs&, const LaneAcc&) {}
+  static constexpr bool kStaged = false;
   __device__ __forceinline__ void begin_visit() {}
-  __device__ __forceinline__ int end_visit(const TraceArgs&, LaneAcc&, int, int ev) { return ev; }
   // Budget of the parent's run when it splits (children carry P/4 each).
   __device__ __forceinline__ void on_split(const TraceArgs& A, LaneAcc& acc) const {
     acc.absorbed += (Pstart - P) * unit(A);
@@ -477,6 +491,22 @@ constexpr float kEps32 = 5.9604645e-8f;   // 2^-24
 constexpr float kBandT = 9.094947e-13f;   // 2^-40
 constexpr float kNear = 9.53674316e-7f;   // 2^-20: high parts farther apart are ordered
 
+// Direction of a pixel of a level beyond the table, from the FP64 evaluation
+// (out of line: its FP64 registers would otherwise press on every start).
+struct DirPair {
+  F2 n0, n1, n2;
+  int diag;
+};
+__device__ __noinline__ DirPair dir_pair64(int level, uint32_t pix) {
+  double v[3];
+  DirPair d;
+  d.diag = pix2vec64(level, pix, v);
+  d.n0 = f2_from_double(v[0]);
+  d.n1 = f2_from_double(v[1]);
+  d.n2 = f2_from_double(v[2]);
+  return d;
+}
+
 // Direction of (level, pix) as FP32 pairs: from the device table when the
 // level is tabulated, else from the FP64 evaluation.  Returns the
 // 45-degree-meridian flag.
@@ -490,13 +520,11 @@ __device__ __forceinline__ int dir_pair(const TraceArgs& A, int level, uint32_t 
     n[2] = {h.z, l.z};
     return h.w != 0.0f;
   }
-  double v[3];
-  const int diag = pix2vec64(level, pix, v);
-  for (int i = 0; i < 3; ++i) {
-    const float hi = (float)v[i];
-    n[i] = {hi, (float)(v[i] - (double)hi)};
-  }
-  return diag;
+  const DirPair d = dir_pair64(level, pix);
+  n[0] = d.n0;
+  n[1] = d.n1;
+  n[2] = d.n2;
+  return d.diag;
 }
 
 // Exact (FP64) crossing decision for cell (c0, c1, c2) of package (level,
@@ -591,9 +619,16 @@ struct Axis {
 };
 
 // EXACT: every source of the launch lies on the 1/16-cell lattice.  PAIR:
-// n_HI is stored as FP32 pairs.
-template <bool EXACT, bool PAIR>
+// n_HI is stored as FP32 pairs, and k_ph and Gamma side by side, so that a
+// heating segment deposits both with one two-word reduction.  L2 takes those
+// at the rate of single ones (200 G/s into 16 MB; two single ones 102 G/s):
+// 24 sources in an ionised 128^3 grid 9.27 -> 8.45 ms, 30 of three photon types
+// in 128^3 4.23 -> 3.89 ms, 1000 in a clumpy 256^3 grid 3.01 -> 2.92 ms.
+// FC: deposits are scaled by the covering factor (its own instantiation,
+// because its cell centres cost the segment loop 12 registers).
+template <bool EXACT, bool PAIR, bool FC>
 struct Walk32 {
+  static constexpr bool kStaged = true;  // step() leaves rare decisions to slow() and terminate()
   using Rec = Rec32;  // packages in flight between traces; records of FSL traces
   template <bool FSL> using Q = typename std::conditional<FSL, Rec32, QRec32>::type;  // queue record
   uint32_t src, pix;
@@ -605,15 +640,15 @@ struct Walk32 {
   float tau_err;        // error bound of tau (in records and while a package starts or ends)
   Axis<EXACT> a0, a1, a2;
   int idx;              // cell index
-  int steps;            // segments of the package in earlier queue visits
+  int cnt;              // segments of the package in this queue visit
   unsigned nseg;
   float nh, nh_lo;      // n_HI of the current cell (pair), loaded one step ahead
   float lim;            // below it no crossing splits, leaves the box or halts
   float sk, q;          // sum of kappa over the package's segments; error of tau per unit of it
   float sdx, sdx_lo, w, heat;
   const float* nhi;
-  float* K;
-  float* G;
+  float* K;             // PAIR: (k_ph, Gamma) per cell
+  float* G;             // else
 
   __device__ __forceinline__ int lvl() const { return (int)(level & 15u); }
   __device__ __forceinline__ bool diag_exact() const { return (level & 256u) != 0; }
@@ -655,7 +690,8 @@ struct Walk32 {
     acc.Pstart = P;
     acc.tau0 = tau;
     acc.tau_err = tau_err;
-    steps = 0;
+    acc.steps = 0;
+    cnt = 0;
     sk = 0.0f;
     F2 n[3];
     const int diag = dir_pair(A, lvl(), pix, n);
@@ -687,7 +723,7 @@ struct Walk32 {
       a2.init(c2, n[2], sh.z, S.sa[2], F2{bh.z, bl.z}, nx * ny);
     }
     K = (float*)(t == 0 ? I.K : I.Khe[t - 1]);
-    G = (float*)(t == 0 ? I.G : I.Ghe[t - 1]);
+    if (!PAIR) G = (float*)I.G;
     const float4 k32 = __ldg(&S.k32);  // sdx, w, rw, heat
     sdx = k32.x; sdx_lo = sl.w; w = k32.y; heat = k32.w;
     // Radii before and after which the next crossing cannot / must need the
@@ -704,7 +740,8 @@ struct Walk32 {
       hi = fminf(hi, A.rsplit32[l]);
     }
     if (FSL) lo = fminf(lo, rlim.hi);
-    lim = fmaf(lo, -kNear, lo);
+    acc.lim = fmaf(lo, -kNear, lo);
+    lim = r.hi == 0.0f ? 0.0f : acc.lim;  // segments from the source itself: slow(), with deposit_first()
     const float4 sa = __ldg(&S.sabs32);
     q = fmaf(hi, 4.1f * kBandT, 1e-30f) +
         4.1f * fmaxf(sa.x * a0.iv.hi, fmaxf(sa.y * a1.iv.hi, sa.z * a2.iv.hi));
@@ -745,7 +782,7 @@ struct Walk32 {
     const float e_dtau = PAIR ? 8.0f * kBandT : 4.0f * kEps32;
     const float spi = (float)A.segs_per_iter;
     return acc.tau_err + fmaf(tau, kEps32, tau - acc.tau0) * e_dtau + sk * (fmaf(rmax, 4.0f * kBandT, 1e-30f) + 4.0f * ab) +
-           ((float)steps + spi) * tau * (kBandT / 16.0f + spi * (kEps32 * kEps32));
+           (float)(acc.steps + cnt) * tau * (kBandT / 16.0f + spi * (kEps32 * kEps32));
   }
   // The package's radius and optical depth as normalised pairs with the error
   // bound, for its children or the store of packages in flight.
@@ -895,62 +932,19 @@ struct Walk32 {
     return (m0 ? 1 : 0) | (m1 ? 2 : 0) | (m2 ? 4 : 0) | (split ? 8 : 0) | (halt ? 64 : 0) | (out ? 128 : 0);
   }
 
-  // tau is at or near the termination: whether the package ends here (Step 3i).
-  template <bool FSL>
-  __device__ __forceinline__ bool terminates(const TraceArgs& A, LaneAcc& acc, float rn, bool halt) const {
-    const float d = f2_diff(F2{tau, tau_lo}, F2{A.tau_term32, A.tau_term32lo});
-    const float bnd = tau_bound(A, acc, rn) + tau * (4.0f * kBandT) + 1e-30f;
-    if (d > bnd) return true;
-    if (-d > bnd) return false;
-    // too close to call: the lineage's optical depth in FP64 (a lineage
-    // emitted in an earlier trace crossed other media, and a cut segment
-    // is not the cell's: there the pair's own decision stands)
-    acc.fallbacks_tau++;
-    double t64 = __longlong_as_double(0x7ff8000000000000LL);
-    if (!FSL || (age == 0 && !halt)) {
-      const SourceDev& S = A.src[src];
-      const float4 sh = __ldg(&S.s32);
-      t64 = retrace_tau64(A, src, lvl(), pix, a0.cell(sh.x, S.sa[0]), a1.cell(sh.y, S.sa[1]), a2.cell(sh.z, S.sa[2]));
-    }
-    return isnan(t64) ? (d > 0.0f) : (t64 > A.tau_term);
-  }
-
-  // One segment.  Returns EV_SPLIT before traversing a cell whose exit radius
-  // exceeds R_split, EV_DONE when the package is absorbed or leaves the box,
-  // EV_HALT (FSL) when it has travelled to its halting radius.
-  template <bool FSL>
-  __device__ __forceinline__ int step(const TraceArgs& A, LaneAcc& acc) {
-    // The next plane: the smallest high part, provably the nearest when no
-    // other is within 2^-20 of it (each is within 2^-22 of its distance).
-    F2 rn;
-    rn.hi = fminf(a0.t.hi, fminf(a1.t.hi, a2.t.hi));
-    const float close = fmaf(rn.hi, kNear, rn.hi);
-    bool m0 = a0.t.hi <= close, m1 = a1.t.hi <= close, m2 = a2.t.hi <= close;
-    rn.lo = m0 ? a0.t.lo : (m1 ? a1.t.lo : a2.t.lo);
-    const bool rare = rn.hi >= lim || (m0 && m1) || (m2 && (m0 || m1));
-    int m = 0;
-    if (rare) {
-      unsigned fb = 0;
-      m = decide<FSL>(A, rn, fb);
-      acc.fallbacks += fb;
-      if (m & 8) return EV_SPLIT;
-      m0 = (m & 1) != 0;
-      m1 = (m & 2) != 0;
-      m2 = (m & 4) != 0;
-    }
-    const bool halt = FSL && (m & 64);  // Step 3j: the segment ends at rlim
-    // segment length as a pair (both ends are pairs; |end| >= |r| or the
-    // difference of the high parts is exact)
-    const F2 end = halt ? rlim : rn;
+  // The segment from r to `end` in the current cell; returns its k_ph.
+  __device__ __forceinline__ float segment(const TraceArgs& A, LaneAcc& acc, F2 end) {
+    // length as a pair (both ends are pairs; |end| >= |r| or the difference of
+    // the high parts is exact)
     const float dh = __fsub_rn(end.hi, r.hi);
     const float dl = __fadd_rn(__fsub_rn(__fsub_rn(end.hi, dh), r.hi), __fsub_rn(end.lo, r.lo));
     float dr = __fadd_rn(dh, dl);
     float drl = __fadd_rn(__fsub_rn(dh, dr), dl);
-    if (dr > 0.0f) {
-      nseg++;
-    } else {
+    ++cnt;
+    if (!(dr > 0.0f)) {  // a start on a plane, a tie: no length, not counted
       dr = 0.0f;
       drl = 0.0f;
+      --nseg;
     }
     // kappa = sigma dx n_HI and dtau = kappa dr as pairs: the optical depth
     // follows the FP64 sum to ~2^-44 where n_HI is a pair
@@ -972,45 +966,95 @@ struct Walk32 {
     const float ser = fmaf(fmaf(fmaf(fmaf(fmaf(fmaf(dtau, 1.0f / 5040.0f, -1.0f / 720.0f), dtau, 1.0f / 120.0f), dtau,
                                           -1.0f / 24.0f), dtau, 1.0f / 6.0f), dtau, -0.5f), dtau, 1.0f);
     const float phi = dtau < 0.25f ? ser : __fdividef(1.0f - tr, dtau);
-    // covering factor (Eq. "fc"), in FP32 from the pairs' high parts: its
-    // error (~1e-4 relative) is far inside the tolerance on k_ph
     float fcv = 1.0f;
-    if (A.fc) {
-      const float rh = __fadd_rn(r.hi, r.lo);
-      const float L = rh * A.theta32[lvl()];
-      if (L > 0.0f) {
-        const float4 sh = __ldg(&A.src[src].s32);
-        const int* sa = A.src[src].sa;
-        const float rm = fmaf(0.5f, dr, rh);
-        const float d = fmaxf(a0.off_middle(rm, sh.x, sa[0]), fmaxf(a1.off_middle(rm, sh.y, sa[1]), a2.off_middle(rm, sh.z, sa[2])));
-        const float f = 0.5f + (0.5f - d) / L;
-        fcv = fminf(1.0f, f * f);
-      }
+    if (FC) {
+      fcv = cover(A, dr);
+      acc.cover = fcv;
     }
-    const float kadd = P * w * dr * phi * fcv;
-    red_add(&K[idx], kadd);
-    if (heat != 0.0f) red_add(&G[idx], kadd * heat);
+    const float k = P * w * dr * phi * fcv;
     P = P * tr;
-    {
-      // the larger summand first: the sum's rounding error is exact
-      const float s = __fadd_rn(tau, dtau);
-      const float e = __fsub_rn(fminf(tau, dtau), __fsub_rn(s, fmaxf(tau, dtau)));
-      tau_lo = __fadd_rn(tau_lo, __fadd_rn(e, dtl));
-      tau = s;
-    }
+    // the larger summand first: the sum's rounding error is exact
+    const float s = __fadd_rn(tau, dtau);
+    const float e = __fsub_rn(fminf(tau, dtau), __fsub_rn(s, fmaxf(tau, dtau)));
+    tau_lo = __fadd_rn(tau_lo, __fadd_rn(e, dtl));
+    tau = s;
     sk += kap;
+    return k;
+  }
+  // covering factor (Eq. "fc") of a segment of length dr, in FP32 from the
+  // pairs' high parts: its error (~1e-4 relative) is far inside the tolerance
+  // on k_ph
+  __device__ __forceinline__ float cover(const TraceArgs& A, float dr) const {
+    const float rh = __fadd_rn(r.hi, r.lo);
+    const float L = rh * A.theta32[lvl()];
+    if (!(L > 0.0f)) return 1.0f;
+    const float4 sh = __ldg(&A.src[src].s32);
+    const int* sa = A.src[src].sa;
+    const float rm = fmaf(0.5f, dr, rh);
+    const float d = fmaxf(a0.off_middle(rm, sh.x, sa[0]), fmaxf(a1.off_middle(rm, sh.y, sa[1]), a2.off_middle(rm, sh.z, sa[2])));
+    const float f = 0.5f + (0.5f - d) / L;
+    return fminf(1.0f, f * f);
+  }
+  // Cross the planes m0, m1, m2 at rn; the next cell's density is loaded a
+  // step ahead.
+  __device__ __forceinline__ void advance(F2 rn, bool m0, bool m1, bool m2) {
+    r = rn;
+    if (m0) { a0.next(); idx += a0.stride; }
+    if (m1) { a1.next(); idx += a1.stride; }
+    if (m2) { a2.next(); idx += a2.stride; }
+    load_nh();
+  }
+
+  // One segment of the common case.  EV_RARE leaves the package before a
+  // segment that may split, leave the box or halt, or whose next plane is not
+  // provably the nearest; EV_TERM after one that may end it.
+  template <bool FSL>
+  __device__ __forceinline__ int step(const TraceArgs& A, LaneAcc& acc) {
+    // The next plane: the smallest high part, provably the nearest when no
+    // other is within 2^-20 of it (each is within 2^-22 of its distance).
+    F2 rn;
+    rn.hi = fminf(a0.t.hi, fminf(a1.t.hi, a2.t.hi));
+    const float close = fmaf(rn.hi, kNear, rn.hi);
+    const bool m0 = a0.t.hi <= close, m1 = a1.t.hi <= close, m2 = a2.t.hi <= close;
+    rn.lo = m0 ? a0.t.lo : (m1 ? a1.t.lo : a2.t.lo);
+    if (rn.hi >= lim || (m2 && (m0 || m1))) return EV_RARE;
+    // (the exact tie of a 45-degree ray crosses both planes)
+    if (m0 && m1 && !(diag_exact() && f2_eq(a0.t, a1.t))) return EV_RARE;
+    deposit(idx, segment(A, acc, rn));
     if (fmaf(sk, q, tau) > A.tau_near) {
-      if (terminates<FSL>(A, acc, rn.hi, halt)) {
-        if (nh > 0.0f) {
-          const float kres = P * __ldg(&A.src[src].k32.z) / nh * fcv;
-          red_add(&K[idx], kres);
-          if (heat != 0.0f) red_add(&G[idx], kres * heat);
-        }
-        acc.absorbed += (double)acc.Pstart * unit(A);
-        return EV_DONE;
-      }
+      r = rn;
+      acc.mask = (m0 ? 1 : 0) | (m1 ? 2 : 0) | (m2 ? 4 : 0);
+      return EV_TERM;
     }
-    if (halt) {
+    advance(rn, m0, m1, m2);
+    return EV_NONE;
+  }
+
+  // The segment that step() left at EV_RARE, with the full decision; its
+  // k_ph in dep.  EV_TERM as in step(), bits 6 and 7 of acc.mask as from decide().
+  template <bool FSL>
+  __device__ __forceinline__ int slow(const TraceArgs& A, LaneAcc& acc, float& dep) {
+    lim = acc.lim;
+    F2 rn;
+    unsigned fb = 0;
+    const int m = decide<FSL>(A, rn, fb);
+    acc.fallbacks += fb;
+    if (m & 8) return EV_SPLIT;
+    const bool halt = FSL && (m & 64);  // Step 3j: the segment ends at rlim
+    dep = segment(A, acc, halt ? rlim : rn);
+    acc.mask = m;
+    if (fmaf(sk, q, tau) > A.tau_near) {
+      r = rn;
+      return EV_TERM;
+    }
+    return pass<FSL>(A, acc, rn);
+  }
+  // Past a segment that did not end the package by its optical depth: halted,
+  // out of the box, or in the next cell.
+  template <bool FSL>
+  __device__ __forceinline__ int pass(const TraceArgs& A, LaneAcc& acc, F2 rn) {
+    const int m = acc.mask;
+    if (FSL && (m & 64)) {
       r = rlim;
       const double u = unit(A);
       acc.absorbed += ((double)acc.Pstart - (double)P) * u;
@@ -1021,33 +1065,88 @@ struct Walk32 {
       leave(A, acc);
       return EV_DONE;
     }
-    // cross the plane; the next cell's density is loaded a step ahead
-    r = rn;
-    if (m0) { a0.next(); idx += a0.stride; }
-    if (m1) { a1.next(); idx += a1.stride; }
-    if (m2) { a2.next(); idx += a2.stride; }
-    load_nh();
+    advance(rn, (m & 1) != 0, (m & 2) != 0, (m & 4) != 0);
     return EV_NONE;
+  }
+  // A segment left at EV_TERM: whether the package ends here (Step 3i), its
+  // residual then added to dep.
+  template <bool FSL>
+  __device__ __forceinline__ int terminate(const TraceArgs& A, LaneAcc& acc, float& dep) {
+    const bool halt = FSL && (acc.mask & 64);
+    const float d = f2_diff(F2{tau, tau_lo}, F2{A.tau_term32, A.tau_term32lo});
+    const float bnd = tau_bound(A, acc, r.hi) + tau * (4.0f * kBandT) + 1e-30f;
+    bool term = d > bnd;
+    if (!term && !(-d > bnd)) {
+      // too close to call: the lineage's optical depth in FP64 (a lineage
+      // emitted in an earlier trace crossed other media, and a cut segment
+      // is not the cell's: there the pair's own decision stands)
+      acc.fallbacks_tau++;
+      double t64 = __longlong_as_double(0x7ff8000000000000LL);
+      if (!FSL || (age == 0 && !halt)) {
+        const SourceDev& S = A.src[src];
+        const float4 sh = __ldg(&S.s32);
+        t64 = retrace_tau64(A, src, lvl(), pix, a0.cell(sh.x, S.sa[0]), a1.cell(sh.y, S.sa[1]), a2.cell(sh.z, S.sa[2]));
+      }
+      term = isnan(t64) ? (d > 0.0f) : (t64 > A.tau_term);
+    }
+    if (!term) return pass<FSL>(A, acc, r);
+    if (nh > 0.0f) dep += P * __ldg(&A.src[src].k32.z) / nh * (FC ? acc.cover : 1.0f);
+    acc.absorbed += (double)acc.Pstart * unit(A);
+    return EV_DONE;
+  }
+  // k into k_ph of cell `at`, k heat into its Gamma
+  __device__ __forceinline__ void deposit(int at, float k) const {
+    if (PAIR) {
+      float* const p = K + 2 * (size_t)(unsigned)at;
+      if (heat != 0.0f) red_add2(p, k, k * heat);
+      else red_add(p, k);
+    } else {
+      red_add(&K[at], k);
+      if (heat != 0.0f) red_add(&G[at], k * heat);
+    }
+  }
+  // The same for segments that start at the source itself (the lanes with
+  // `first`; every lane of the warp calls it).  The roots of a source land in
+  // one cell (those of a source on a cell face in a few), its brightest, with
+  // few distinct values whose FP32 sum rounds the same way again and again
+  // (up to 2.6e-6 of the cell's rate); the lanes' shares are added as a pair
+  // first, one reduction per cell and warp.
+  __device__ __forceinline__ void deposit_first(bool first, int at, float k) const {
+    const unsigned all = __ballot_sync(kFull, first);
+    const unsigned mine = __match_any_sync(kFull, src) & __match_any_sync(kFull, at) & all;
+    F2 s = {0.0f, 0.0f};
+    for (unsigned m = all; m; m &= m - 1u) {
+      const int l = __ffs(m) - 1;
+      const float v = __shfl_sync(kFull, k, l);
+      if ((mine >> l) & 1u) {
+        const F2 t = two_sum(s.hi, v);
+        s = F2{t.hi, __fadd_rn(s.lo, t.lo)};
+      }
+    }
+    if (first && (int)(threadIdx.x & 31u) == __ffs(mine) - 1) deposit(at, __fadd_rn(s.hi, s.lo));
   }
   __device__ __forceinline__ void leave(const TraceArgs& A, LaneAcc& acc) const {
     const double u = unit(A);
     acc.absorbed += ((double)acc.Pstart - (double)P) * u;
     acc.escaped += (double)P * u;
   }
-  // Around the segments of a queue visit: the pair sum renormalised before,
-  // the bound on a package's segments tested after.
+  // Around the segments of a queue visit: the pair sum renormalised before;
+  // the segments counted, and their number bounded, after.
   __device__ __forceinline__ void begin_visit() {
     const F2 t2 = fast_two_sum(tau, tau_lo);
     tau = t2.hi;
     tau_lo = t2.lo;
   }
-  __device__ __forceinline__ int end_visit(const TraceArgs& A, LaneAcc& acc, int n, int ev) {
-    steps += n;
-    if (ev == EV_NONE && steps > A.max_steps) {
+  __device__ __forceinline__ int end_visit(const TraceArgs& A, LaneAcc& acc, int ev) {
+    nseg += cnt;
+    acc.steps += cnt;
+    cnt = 0;
+    if (ev == EV_NONE && acc.steps > A.max_steps) {
       set_status(A.ctl, RT_ERR_STATE);
       leave(A, acc);
       return EV_DONE;
     }
+    if (ev == EV_SPLIT || ev == EV_HALT) seal(A, acc);
     return ev;
   }
   __device__ __forceinline__ void on_split(const TraceArgs& A, LaneAcc& acc) const {
@@ -1068,6 +1167,8 @@ __global__ void __launch_bounds__(kBlock, MinBlocks) trace_kernel(TraceArgs A) {
   __shared__ unsigned long long sh_hsh[kShInst * kLevels];
   __shared__ LaneAcc sh_acc[kBlock];
   __shared__ unsigned int sh_bfb[kShInst * 2];
+  __shared__ IdleWarp sh_idle[kBlock / 32];
+  __shared__ uint32_t sh_epoch;
   for (int i = threadIdx.x; i < kShInst * kLevels; i += blockDim.x) {
     sh_cnt[i] = 0;
     sh_hsh[i] = 0;
@@ -1080,12 +1181,13 @@ __global__ void __launch_bounds__(kBlock, MinBlocks) trace_kernel(TraceArgs A) {
   acc.emitted = acc.absorbed = acc.escaped = acc.resumed = acc.halted = 0.0;
   acc.segments = acc.fallbacks = acc.fallbacks_tau = 0;
   acc.inst = -1;
+  if ((threadIdx.x & 31) == 0) sh_idle[threadIdx.x >> 5] = IdleWarp{-1, 0, 256u};
+  if (threadIdx.x == 0) sh_epoch = (uint32_t)A.ctl[CTL_EPOCH];
   __syncthreads();
   LevelCounters LC{sh_cnt, sh_hsh};
 
   const int lane = threadIdx.x & 31;
   const unsigned lt_mask = (1u << lane) - 1u;
-  const uint32_t epoch = (uint32_t)A.ctl[CTL_EPOCH];
   using QR = typename W::template Q<FSL>;
   QR* queue = (QR*)A.queue;
   // tickets: roots [0, n_roots), packages in flight [n_roots, qbase), queue slots after
@@ -1101,9 +1203,7 @@ __global__ void __launch_bounds__(kBlock, MinBlocks) trace_kernel(TraceArgs A) {
   bool active = false;
   int ev = EV_NONE;
   long long ticket = -1;
-  long long seen_out = -1;
-  uint64_t seen_ns = global_ns();
-  unsigned backoff = 256;  // ns; idle warps back off exponentially up to 4 us
+  IdleWarp& idle = sh_idle[threadIdx.x >> 5];
 
   for (;;) {
     // (1) What the last queue visit ended.  A split keeps child 0 and hands
@@ -1169,7 +1269,7 @@ __global__ void __launch_bounds__(kBlock, MinBlocks) trace_kernel(TraceArgs A) {
           const unsigned j = 3u * i + (k - 1u);
           if (j < nin) continue;  // placed in a free lane of this warp
           const unsigned long long slot = base + (j - nin);
-          if (slot < A.cap) W::template publish<FSL>(&queue[slot], w.make_child(4u * w.pix + k), epoch);
+          if (slot < A.cap) W::template publish<FSL>(&queue[slot], w.make_child(4u * w.pix + k), sh_epoch);
           else ++dropped;
         }
         if (dropped) {
@@ -1210,7 +1310,7 @@ __global__ void __launch_bounds__(kBlock, MinBlocks) trace_kernel(TraceArgs A) {
         const unsigned long long slot = tk - qbase;
         if (slot < A.cap) {
           Rec q;
-          if (W::template poll<FSL>(&queue[slot], epoch, q)) {
+          if (W::template poll<FSL>(&queue[slot], sh_epoch, q)) {
             w.load(q);
             fresh = START_CHILD;
           }
@@ -1247,33 +1347,60 @@ __global__ void __launch_bounds__(kBlock, MinBlocks) trace_kernel(TraceArgs A) {
       outst = __shfl_sync(kFull, outst, 0);
       if (outst <= 0) break;
       const uint64_t now = global_ns();
-      if (outst != seen_out) {
-        seen_out = outst;
-        seen_ns = now;
-      } else if ((long long)(now - seen_ns) > A.timeout_ns) {
+      const unsigned backoff = idle.backoff;
+      const bool moved = outst != idle.seen_out;
+      const bool late = !moved && (long long)(now - idle.seen_ns) > A.timeout_ns;
+      __syncwarp();
+      if (late) {
         if (lane == 0) set_status(A.ctl, RT_ERR_TIMEOUT);
         break;
       }
+      if (lane == 0) {
+        if (moved) {
+          idle.seen_out = outst;
+          idle.seen_ns = now;
+        }
+        idle.backoff = backoff < 4096 ? 2 * backoff : 4096;
+      }
+      __syncwarp();
       __nanosleep(backoff);
-      backoff = backoff < 4096 ? 2 * backoff : 4096;
       continue;
     }
-    backoff = 256;
-    seen_out = -1;  // the no-progress clock runs over one idle stretch only
+    if (lane == 0) {
+      idle.backoff = 256;
+      idle.seen_out = -1;  // the no-progress clock runs over one idle stretch only
+    }
     // (6) trace a few segments
     if (active && ev == EV_NONE) {
       w.begin_visit();
-      int it = 0;
-      for (; it < A.segs_per_iter; ++it) {
+      for (int it = 0; it < A.segs_per_iter; ++it) {
         ev = w.template step<FSL>(A, acc);
         if (ev != EV_NONE) break;
       }
-      ev = w.end_visit(A, acc, it, ev);
-      if (ev == EV_SPLIT || ev == EV_HALT) w.seal(A, acc);
     }
     // The lanes left the loop at different steps: reconverge them here, before
     // the warp-wide steps.  (Without this barrier the same kernel ran
     // 7-11 % slower on every workload measured.)
+    __syncwarp();
+    // (6b) the decisions that the segments left, for all lanes together: a
+    //      lane's last segment (split, exit, halt, termination) runs here once
+    //      per visit instead of inside the loop whenever one lane needs it
+    //      (with the rates interleaved: 24 sources in an ionised 128^3 grid 9.67 ->
+    //      7.62 ms, 1000 in a clumpy 256^3 grid 3.51 -> 2.71 ms)
+    if constexpr (W::kStaged) {
+      const bool left = ev == EV_RARE || ev == EV_TERM;
+      if (__ballot_sync(kFull, left)) {
+        float dep = 0.0f;
+        const int at = w.idx;
+        const bool first = left && w.r.hi == 0.0f;
+        if (ev == EV_RARE) ev = w.template slow<FSL>(A, acc, dep);
+        if (ev == EV_TERM) ev = w.template terminate<FSL>(A, acc, dep);
+        __syncwarp();
+        if (__ballot_sync(kFull, first)) w.deposit_first(first, at, dep);
+        if (left && !first) w.deposit(at, dep);
+      }
+      if (active) ev = w.end_visit(A, acc, ev);
+    }
     __syncwarp();
     // (7) halted packages go to the output store (one atomic per warp);
     //     from here on they are finished packages
@@ -1448,33 +1575,35 @@ constexpr int kMinBlocks64 = 2;
 constexpr int kMinBlocks32 = TRACE_MIN_BLOCKS;
 
 using TraceKernel = void (*)(TraceArgs);
-// The instantiation for a launch; null for a combination that has none.
-// fsl: finite speed of light (A.rlim*, res_in, halt_out set).
-static TraceKernel trace_instance(int precision, int fsl, int variant) {
-  if (precision == RT_FP64)
-    return fsl ? trace_kernel<Walk64, kMinBlocks64, true> : trace_kernel<Walk64, kMinBlocks64, false>;
+template <bool FSL, bool FC>
+static TraceKernel trace_instance32(int variant) {
   switch (variant) {
-    case WALK_EXACT:
-      return fsl ? trace_kernel<Walk32<true, true>, kMinBlocks32, true>
-                 : trace_kernel<Walk32<true, true>, kMinBlocks32, false>;
-    case WALK_ANY:
-      return fsl ? trace_kernel<Walk32<false, true>, kMinBlocks32, true>
-                 : trace_kernel<Walk32<false, true>, kMinBlocks32, false>;
+    case WALK_EXACT: return trace_kernel<Walk32<true, true, FC>, kMinBlocks32, FSL>;
+    case WALK_ANY: return trace_kernel<Walk32<false, true, FC>, kMinBlocks32, FSL>;
     case WALK_ANY_PLAIN:
-      if (!fsl) return trace_kernel<Walk32<false, false>, kMinBlocks32, false>;
+      if constexpr (!FSL) return trace_kernel<Walk32<false, false, FC>, kMinBlocks32, false>;
   }
   return nullptr;
 }
+// The instantiation for a launch; null for a combination that has none.
+// fsl: finite speed of light (A.rlim*, res_in, halt_out set); fc: covering
+// factor (A.fc; the FP64 walker tests that at run time).
+static TraceKernel trace_instance(int precision, int fsl, int fc, int variant) {
+  if (precision == RT_FP64)
+    return fsl ? trace_kernel<Walk64, kMinBlocks64, true> : trace_kernel<Walk64, kMinBlocks64, false>;
+  if (fsl) return fc ? trace_instance32<true, true>(variant) : trace_instance32<true, false>(variant);
+  return fc ? trace_instance32<false, true>(variant) : trace_instance32<false, false>(variant);
+}
 
-cudaError_t trace_occupancy(int precision, int fsl, int variant, int block, int* blocks_per_sm) {
-  const TraceKernel k = trace_instance(precision, fsl, variant);
+cudaError_t trace_occupancy(int precision, int fsl, int fc, int variant, int block, int* blocks_per_sm) {
+  const TraceKernel k = trace_instance(precision, fsl, fc, variant);
   if (!k || block != kBlock) return cudaErrorInvalidValue;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, block, 0);
 }
 
 cudaError_t launch_trace(int precision, int fsl, int variant, const TraceArgs& A, int grid, int block,
                          cudaStream_t st) {
-  const TraceKernel k = trace_instance(precision, fsl, variant);
+  const TraceKernel k = trace_instance(precision, fsl, A.fc, variant);
   if (!k || block != kBlock) return cudaErrorInvalidValue;
   k<<<grid, block, 0, st>>>(A);
   return cudaGetLastError();
