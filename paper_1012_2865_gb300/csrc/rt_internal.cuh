@@ -151,7 +151,7 @@ inline size_t blk_rows_bytes(int num_sms, int rows) {
   return (size_t)num_sms * kBlkMaxPerSM * (size_t)rows * kBlkRow * sizeof(double);
 }
 
-// Queue records.  The tag word is written last with release semantics and
+// Queue records.  The tag word is written last, after a fence, and
 // equals the trace's epoch once the record is complete.  The same layouts
 // hold packages in flight between traces (finite speed of light), where the
 // tag is not used as one.
@@ -260,8 +260,8 @@ __device__ __forceinline__ uint32_t ld_relaxed_u32(const uint32_t* p) {
   asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
 }
-__device__ __forceinline__ void st_release_u32(uint32_t* p, uint32_t v) {
-  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+__device__ __forceinline__ void st_relaxed_u32(uint32_t* p, uint32_t v) {
+  asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 __device__ __forceinline__ long long ld_acquire_s64(const unsigned long long* p) {
   long long v;
