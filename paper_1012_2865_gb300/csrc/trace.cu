@@ -588,6 +588,11 @@ struct Axis {
     else ++k;
     plane();
   }
+  __device__ __forceinline__ void back() {
+    if (EXACT) d -= 1.0f;
+    else --k;
+    plane();
+  }
   // Cell c of an axis with direction n, source coordinate s (EXACT) or
   // sa + sb (general), dim cells and index stride `step`.
   __device__ __forceinline__ void init(int c, F2 n, float s, int sa, F2 sb, int step) {
@@ -935,8 +940,8 @@ struct Walk32 {
     return (m0 ? 1 : 0) | (m1 ? 2 : 0) | (m2 ? 4 : 0) | (split ? 8 : 0) | (halt ? 64 : 0) | (out ? 128 : 0);
   }
 
-  // The segment from r to `end` in the current cell; returns its k_ph.
-  __device__ __forceinline__ float segment(const TraceArgs& A, LaneAcc& acc, F2 end) {
+  // The segment from r to `end` in a cell of density (nh, nh_lo); returns its k_ph.
+  __device__ __forceinline__ float segment(const TraceArgs& A, LaneAcc& acc, F2 r, F2 end, float nh, float nh_lo) {
     // length as a pair (both ends are pairs; |end| >= |r| or the difference of
     // the high parts is exact)
     const float dh = __fsub_rn(end.hi, r.hi);
@@ -971,7 +976,7 @@ struct Walk32 {
     const float phi = dtau < 0.25f ? ser : __fdividef(1.0f - tr, dtau);
     float fcv = 1.0f;
     if (FC) {
-      fcv = cover(A, dr);
+      fcv = cover(A, r, dr);
       acc.cover = fcv;
     }
     const float k = P * w * dr * phi * fcv;
@@ -987,7 +992,7 @@ struct Walk32 {
   // covering factor (Eq. "fc") of a segment of length dr, in FP32 from the
   // pairs' high parts: its error (~1e-4 relative) is far inside the tolerance
   // on k_ph
-  __device__ __forceinline__ float cover(const TraceArgs& A, float dr) const {
+  __device__ __forceinline__ float cover(const TraceArgs& A, F2 r, float dr) const {
     const float rh = __fadd_rn(r.hi, r.lo);
     const float L = rh * A.theta32[lvl()];
     if (!(L > 0.0f)) return 1.0f;
@@ -1023,13 +1028,25 @@ struct Walk32 {
     if (rn.hi >= lim || (m2 && (m0 || m1))) return EV_RARE;
     // (the exact tie of a 45-degree ray crosses both planes)
     if (m0 && m1 && !(diag_exact() && f2_eq(a0.t, a1.t))) return EV_RARE;
-    deposit(idx, segment(A, acc, rn));
+    // cross first: the next cell's density arrives while this segment's
+    // absorption is worked out (24 sources in an ionised 128^3 grid 7.30 -> 6.81 ms)
+    const int at = idx;
+    const F2 r0 = r;
+    const float nh0 = nh, nh0_lo = nh_lo;
+    if (!FC) advance(rn, m0, m1, m2);
+    deposit(at, segment(A, acc, r0, rn, nh0, nh0_lo));
+    if (FC) advance(rn, m0, m1, m2);  // the covering factor reads the cell from the planes
     if (fmaf(sk, q, tau) > A.tau_near) {
-      r = rn;
+      // back to the cell (terminate() decides, and crosses again)
+      if (m0) a0.back();
+      if (m1) a1.back();
+      if (m2) a2.back();
+      idx = at;
+      nh = nh0;
+      nh_lo = nh0_lo;
       acc.mask = (m0 ? 1 : 0) | (m1 ? 2 : 0) | (m2 ? 4 : 0);
       return EV_TERM;
     }
-    advance(rn, m0, m1, m2);
     return EV_NONE;
   }
 
@@ -1044,7 +1061,7 @@ struct Walk32 {
     acc.fallbacks += fb;
     if (m & 8) return EV_SPLIT;
     const bool halt = FSL && (m & 64);  // Step 3j: the segment ends at rlim
-    dep = segment(A, acc, halt ? rlim : rn);
+    dep = segment(A, acc, r, halt ? rlim : rn, nh, nh_lo);
     acc.mask = m;
     if (fmaf(sk, q, tau) > A.tau_near) {
       r = rn;
