@@ -39,12 +39,12 @@ cudaError_t launch_read_rates(int precision, long long n, const void* K, const v
 cudaError_t launch_write_rates(long long n, const void* k, const void* g, int dtype, void* kg, double scale,
                                cudaStream_t st);
 cudaError_t launch_complement(long long n, const double* x, double* out, cudaStream_t st);
-cudaError_t launch_commit_state(int precision, long long n, unsigned long long* ctl, const double* sn,
-                               const double* sx, const double* sz, double* nH, double* xHI, double* xHII, void* nhi,
-                               cudaStream_t st);
-cudaError_t launch_timestep(long long n, int nx, int ny, int nz, const double* nH, const double* xHI, const void* K,
-                            int fp64_rates, double sdx, double tau_front, float eps, float alpha, float dt_max,
-                            float unit, float* dtc, unsigned int* out, cudaStream_t st);
+cudaError_t launch_commit_state(int precision, long long n, unsigned long long* ctl, unsigned long long* verdict,
+                               const double* sn, const double* sx, const double* sz, double* nH, double* xHI,
+                               double* xHII, void* nhi, cudaStream_t st);
+cudaError_t launch_timestep(int nx, int ny, int nz, const double* nH, const double* xHI, const void* K, int fp64_rates,
+                            double sdx, double tau_front, float eps, float alpha, float dt_max, float unit,
+                            unsigned int* out, unsigned long long* done, cudaStream_t st);
 cudaError_t launch_check_state(long long n, const double* nH, const double* x, unsigned long long* bad,
                                cudaStream_t st);
 cudaError_t launch_check_density(long long n, const double* a, unsigned long long* bad, cudaStream_t st);
@@ -171,8 +171,6 @@ struct TraceState {
   }
 };
 
-constexpr int kAccWords = 8;  // photon budget sums per grid (see InstDev.acc)
-
 // Packages in flight between traces (finite speed of light): two stores used
 // alternately (the next trace continues what the last one halted into
 // buf[in] and halts into the other), the halting radius per age on the
@@ -215,8 +213,8 @@ struct rt_grid {
   void* nhi = nullptr;  // FP64, or FP32 pairs
   void* K = nullptr;    // FP64, or (k_ph, Gamma) FP32 pairs (then G is null)
   void* G = nullptr;
-  double* acc = nullptr;               // kAccWords doubles
-  unsigned long long* cnt = nullptr;   // kCntWords
+  double* acc = nullptr;               // kAccWords doubles, behind the control words (ts.ctl)
+  unsigned long long* cnt = nullptr;   // kCntWords, behind them
   InstDev* inst_dev = nullptr;
   struct SrcIn { double pos[3], ndot, e_ph, sigma; int type = 0; };
   // helium absorbers and rates of photon types 1 (He I) and 2 (He II), once set
@@ -255,7 +253,6 @@ struct rt_grid {
   double* xHII_alt = nullptr;                // into them and they swap with xHI, xHII on commit
   char* dn_stage = nullptr;                  // 3 * ncell * 8 bytes: k_ph, Gamma, x_HI
   std::string set_err;                       // message of a rejected asynchronous state
-  bool check_words_set = false;              // CTL_CHECK_N/X hold ~0 (then kept so by each commit)
   ~rt_grid() {
     if (up) cudaStreamSynchronize(up);
     if (dn) cudaStreamSynchronize(dn);
@@ -265,7 +262,7 @@ struct rt_grid {
     if (up) cudaStreamDestroy(up);
     if (dn) cudaStreamDestroy(dn);
     cudaFree(nH); cudaFree(xHI); cudaFree(xHII); cudaFree(nhi); cudaFree(K); cudaFree(G);
-    cudaFree(acc); cudaFree(cnt); cudaFree(inst_dev); cudaFree(src_dev);
+    cudaFree(inst_dev); cudaFree(src_dev);
     for (int t = 0; t < 2; ++t) {
       if (nhe[t] != nhe64[t]) cudaFree(nhe[t]);
       cudaFree(nhe64[t]); cudaFree(Khe[t]); cudaFree(Ghe[t]);
@@ -332,25 +329,19 @@ int rt_ctx_destroy(rt_ctx* ctx) {
   return RT_OK;
 }
 
-// Range check of a state already on the device (nH may be NULL), on stream
-// st: RT_OK, or RT_ERR_INVALID_ARG naming the first bad cell and its value.
-// Synchronises st.
-static int check_state(const char* who, long long ncell, const double* nH, const double* x, cudaStream_t st) {
-  unsigned long long* bad = nullptr;
-  CUDA_TRY(cudaMallocAsync((void**)&bad, 2 * sizeof(unsigned long long), st));
-  unsigned long long h[2] = {0, 0};
-  cudaError_t e = cudaMemsetAsync(bad, 0xff, 2 * sizeof(unsigned long long), st);
-  if (e == cudaSuccess) e = launch_check_state(ncell, nH, x, bad, st);
-  if (e == cudaSuccess) g_launches.fetch_add(1);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(h, bad, sizeof h, cudaMemcpyDeviceToHost, st);
+// The verdict of a state check from device words (first bad n_H cell, x_HI
+// cell; ~0 = none): RT_OK, or RT_ERR_INVALID_ARG naming the first bad cell and
+// its value.  Synchronises st; rb: 16 pinned bytes.
+static int read_verdict(const char* who, const unsigned long long* words, unsigned long long* rb, const double* nH,
+                        const double* x, cudaStream_t st) {
+  cudaError_t e = cudaMemcpyAsync(rb, words, 2 * sizeof *rb, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  cudaFreeAsync(bad, st);
   if (e != cudaSuccess) return fail(RT_ERR_CUDA, "%s: state check: %s", who, cudaGetErrorString(e));
   for (int k = 0; k < 2; ++k) {
-    if (h[k] == ~0ULL) continue;
+    if (rb[k] == ~0ULL) continue;
     double v = 0.0;
-    cudaMemcpy(&v, (k == 0 ? nH : x) + h[k], sizeof v, cudaMemcpyDeviceToHost);
-    return fail(RT_ERR_INVALID_ARG, "%s: %s[%llu] = %g", who, k == 0 ? "n_H" : "x_HI", h[k], v);
+    cudaMemcpy(&v, (k == 0 ? nH : x) + rb[k], sizeof v, cudaMemcpyDeviceToHost);
+    return fail(RT_ERR_INVALID_ARG, "%s: %s[%llu] = %g", who, k == 0 ? "n_H" : "x_HI", rb[k], v);
   }
   return RT_OK;
 }
@@ -398,10 +389,10 @@ int rt_create_grid(rt_ctx* ctx, const rt_grid_desc* d, void* stream, rt_grid** o
   ALLOC(g->nhi, n8);
   ALLOC(g->K, n8);
   if (d->precision == RT_FP64) ALLOC(g->G, n8);
-  ALLOC(g->acc, kAccWords * sizeof(double));
-  ALLOC(g->cnt, kCntWords * sizeof(unsigned long long));
   ALLOC(g->inst_dev, sizeof(InstDev));
-  ALLOC(g->ts.ctl, CTL_N * sizeof(unsigned long long));
+  ALLOC(g->ts.ctl, kWordsAll * sizeof(unsigned long long));
+  g->acc = (double*)(g->ts.ctl + kWordsAcc);
+  g->cnt = g->ts.ctl + kWordsCnt;
   ALLOC(g->ts.blk, blk_rows_bytes(ctx->num_sms, 1));
   g->ts.blk_blocks = ctx->num_sms * kBlkMaxPerSM;
   g->ts.blk_rows = 1;
@@ -409,24 +400,34 @@ int rt_create_grid(rt_ctx* ctx, const rt_grid_desc* d, void* stream, rt_grid** o
   cudaStream_t st = g->stream;
   if ((rc = upload(g->nH, d->n_H, n8, d->mem_kind, st)) != RT_OK) { delete g; return rc; }
   if ((rc = upload(g->xHI, d->x_HI, n8, d->mem_kind, st)) != RT_OK) { delete g; return rc; }
-  // the values are checked on the device once they are there
-  if ((rc = check_state("rt_create_grid", ncell, g->nH, g->xHI, st)) != RT_OK) { delete g; return rc; }
+  // the values are checked on the device once they are there; the check words
+  // start (and every check leaves them) at ~0
+  cudaError_t e = cudaMallocHost(&g->host_rb, 4096);
+  if (e == cudaSuccess) e = cudaMemsetAsync(g->ts.ctl, 0, kWordsAll * sizeof(unsigned long long), st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(g->ts.ctl + CTL_CHECK_N, 0xff, 2 * sizeof(unsigned long long), st);
+  const unsigned int inf[2] = {0x7f800000u, 0u};
+  if (e == cudaSuccess) e = cudaMemcpyAsync(g->ts.ctl + kWordsStep, inf, sizeof inf, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = launch_check_state(ncell, g->nH, g->xHI, g->ts.ctl + CTL_CHECK_N, st);
+  if (e != cudaSuccess) { delete g; return fail(RT_ERR_CUDA, "rt_create_grid: state check: %s", cudaGetErrorString(e)); }
+  g_launches.fetch_add(1);
+  if ((rc = read_verdict("rt_create_grid", g->ts.ctl + CTL_CHECK_N, (unsigned long long*)g->host_rb, g->nH, g->xHI, st)) != RT_OK) {
+    delete g;
+    return rc;
+  }
   if (d->x_HII) {
     if ((rc = upload(g->xHII, d->x_HII, n8, d->mem_kind, st)) != RT_OK) { delete g; return rc; }
   } else {
-    cudaError_t e = launch_complement(ncell, g->xHI, g->xHII, st);
+    e = launch_complement(ncell, g->xHI, g->xHII, st);
     if (e != cudaSuccess) { delete g; return fail(RT_ERR_CUDA, "complement: %s", cudaGetErrorString(e)); }
     g_launches.fetch_add(1);
   }
-  cudaError_t e = launch_refresh(g->precision, ncell, g->nH, g->xHI, g->nhi, st);
+  e = launch_refresh(g->precision, ncell, g->nH, g->xHI, g->nhi, st);
   if (e != cudaSuccess) { delete g; return fail(RT_ERR_CUDA, "refresh: %s", cudaGetErrorString(e)); }
   g_launches.fetch_add(1);
-  e = cudaMemsetAsync(g->ts.ctl, 0, CTL_N * sizeof(unsigned long long), st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(g->K, 0, n8, st);
+  e = cudaMemsetAsync(g->K, 0, n8, st);
   if (e == cudaSuccess && g->G) e = cudaMemsetAsync(g->G, 0, n8, st);
   const InstDev I = inst_of(g);
   if (e == cudaSuccess) e = cudaMemcpyAsync(g->inst_dev, &I, sizeof I, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMallocHost(&g->host_rb, 4096);
   if (e == cudaSuccess) e = cudaEventCreate(&g->ev0);
   if (e == cudaSuccess) e = cudaEventCreate(&g->ev1);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -884,13 +885,11 @@ static void note_rejected_state(rt_grid* g, unsigned long long bad_n, unsigned l
 }
 
 static int read_budget(rt_grid* g, rt_budget* out) {
-  double* hacc = (double*)g->host_rb;
-  unsigned long long* hcnt = (unsigned long long*)((char*)g->host_rb + 64);
-  unsigned long long* hctl = (unsigned long long*)((char*)g->host_rb + 512);
+  unsigned long long* hctl = (unsigned long long*)g->host_rb;
+  const double* hacc = (const double*)(hctl + kWordsAcc);
+  const unsigned long long* hcnt = hctl + kWordsCnt;
   cudaStream_t st = g->stream;
-  CUDA_TRY(cudaMemcpyAsync(hacc, g->acc, kAccWords * sizeof(double), cudaMemcpyDeviceToHost, st));
-  CUDA_TRY(cudaMemcpyAsync(hcnt, g->cnt, kCntWords * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
-  CUDA_TRY(cudaMemcpyAsync(hctl, g->ts.ctl, CTL_N * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
+  CUDA_TRY(cudaMemcpyAsync(hctl, g->ts.ctl, kWordsRead * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
   CUDA_TRY(cudaStreamSynchronize(st));
   memset(out, 0, sizeof *out);
   out->emitted = hacc[0];
@@ -1020,33 +1019,39 @@ int rt_set_state(rt_grid* g, const double* n_H, const double* x_HI, const double
   const long long ncell = g->ncell;
   const size_t n8 = (size_t)ncell * 8;
   cudaStream_t st = g->stream;
-  // stage the new state on the device, check it there, and only then replace
-  // the grid's state (which an invalid call leaves unchanged)
-  const int nf = (n_H ? 1 : 0) + 1 + (x_HII ? 1 : 0);
+  // The new state is checked where it lies on the device (a host state is
+  // staged there first) and replaces the grid's in the next kernel, unless a
+  // cell failed (an invalid call leaves the grid unchanged); then the caller
+  // learns the verdict.  (Staging device arrays too, in memory allocated for
+  // the call, and copying them after the verdict took 360 us for a 128^3 state
+  // and 250 us for a 32^3 one, now 66 and 38 us.)
+  const double *sn = n_H, *sx = x_HI, *sz = x_HII;
   double* stage = nullptr;
-  CUDA_TRY(cudaMallocAsync((void**)&stage, nf * n8, st));
-  double* sn = n_H ? stage : nullptr;
-  double* sx = stage + (n_H ? ncell : 0);
-  double* sz = x_HII ? sx + ncell : nullptr;
   int rc = RT_OK;
-  if (n_H) rc = upload(sn, n_H, n8, mem_kind, st);
-  if (!rc) rc = upload(sx, x_HI, n8, mem_kind, st);
-  if (!rc && x_HII) rc = upload(sz, x_HII, n8, mem_kind, st);
-  if (!rc) rc = check_state("rt_set_state", ncell, sn, sx, st);
-  if (rc) {
-    cudaFreeAsync(stage, st);
-    return rc;
+  if (mem_kind == RT_MEM_HOST) {
+    const int nf = (n_H ? 1 : 0) + 1 + (x_HII ? 1 : 0);
+    CUDA_TRY(cudaMallocAsync((void**)&stage, nf * n8, st));
+    double* d = stage;
+    const double** dst[3] = {&sn, &sx, &sz};
+    for (int f = 0; f < 3 && !rc; ++f) {
+      if (!*dst[f]) continue;
+      rc = upload(d, *dst[f], n8, mem_kind, st);
+      *dst[f] = d;
+      d += ncell;
+    }
   }
-  if (n_H) CUDA_TRY(cudaMemcpyAsync(g->nH, sn, n8, cudaMemcpyDeviceToDevice, st));
-  CUDA_TRY(cudaMemcpyAsync(g->xHI, sx, n8, cudaMemcpyDeviceToDevice, st));
-  if (x_HII) {
-    CUDA_TRY(cudaMemcpyAsync(g->xHII, sz, n8, cudaMemcpyDeviceToDevice, st));
-  } else {
-    LAUNCH_TRY(launch_complement(ncell, g->xHI, g->xHII, st));
+  if (!rc) {
+    cudaError_t e = launch_check_state(ncell, sn, sx, g->ts.ctl + CTL_CHECK_N, st);
+    if (e == cudaSuccess)
+      e = launch_commit_state(g->precision, ncell, g->ts.ctl, g->ts.ctl + kWordsVerdict, sn, sx, sz, g->nH, g->xHI,
+                              g->xHII, g->nhi, st);
+    if (e != cudaSuccess) rc = fail(RT_ERR_CUDA, "rt_set_state: %s", cudaGetErrorString(e));
+    else g_launches.fetch_add(2);
   }
-  LAUNCH_TRY(launch_refresh(g->precision, ncell, g->nH, g->xHI, g->nhi, st));
-  CUDA_TRY(cudaFreeAsync(stage, st));
-  return RT_OK;
+  if (!rc)
+    rc = read_verdict("rt_set_state", g->ts.ctl + kWordsVerdict, (unsigned long long*)((char*)g->host_rb + 2048), sn, sx, st);
+  if (stage) cudaFreeAsync(stage, st);
+  return rc;
 }
 
 // The FP32-mixed grid keeps Gamma in eV/s (FP32 erg/s values of faint cells
@@ -1065,11 +1070,6 @@ static int ensure_async(rt_grid* g, bool stage_up, bool stage_dn) {
   const size_t n8 = (size_t)g->ncell * 8;
   if (stage_up && !g->up_stage) CUDA_TRY(cudaMalloc((void**)&g->up_stage, 3 * n8));  // uploads with n_H
   if (stage_dn && !g->dn_stage) CUDA_TRY(cudaMalloc((void**)&g->dn_stage, 3 * n8));
-  if (!g->check_words_set) {
-    // ~0 = no failing cell; every commit leaves them so for the next upload
-    CUDA_TRY(cudaMemsetAsync(g->ts.ctl + CTL_CHECK_N, 0xff, 2 * sizeof(unsigned long long), g->stream));
-    g->check_words_set = true;
-  }
   return RT_OK;
 }
 
@@ -1120,7 +1120,7 @@ int rt_set_state_async(rt_grid* g, const double* n_H, const double* x_HI, const 
     sz = x_HII ? d + 2 * n : nullptr;
   }
   LAUNCH_TRY(launch_check_state(n, sn, sx, g->ts.ctl + CTL_CHECK_N, st));
-  LAUNCH_TRY(launch_commit_state(g->precision, n, g->ts.ctl, sn, sx, sz, g->nH, g->xHI, g->xHII, g->nhi, st));
+  LAUNCH_TRY(launch_commit_state(g->precision, n, g->ts.ctl, nullptr, sn, sx, sz, g->nH, g->xHI, g->xHII, g->nhi, st));
   CUDA_TRY(cudaEventRecord(g->ev_commit, st));
   return RT_OK;
 }
@@ -1368,25 +1368,16 @@ int rt_timestep(rt_grid* g, double eps_ion, double alpha_B, double sigma_front, 
   if (int rcw = wait_batch(g)) return rcw;
   CUDA_TRY(cudaSetDevice(g->ctx->device));
   cudaStream_t st = g->stream;
-  const long long n = g->ncell;
-  char* scratch = nullptr;
-  CUDA_TRY(cudaMallocAsync((void**)&scratch, (size_t)n * sizeof(float) + 256, st));
-  unsigned int* out = (unsigned int*)(scratch + (((size_t)n * sizeof(float) + 255) & ~(size_t)255));
+  unsigned int* out = (unsigned int*)(g->ts.ctl + kWordsStep);
   unsigned int* h = (unsigned int*)((char*)g->host_rb + 3072);
-  *h = 0x7f800000u;  // +inf
-  cudaError_t e = cudaMemcpyAsync(out, h, sizeof *h, cudaMemcpyHostToDevice, st);
   // finite dt_max: values in units of dt_max (cells outside the front hold 1)
   const bool finite = isfinite(dt_max) && dt_max < 3.0e38;
   const float dmax = finite ? (float)dt_max : 3.0e38f;
-  if (e == cudaSuccess)
-    e = launch_timestep(n, g->nx, g->ny, g->nz, g->nH, g->xHI, g->K, g->precision == RT_FP64,
-                        sigma_front * g->dx, tau_front, (float)eps_ion, (float)alpha_B, dmax, finite ? dmax : 1.0f,
-                        (float*)scratch, out, st);
-  if (e == cudaSuccess) g_launches.fetch_add(2);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(h, out, sizeof *h, cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  cudaFreeAsync(scratch, st);
-  if (e != cudaSuccess) return fail(RT_ERR_CUDA, "rt_timestep: %s", cudaGetErrorString(e));
+  LAUNCH_TRY(launch_timestep(g->nx, g->ny, g->nz, g->nH, g->xHI, g->K, g->precision == RT_FP64, sigma_front * g->dx,
+                             tau_front, (float)eps_ion, (float)alpha_B, dmax, finite ? dmax : 1.0f, out,
+                             g->ts.ctl + kWordsStep + 1, st));
+  CUDA_TRY(cudaMemcpyAsync(h, out + 1, sizeof *h, cudaMemcpyDeviceToHost, st));
+  CUDA_TRY(cudaStreamSynchronize(st));
   float v;
   memcpy(&v, h, sizeof v);
   double dt = finite ? (v >= 1.0f ? dt_max : (double)v * dt_max) : (v >= 3.0e38f ? dt_max : (double)v);
@@ -1944,10 +1935,9 @@ int rt_batch_get_budget(rt_batch* b, int slot, rt_budget* out) {
   if (rc) return rc;
   const int status = bs.status;
   rt_grid* g = b->slots[slot];
-  double* hacc = (double*)g->host_rb;
-  unsigned long long* hcnt = (unsigned long long*)((char*)g->host_rb + 64);
-  CUDA_TRY(cudaMemcpyAsync(hacc, g->acc, kAccWords * sizeof(double), cudaMemcpyDeviceToHost, b->stream));
-  CUDA_TRY(cudaMemcpyAsync(hcnt, g->cnt, kCntWords * sizeof(unsigned long long), cudaMemcpyDeviceToHost, b->stream));
+  const double* hacc = (const double*)g->host_rb;
+  const unsigned long long* hcnt = (const unsigned long long*)g->host_rb + kAccWords;
+  CUDA_TRY(cudaMemcpyAsync(g->host_rb, g->acc, (kAccWords + kCntWords) * sizeof(double), cudaMemcpyDeviceToHost, b->stream));
   CUDA_TRY(cudaStreamSynchronize(b->stream));
   memset(out, 0, sizeof *out);
   out->emitted = hacc[0];

@@ -44,6 +44,18 @@ enum CtlWord {
   CTL_N = 64             // words (512 bytes)
 };
 
+// A grid's words in one allocation: the control words, then the budget sums
+// and counters that a trace leaves (read back together with them), then the
+// verdict of a state check (first bad n_H cell, x_HI cell; ~0 = none) and the
+// timestep's minimum (running, and of the last call).
+constexpr int kAccWords = 8;  // photon budget sums per grid (see InstDev.acc)
+constexpr int kWordsAcc = CTL_N;
+constexpr int kWordsCnt = kWordsAcc + kAccWords;
+constexpr int kWordsRead = kWordsCnt + 2 * kLevels + 3;
+constexpr int kWordsVerdict = kWordsRead + 1;
+constexpr int kWordsStep = kWordsVerdict + 2;
+constexpr int kWordsAll = kWordsStep + 2;
+
 // trace_init_kernel modes for the in-flight stores (finite speed of light)
 enum FlightMode {
   FLIGHT_OFF = 0,      // nothing in flight: RESUME = HALTED = 0
@@ -136,6 +148,7 @@ constexpr int kCntSegments = 2 * kLevels;
 constexpr int kCntFallbacks = 2 * kLevels + 1;
 constexpr int kCntFallbacksTau = 2 * kLevels + 2;
 constexpr int kCntWords = 2 * kLevels + 3;
+static_assert(kWordsRead == kWordsCnt + kCntWords, "layout of a grid's words");
 
 // Per-block budget rows of a trace launch (global memory, one buffer per
 // grid or batch): for each block and each of the launch's first kBlkGrids

@@ -1,0 +1,94 @@
+"""State and rate fields through the C ABI at sizes where the kernels behind
+them change form: odd cell counts and misaligned device arrays (no 16-byte
+accesses), a rejected state that must leave the grid as it was, k_ph and Gamma
+of a mixed grid written and read back in either type and place, and timestep
+tiles that the grid does not fill."""
+import numpy as np
+import pytest
+
+import parity
+from oracle import timestep
+from paper_1012_2865_gb300 import native, synth
+
+pytestmark = pytest.mark.gpu
+
+
+def _medium(dims, seed=4, sources=2):
+    rng = np.random.default_rng(seed)
+    box = synth.box_cm(dims[0], 6.6 * dims[0] / 32)
+    n = int(np.prod(dims))
+    pos, ndot, e, sg = synth.random_sources(dims, box / dims[0], sources, 1e48, 1e49, rng)
+    return synth._grid(dims, box, rng.uniform(1e-3, 1e-2, n), rng.uniform(1e-3, 1.0, n), pos, ndot, e, sg)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32_mixed"])
+@pytest.mark.parametrize("dims,skip", [((3, 5, 7), 0), ((4, 5, 6), 0), ((4, 5, 6), 1), ((33, 9, 8), 1)])
+def test_device_state_replaces_and_rejects(precision, dims, skip):
+    import torch
+    g = _medium(dims)
+    n = int(np.prod(dims))
+    rng = np.random.default_rng(8)
+    want = _medium(dims, seed=9)
+    want.update({k: g[k] for k in ("pos_cm", "ndot", "e_ph_eV", "sigma_cm2")})
+
+    def dev(a):  # a contiguous device array, off 16-byte alignment where skip is 1
+        t = torch.zeros(n + skip, dtype=torch.float64, device="cuda")
+        t[skip:] = torch.tensor(a, dtype=torch.float64)
+        return t[skip:]
+
+    grid = native.Grid(parity.ctx(), g, precision)
+    for field, cell, value in (("x_HI", n - 1, 1.5), ("x_HI", 0, float("nan")), ("n_H", n // 2, -1.0)):
+        bad = {"x_HI": rng.uniform(0, 1, n), "n_H": rng.uniform(0, 1, n)}
+        bad[field][cell] = value
+        with pytest.raises(native.RtError, match=rf"{field}\[{cell}\]"):
+            native.rt_set_state(grid.h, dev(bad["x_HI"]), n_H=dev(bad["n_H"]))
+    np.testing.assert_array_equal(grid.rates()["x_HI"], g["x_HI"])
+    ref = native.Grid(parity.ctx(), want, precision)
+    native.rt_set_state(grid.h, dev(want["x_HI"]), dev(want["x_HII"]), dev(want["n_H"]))
+    a, b = grid.trace(**synth.DEFAULT_PARAMS), ref.trace(**synth.DEFAULT_PARAMS)
+    np.testing.assert_array_equal(a["counts"], b["counts"])
+    assert a["segments"] == b["segments"]
+    np.testing.assert_array_equal(grid.rates()["x_HI"], want["x_HI"])
+    np.testing.assert_array_equal(grid.x_HII(), want["x_HII"])
+    # FP32 deposits: at most 200 a cell here, each rounding by 2^-24 of the sum
+    np.testing.assert_allclose(grid.rates()["kph"], ref.rates()["kph"], rtol=200 * 2.0 ** -24)
+    grid.close()
+    ref.close()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32_mixed"])
+def test_rates_round_trip(precision):
+    import torch
+    dims = (5, 3, 7)
+    n = int(np.prod(dims))
+    grid = native.Grid(parity.ctx(), _medium(dims), precision)
+    rng = np.random.default_rng(2)
+    k = synth.round_f32(10.0 ** rng.uniform(-30, -8, n))
+    gam = 10.0 ** rng.uniform(-44, -20, n)
+    k[0] = gam[0] = 0.0
+    native.rt_set_rates(grid.h, k, gam)
+    for dtype, np_dtype in ((native.RT_DTYPE_F64, np.float64), (native.RT_DTYPE_F32, np.float32)):
+        for where in ("host", "device"):
+            r = native.rt_get_rates(grid.h, n, dtype, where)
+            got = {q: np.asarray(v.cpu() if where == "device" else v) for q, v in r.items()}
+            assert got["kph"].dtype == np_dtype
+            np.testing.assert_array_equal(got["kph"], k.astype(np_dtype))
+            # Gamma passes through FP32 eV/s on the mixed path and FP32 outputs (2^-24 each, and the
+            # smallest FP32 number where it is subnormal)
+            tol = 0.0 if precision == "fp64" and dtype == native.RT_DTYPE_F64 else 2.0 ** -22
+            np.testing.assert_allclose(got["gamma"], gam, rtol=tol, atol=0.0 if tol == 0.0 else 1.5e-45)
+    t = torch.tensor(k * 2, device="cuda")
+    native.rt_set_rates(grid.h, t, torch.tensor(gam, device="cuda"))
+    np.testing.assert_array_equal(grid.rates()["kph"], k * 2)
+    grid.close()
+
+
+@pytest.mark.parametrize("dims", [(1, 1, 1), (32, 8, 8), (33, 9, 9), (31, 7, 17), (3, 40, 2), (70, 1, 5)])
+def test_timestep_on_partial_tiles(dims):
+    g = _medium(dims, sources=1)
+    grid, _, r = parity.run_gpu(g, "fp32_mixed")
+    for kw in (dict(dt_max=1e16, tau_front=0.02), dict(dt_max=1e16, tau_front=0.0), dict(dt_max=1e16, tau_front=0.02)):
+        want = timestep.rt_timestep(tuple(dims), g["box_len_cm"] / dims[0], g["n_H"], r["x_HI"],
+                                    np.asarray(r["kph"], dtype=np.float64), **kw)
+        assert native.rt_timestep(grid.h, **kw) == pytest.approx(want, rel=1e-5)
+    grid.close()
