@@ -112,6 +112,20 @@ __device__ __forceinline__ double f32_widen_bits(float f) {
 }
 // hi + lo rounded to binary64 with one FP64 addition.
 __device__ __forceinline__ double f2_to_double_bits(F2 a) { return __dadd_rn(f32_widen_bits(a.hi), f32_widen_bits(a.lo)); }
+// Chopped FP32 value of a double (relative error below 2^-23; below the FP32
+// normal range: 0), and an FP32 number as a double (subnormals: 0), by moving
+// the fields: for corrections that are themselves only good to FP32.
+__device__ __forceinline__ float f32_chop(double v) {
+  const int hi = __double2hiint(v);
+  const int e = ((hi >> 20) & 0x7ff) - 896;
+  const unsigned m = ((unsigned)e << 23) | ((unsigned)(hi & 0xfffff) << 3) | ((unsigned)__double2loint(v) >> 29);
+  return __uint_as_float(((unsigned)hi & 0x80000000u) | (e > 0 ? m : 0u));
+}
+__device__ __forceinline__ double f64_wide(float f) {
+  const unsigned b = __float_as_uint(f);
+  const unsigned hi = (b & 0x80000000u) | ((((b >> 23) & 0xffu) + 896u) << 20) | ((b & 0x7fffffu) >> 3);
+  return (b & 0x7f800000u) ? __hiloint2double((int)hi, (int)(b << 29)) : 0.0;
+}
 __device__ __forceinline__ float f2_to_float(F2 a) { return __fadd_rn(a.hi, a.lo); }
 // a + b rounded to FP32: f2_to_float(f2_add(a, b)) without the final
 // renormalisation (the same value)

@@ -92,3 +92,36 @@ def test_timestep_on_partial_tiles(dims):
                                     np.asarray(r["kph"], dtype=np.float64), **kw)
         assert native.rt_timestep(grid.h, **kw) == pytest.approx(want, rel=1e-5)
     grid.close()
+
+
+@pytest.mark.parametrize("batched", [False, True])
+def test_fp64_update_over_its_whole_range(batched):
+    """Fractions, rates and densities inside and outside the range of the FP64
+    update's FP32 guesses.  Each of the 10 substeps rounds by at most five
+    units of 2^-53 on either side."""
+    import oracle
+    dims = (24, 20, 18)
+    n = int(np.prod(dims))
+    g = _medium(dims)
+    rng = np.random.default_rng(6)
+    small = 10.0 ** rng.uniform(-40, -0.31, n)
+    x_small = rng.random(n) < 0.5
+    g["x_HI"] = np.where(x_small, small, 1.0 - small)
+    g["x_HII"] = np.where(x_small, 1.0 - small, small)
+    g["n_H"] = 10.0 ** rng.uniform(-8, 12, n)
+    k = np.where(rng.random(n) < 0.1, 0.0, 10.0 ** rng.uniform(-45, 8, n))
+    grid = native.Grid(parity.ctx(), g, "fp64")
+    native.rt_set_rates(grid.h, k, np.zeros(n))
+    if batched:
+        b = native.Batch(parity.ctx())
+        b.add(grid)
+        b.chem(synth.MYR_S, 10, synth.ALPHA_B)
+    else:
+        grid.chem(synth.MYR_S, 10, synth.ALPHA_B)
+    x_o, z_o = oracle.chem(g["n_H"], g["x_HI"], g["x_HII"], k, synth.MYR_S, 10, synth.ALPHA_B)
+    tol = 2 * 10 * 5 * 2.0 ** -53
+    np.testing.assert_allclose(grid.rates()["x_HI"], x_o, rtol=tol, atol=0)
+    np.testing.assert_allclose(grid.x_HII(), z_o, rtol=tol, atol=0)
+    if batched:
+        b.close()
+    grid.close()
