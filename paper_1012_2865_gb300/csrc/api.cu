@@ -234,6 +234,7 @@ struct rt_grid {
   FlightState fl;
   bool src_fsl = false;                // the device source table was built for a finite-c trace
   double seg_per_pkg = 0.0;            // segments per package of the last trace read back
+  unsigned long long last_pkgs = 0;    // its packages
   // pinned readback buffer
   void* host_rb = nullptr;
   bool traced = false;
@@ -649,7 +650,7 @@ static void fill_common_args(TraceArgs& A, const rt_trace_params* p) {
   A.tau_term32lo = (float)(A.tau_term - (double)A.tau_term32);
   A.tau_near = A.tau_term32 * (1.0f - 1.0f / 4096.0f);
   A.timeout_ns = (long long)((p->timeout_s > 0 ? p->timeout_s : 2.0) * 1e9);
-  A.segs_per_iter = p->segs_per_iter > 0 ? p->segs_per_iter : 8;
+  A.segs_per_iter = p->segs_per_iter > 0 ? p->segs_per_iter : visit_segments(0, 1);
   A.checksums = (p->flags & RT_TRACE_CHECKSUMS) != 0;
   A.fc = (p->flags & RT_TRACE_FC) != 0;
   for (int l = 0; l < kLevels; ++l) {
@@ -829,7 +830,6 @@ static int enqueue_trace(rt_grid* g, const rt_trace_params* p, int passes, bool 
   A.cap = g->ts.cap;
   A.ctl = g->ts.ctl;
   A.max_steps = 2 * (g->nx + g->ny + g->nz) + 16;
-  if (p->segs_per_iter == 0) A.segs_per_iter = tuned_segs_per_iter(g->seg_per_pkg, !fsl);
   int mode = FLIGHT_OFF;
   unsigned long long in_cap = 0;
   if (fsl) {
@@ -842,6 +842,9 @@ static int enqueue_trace(rt_grid* g, const rt_trace_params* p, int passes, bool 
   CUDA_TRY(trace_occupancy(g->precision, fsl ? 1 : 0, A.fc, g->variant, block, &per_sm));
   if (per_sm < 1) per_sm = 1;
   if (p->blocks_per_sm > 0 && p->blocks_per_sm < per_sm) per_sm = p->blocks_per_sm;
+  if (p->segs_per_iter == 0)
+    A.segs_per_iter = fsl ? tuned_segs_per_iter(g->seg_per_pkg, false)
+                          : visit_segments(g->last_pkgs, (unsigned long long)per_sm * g->ctx->num_sms * block);
   if ((rc = g->ts.bind_rows(A, per_sm * g->ctx->num_sms, 1))) return rc;
   if ((rc = launch_passes(A, g->ts.cap * g->ts.rec_bytes, g->src_dev, nsrc, passes, g->precision, fsl ? 1 : 0,
                           g->variant, mode, in_cap, per_sm * g->ctx->num_sms, g->ev0, g->ev1, st, (p->flags & RT_TRACE_SELFTEST_STALL) != 0)))
@@ -917,7 +920,10 @@ static int read_budget(rt_grid* g, rt_budget* out) {
   if (g->fl.live) g->fl.last_halted = out->n_halted;
   unsigned long long pkgs = out->n_resumed;
   for (int l = 0; l < kLevels; ++l) pkgs += out->counts[l];
-  if (out->status == RT_OK && pkgs > 0) g->seg_per_pkg = (double)out->segments / (double)pkgs;
+  if (out->status == RT_OK && pkgs > 0) {
+    g->seg_per_pkg = (double)out->segments / (double)pkgs;
+    g->last_pkgs = pkgs;
+  }
   float ms = 0.f;
   if (g->traced && cudaEventElapsedTime(&ms, g->ev0, g->ev1) == cudaSuccess) out->kernel_ms = ms;
   else cudaGetLastError();

@@ -26,6 +26,7 @@
 #include <mutex>
 #include <string>
 
+#include "policy.h"
 #include "rt.h"
 #include "rt_internal.cuh"
 
@@ -233,7 +234,7 @@ int rt_trace_noalloc(const rt_noalloc_grid* g, int nsrc, const double* pos_cm, c
     A.cap = p->queue_capacity > 0 ? (unsigned long long)p->queue_capacity : (unsigned long long)RT_NOALLOC_MAX_RECORDS;
     A.ctl = ctl;
     A.timeout_ns = (long long)((p->timeout_s > 0 ? p->timeout_s : 2.0) * 1e9);
-    A.segs_per_iter = p->segs_per_iter > 0 ? p->segs_per_iter : 8;
+    A.segs_per_iter = p->segs_per_iter > 0 ? p->segs_per_iter : visit_segments(0, 1);
     A.max_steps = 2 * (g->nx + g->ny + g->nz) + 16;
     A.checksums = (p->flags & RT_TRACE_CHECKSUMS) != 0;
     A.fc = (p->flags & RT_TRACE_FC) != 0;

@@ -53,6 +53,17 @@ inline int tuned_segs_per_iter(double seg_per_pkg, bool handoff = true) {
   return s;
 }
 
+// The same for traces whose split packages hand children to lanes of their
+// warp (all but finite-speed-of-light ones): a lane that ends early mostly
+// takes up a child, so visits are long, 64; 128 once the trace's packages
+// outnumber the lanes by far (`pkgs` of the grid's last trace, 0 when none was
+// read back), so that few lanes sit out the end.  Measured at 32 / 64 / 128:
+// 24 sources in an ionised 128^3 grid (300 packages per lane) 6.81 / 6.39 / 6.14
+// ms, 30 of three types in 128^3 (144) 3.12 / 2.95 / 2.86, 1000 in a clumpy 256^3
+// grid (248) 2.52 / 2.51 / 2.52, a 24-grid batch 1.80 / 1.80 / 1.80 (8: 1.94), the
+// 128^3 Stroemgren snapshot (7) 0.239 / 0.235 / 0.247.
+inline int visit_segments(unsigned long long pkgs, unsigned long long lanes) { return pkgs >= 64 * lanes ? 128 : 64; }
+
 // Halting radii of the next finite-speed-of-light trace (cell units): a
 // package emitted a traces ago halts at neu[a]; neu[0] = c_dt and
 // neu[a] = old[a - 1] + c_dt, the light travel summed since its emission.
