@@ -38,9 +38,12 @@ __device__ __forceinline__ float f2_diff(F2 a, F2 b) {
 }
 __device__ __forceinline__ bool f2_less(F2 a, F2 b) { return a.hi < b.hi || (a.hi == b.hi && a.lo < b.lo); }
 __device__ __forceinline__ bool f2_eq(F2 a, F2 b) { return a.hi == b.hi && a.lo == b.lo; }
-// 1 / (n.hi + n.lo) as a pair (one Newton correction)
+// 1 / (n.hi + n.lo) as a pair: the approximate reciprocal (2^-23), one Newton
+// step in FP32, one for the low part (|n| in the normal range's middle, as
+// direction components are)
 __device__ __forceinline__ F2 f2_recip(F2 n) {
-  const float q = __frcp_rn(n.hi);
+  const float q0 = __fdividef(1.0f, n.hi);
+  const float q = fmaf(fmaf(-n.hi, q0, 1.0f), q0, q0);
   float e = fmaf(-n.hi, q, 1.0f);
   e = fmaf(-n.lo, q, e);
   return fast_two_sum(q, __fmul_rn(e, q));

@@ -457,9 +457,9 @@ struct Walk64 {
 // level0 is pix >> 2 (level - level0); at each split the lineage continues
 // with the child on the path to pix.  If the lineage does not
 // reach that cell at that level (returns NaN; the caller then keeps its FP32
-// decision).  Takes values only, like decide64.
-__device__ __noinline__ double retrace_tau64(const TraceArgs& A, uint32_t src, int level, uint32_t pix, int tc0,
-                                             int tc1, int tc2) {
+// decision).
+__device__ __forceinline__ double retrace_tau64(const TraceArgs& A, uint32_t src, int level, uint32_t pix, int tc0,
+                                                int tc1, int tc2) {
   const SourceDev& S = A.src[src];
   const InstDev& I = A.inst[S.inst];
   const double s0 = S.s[0], s1 = S.s[1], s2 = S.s[2];
@@ -570,11 +570,10 @@ __device__ __forceinline__ int dir_pair(const TraceArgs& A, int level, uint32_t 
 // Exact (FP64) crossing decision for cell (c0, c1, c2) of package (level,
 // pix) of source src: bit 3 = split, bits 0-2 = axes that reach the next
 // plane first, bit 6 = the crossing lies beyond the halting radius rlim
-// (+inf without a finite speed of light).  A free function taking values,
-// so that calling it does not force the caller's walker state into local
-// memory.
-__device__ __noinline__ int decide64(const TraceArgs& A, uint32_t src, int level, uint32_t pix, int c0, int c1,
-                                     int c2, double rlim) {
+// (+inf without a finite speed of light).  Inlined where it is used once: as a
+// call it cost the kernel's caller-saved registers (28 spilled words).
+__device__ __forceinline__ int decide64(const TraceArgs& A, uint32_t src, int level, uint32_t pix, int c0, int c1,
+                                        int c2, double rlim) {
   const SourceDev& S = A.src[src];
   double n[3];
   pix2vec64(level, pix, n);
@@ -729,7 +728,7 @@ struct Walk32 {
   template <bool FSL>
   __device__ __forceinline__ bool start(const TraceArgs& A, LaneAcc& acc, bool given, uint32_t cell) {
     const SourceDev& S = A.src[src];
-    const InstDev& I = A.inst[S.inst];
+    const InstDev& I = A.inst[A.ninst == 1 ? 0 : S.inst];  // (one dependent load less)
     const float4 sh = __ldg(&S.s32);
     const float4 sl = __ldg(&S.slo32);
     acc.Pstart = P;
@@ -748,9 +747,20 @@ struct Walk32 {
       c1 = (int)((cell / (uint32_t)nx) % (uint32_t)ny);
       c2 = (int)(cell / ((uint32_t)nx * (uint32_t)ny));
     } else {
-      c0 = cell_of(f2_add(F2{sh.x, sl.x}, f2_mul(r, n[0])), n[0].hi);
-      c1 = cell_of(f2_add(F2{sh.y, sl.y}, f2_mul(r, n[1])), n[1].hi);
-      c2 = cell_of(f2_add(F2{sh.z, sl.z}, f2_mul(r, n[2])), n[2].hi);
+      // the point in FP32 where that is clear of every plane by more than its
+      // error, else as pairs
+      const float u0 = fmaf(r.hi, n[0].hi, sh.x), u1 = fmaf(r.hi, n[1].hi, sh.y), u2 = fmaf(r.hi, n[2].hi, sh.z);
+      const float f0 = floorf(u0), f1 = floorf(u1), f2 = floorf(u2);
+      const float far = fmaxf(fabsf(u0 - f0 - 0.5f), fmaxf(fabsf(u1 - f1 - 0.5f), fabsf(u2 - f2 - 0.5f)));
+      if (far < 0.5f - 8.0f * kEps32 * (r.hi + fmaxf(sh.x, fmaxf(sh.y, sh.z)))) {
+        c0 = (int)f0;
+        c1 = (int)f1;
+        c2 = (int)f2;
+      } else {
+        c0 = cell_of(f2_add(F2{sh.x, sl.x}, f2_mul(r, n[0])), n[0].hi);
+        c1 = cell_of(f2_add(F2{sh.y, sl.y}, f2_mul(r, n[1])), n[1].hi);
+        c2 = cell_of(f2_add(F2{sh.z, sl.z}, f2_mul(r, n[2])), n[2].hi);
+      }
       if (c0 < 0 || c0 >= nx || c1 < 0 || c1 >= ny || c2 < 0 || c2 >= nz) return false;
     }
     idx = c0 + nx * (c1 + ny * c2);
@@ -771,14 +781,14 @@ struct Walk32 {
     if (!PAIR) G = (float*)I.G;
     const float4 k32 = __ldg(&S.k32);  // sdx, w, rw, heat
     sdx = k32.x; sdx_lo = sl.w; w = k32.y; heat = k32.w;
-    // Radii before and after which the next crossing cannot / must need the
-    // full decision: the exit plane of each axis (its distance from the
-    // source in FP32, widened by the rounding of s and of the product), the
-    // split radius and the halting radius.
-    float lo = kFar, hi = kFar;
-    exit_of(a0, n[0].hi < 0.0f ? sh.x : (float)nx - sh.x, (float)nx, lo, hi);
-    exit_of(a1, n[1].hi < 0.0f ? sh.y : (float)ny - sh.y, (float)ny, lo, hi);
-    exit_of(a2, n[2].hi < 0.0f ? sh.z : (float)nz - sh.z, (float)nz, lo, hi);
+    // The radius below which no crossing splits, leaves the box or halts: the
+    // exit plane of each axis (its distance from the source in FP32, less the
+    // rounding of s and of the product), the split and the halting radius;
+    // and a bound on the radius for the error of tau.
+    float lo = exit_of(a0, n[0].hi < 0.0f ? sh.x : (float)nx - sh.x, (float)nx);
+    lo = fminf(lo, exit_of(a1, n[1].hi < 0.0f ? sh.y : (float)ny - sh.y, (float)ny));
+    lo = fminf(lo, exit_of(a2, n[2].hi < 0.0f ? sh.z : (float)nz - sh.z, (float)nz));
+    float hi = (float)nx + (float)ny + (float)nz;
     const int l = lvl();
     if (l < A.max_level) {
       lo = fminf(lo, A.rsplit32[l]);
@@ -792,12 +802,8 @@ struct Walk32 {
         4.1f * fmaxf(sa.x * a0.iv.hi, fmaxf(sa.y * a1.iv.hi, sa.z * a2.iv.hi));
     return true;
   }
-  __device__ __forceinline__ static void exit_of(const Axis<EXACT>& a, float d, float dim, float& lo, float& hi) {
-    const float m = dim * (8.0f * kEps32);
-    if (a.iv.hi > 0.0f) {
-      lo = fminf(lo, (d - m) * a.iv.hi);
-      hi = fminf(hi, (d + m) * a.iv.hi);
-    }
+  __device__ __forceinline__ static float exit_of(const Axis<EXACT>& a, float d, float dim) {
+    return a.iv.hi > 0.0f ? fmaf(dim, -8.0f * kEps32, d) * a.iv.hi : kFar;
   }
   __device__ __forceinline__ void set_rlim(const TraceArgs& A) {
     if ((int)age < A.n_ages) {
