@@ -115,6 +115,18 @@ __device__ __forceinline__ double f32_widen_bits(float f) {
 }
 // hi + lo rounded to binary64 with one FP64 addition.
 __device__ __forceinline__ double f2_to_double_bits(F2 a) { return __dadd_rn(f32_widen_bits(a.hi), f32_widen_bits(a.lo)); }
+// 1 / v and 1 / sqrt(v) to ~2^-23, v in the normal range (no fix-up of
+// subnormal operands)
+__device__ __forceinline__ float rcp_approx(float v) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+  return r;
+}
+__device__ __forceinline__ float rsqrt_approx(float v) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+  return r;
+}
 // Chopped FP32 value of a double (relative error below 2^-23; below the FP32
 // normal range: 0), and an FP32 number as a double (subnormals: 0), by moving
 // the fields: for corrections that are themselves only good to FP32.
