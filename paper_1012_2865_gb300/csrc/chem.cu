@@ -165,10 +165,10 @@ __global__ void chem_kernel(long long ncell, const double* __restrict__ nH, doub
 // instructions a substep (their operands change where a cell changes form),
 // the residual's pairs are only renormalised where that shows in the result,
 // and the Newton step's quotient is an approximate reciprocal with one
-// residual: 128^3 cells, 10 substeps, the
-// whole call 102 -> 70 us.  Over 10 substeps the error
-// against 113 bits is 4.2e-13 at most and 6.0e-15 on average in x_HI, 5.1e-13
-// and 4.9e-15 in x_HII (4.2e-13, 6.0e-15, 1.5e-12 and 4.9e-15 before).
+// residual: 128^3 cells, 10 substeps, the whole call 102 -> 70 us.  Over 10
+// substeps the error against 113 bits is 4.2e-13 at most and 6.0e-15 on average
+// in x_HI, 5.1e-13 and 4.9e-15 in x_HII (4.2e-13, 6.0e-15, 1.5e-12 and 4.9e-15
+// before).
 //
 // Same backward-Euler step for the FP32-mixed path, solved by FP32 + one
 // Newton correction: the smaller fraction is first obtained in FP32 from its
@@ -199,6 +199,19 @@ __global__ void chem_mixed_kernel(long long ncell, const double* __restrict__ nH
   }
 }
 
+// Range tests on the bit patterns (FP64 comparisons run on the FP64 pipe and
+// bound the kernels that make them; with these tests a 256^3 check takes 24
+// instead of 69 us, its commit 118 instead of 162): a finite
+// number >= 0, a number in [0, 1] (either zero included).
+__device__ __forceinline__ bool good_density(double v) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(v);
+  return u < 0x7FF0000000000000ULL || u == 0x8000000000000000ULL;
+}
+__device__ __forceinline__ bool good_fraction(double v) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(v);
+  return u <= 0x3FF0000000000000ULL || u == 0x8000000000000000ULL;
+}
+
 template <typename NT>
 __global__ void refresh_nhi_kernel(long long ncell, const double* __restrict__ nH,
                                    const double* __restrict__ xHI, NT* __restrict__ nhi) {
@@ -213,7 +226,7 @@ __global__ void refresh_nhi_pair_kernel(long long ncell, const double* __restric
                                         const double* __restrict__ xHI, float2* __restrict__ nhi) {
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < ncell;
        c += (long long)gridDim.x * blockDim.x) {
-    const F2 v = f2_from_double(__dmul_rn(nH[c], xHI[c]));
+    const F2 v = f2_from_double_bits(__dmul_rn(nH[c], xHI[c]));
     nhi[c] = make_float2(v.hi, v.lo);
   }
 }
@@ -222,7 +235,7 @@ __global__ void refresh_nhi_pair_kernel(long long ncell, const double* __restric
 __global__ void pair_kernel(long long ncell, const double* __restrict__ src, float2* __restrict__ dst) {
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < ncell;
        c += (long long)gridDim.x * blockDim.x) {
-    const F2 v = f2_from_double(src[c]);
+    const F2 v = f2_from_double_bits(src[c]);
     dst[c] = make_float2(v.hi, v.lo);
   }
 }
@@ -231,7 +244,7 @@ __global__ void pair_kernel(long long ncell, const double* __restrict__ src, flo
 __global__ void check_density_kernel(long long n, const double* __restrict__ a, unsigned long long* __restrict__ bad) {
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n; c += (long long)gridDim.x * blockDim.x) {
     const double v = a[c];
-    if (!(v >= 0.0) || isinf(v)) atomicMin(bad, (unsigned long long)c);
+    if (!good_density(v)) atomicMin(bad, (unsigned long long)c);
   }
 }
 
@@ -243,12 +256,22 @@ __global__ void convert_kernel(long long n, const ST* __restrict__ src, double* 
 }
 
 // Gamma of an FP32-mixed grid, eV/s, in erg/s as FP32: the product with scale
-// as an FP32 pair, rounded (the FP64 pipe is a small fraction of the FP32 one);
-// results near or below the FP32 normal range through FP64.
+// as an FP32 pair, rounded (the FP64 pipe is a small fraction of the FP32 one).
+// Small results (an optically thick cell's) would lose the product's low part
+// below the FP32 range and are formed 2^64 times larger; results below the
+// FP32 normal range go through FP64, out of line so that its instructions are
+// not predicated into every cell.
+__device__ __noinline__ float scale64(float v, double scale) { return (float)((double)v * scale); }
 __device__ __forceinline__ float scale32(float v, double scale, float sh, float sl) {
-  const float p = __fmul_rn(v, sh);
-  if (fabsf(p) < 1e-30f) return v == 0.0f ? 0.0f : (float)((double)v * scale);
-  return __fadd_rn(p, fmaf(v, sl, fmaf(v, sh, -p)));
+  float p = __fmul_rn(v, sh), up = 1.0f;
+  if (fabsf(p) < 1e-30f) {
+    if (v == 0.0f) return 0.0f;
+    if (fabsf(p) < 2.4e-38f || sh < 1e-20f) return scale64(v, scale);
+    v *= 18446744073709551616.0f;  // 2^64
+    p = __fmul_rn(v, sh);
+    up = 5.4210108624275222e-20f;  // 2^-64
+  }
+  return __fmul_rn(__fadd_rn(p, fmaf(v, sl, fmaf(v, sh, -p))), up);
 }
 // k_ph, Gamma (times scale) and x_HI for the caller, each where its output is
 // given.  MIXED: kg holds (k_ph, Gamma) pairs, else K and G are FP64 arrays.
@@ -272,6 +295,38 @@ __global__ void read_rates_kernel(long long n, const void* __restrict__ K, const
     if (ox) ox[c] = (DT)x[c];
   }
 }
+// The FP32 outputs of an FP32-mixed grid four cells at a time (16-byte
+// accesses), for 16-byte aligned outputs; the last n % 4 cells by block 0.
+// Bound by memory: 28 bytes a cell, 71 us for 256^3 (6.6 TB/s).
+// One cell a thread with FP64 conversions and products took 140 us, the FP64
+// pipe's time.
+__global__ void read_rates4_kernel(long long n, const float2* __restrict__ kg, const double* __restrict__ x,
+                                   float* __restrict__ ok, float* __restrict__ og, float* __restrict__ ox,
+                                   double scale) {
+  const float sh = (float)scale, sl = (float)(scale - (double)sh);
+  const long long n4 = n / 4;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n4; i += (long long)gridDim.x * blockDim.x) {
+    if (ok || og) {
+      const float4 a = ((const float4*)kg)[2 * i], b = ((const float4*)kg)[2 * i + 1];
+      if (ok) ((float4*)ok)[i] = make_float4(a.x, a.z, b.x, b.z);
+      if (og)
+        ((float4*)og)[i] = make_float4(scale32(a.y, scale, sh, sl), scale32(a.w, scale, sh, sl),
+                                       scale32(b.y, scale, sh, sl), scale32(b.w, scale, sh, sl));
+    }
+    if (ox) {
+      const double2 u = ((const double2*)x)[2 * i], v = ((const double2*)x)[2 * i + 1];
+      ((float4*)ox)[i] = make_float4(f2_from_double_bits(u.x).hi, f2_from_double_bits(u.y).hi,
+                                     f2_from_double_bits(v.x).hi, f2_from_double_bits(v.y).hi);
+    }
+  }
+  const long long c = 4 * n4 + threadIdx.x;
+  if (blockIdx.x == 0 && c < n) {
+    if (ok) ok[c] = kg[c].x;
+    if (og) og[c] = scale32(kg[c].y, scale, sh, sl);
+    if (ox) ox[c] = f2_from_double_bits(x[c]).hi;
+  }
+}
+
 // The caller's k_ph and Gamma (times scale) into an FP32-mixed grid.
 template <typename ST>
 __global__ void write_rates_kernel(long long n, const ST* __restrict__ k, const ST* __restrict__ g,
@@ -295,10 +350,10 @@ __global__ void check_state_kernel(long long n, const double* __restrict__ nH, c
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n; c += (long long)gridDim.x * blockDim.x) {
     if (nH) {
       const double v = nH[c];
-      if (!(v >= 0.0) || isinf(v)) atomicMin(&bad[0], (unsigned long long)c);
+      if (!good_density(v)) atomicMin(&bad[0], (unsigned long long)c);
     }
     const double xv = x[c];
-    if (!(xv >= 0.0 && xv <= 1.0)) atomicMin(&bad[1], (unsigned long long)c);
+    if (!good_fraction(xv)) atomicMin(&bad[1], (unsigned long long)c);
   }
 }
 
@@ -309,12 +364,12 @@ __global__ void check_state2_kernel(long long n2, const double2* __restrict__ nH
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n2; i += (long long)gridDim.x * blockDim.x) {
     if (nH) {
       const double2 v = nH[i];
-      if (!(v.x >= 0.0) || isinf(v.x)) atomicMin(&bad[0], (unsigned long long)(2 * i));
-      if (!(v.y >= 0.0) || isinf(v.y)) atomicMin(&bad[0], (unsigned long long)(2 * i + 1));
+      if (!good_density(v.x)) atomicMin(&bad[0], (unsigned long long)(2 * i));
+      if (!good_density(v.y)) atomicMin(&bad[0], (unsigned long long)(2 * i + 1));
     }
     const double2 xv = x[i];
-    if (!(xv.x >= 0.0 && xv.x <= 1.0)) atomicMin(&bad[1], (unsigned long long)(2 * i));
-    if (!(xv.y >= 0.0 && xv.y <= 1.0)) atomicMin(&bad[1], (unsigned long long)(2 * i + 1));
+    if (!good_fraction(xv.x)) atomicMin(&bad[1], (unsigned long long)(2 * i));
+    if (!good_fraction(xv.y)) atomicMin(&bad[1], (unsigned long long)(2 * i + 1));
   }
 }
 
@@ -375,7 +430,7 @@ __global__ void commit_state_kernel(long long n, unsigned long long* ctl, unsign
     xHII[c] = sz ? sz[c] : __dsub_rn(1.0, x);
     const double v = __dmul_rn(h, x);
     if (PAIR) {
-      const F2 p = f2_from_double(v);
+      const F2 p = f2_from_double_bits(v);
       ((float2*)nhi)[c] = make_float2(p.hi, p.lo);
     } else {
       ((double*)nhi)[c] = v;
@@ -401,7 +456,7 @@ __global__ void commit_state2_kernel(long long n2, unsigned long long* ctl, unsi
     xHII[i] = sz ? sz[i] : make_double2(__dsub_rn(1.0, x.x), __dsub_rn(1.0, x.y));
     const double v0 = __dmul_rn(h.x, x.x), v1 = __dmul_rn(h.y, x.y);
     if (PAIR) {
-      const F2 p0 = f2_from_double(v0), p1 = f2_from_double(v1);
+      const F2 p0 = f2_from_double_bits(v0), p1 = f2_from_double_bits(v1);
       ((float4*)nhi)[i] = make_float4(p0.hi, p0.lo, p1.hi, p1.lo);
     } else {
       ((double2*)nhi)[i] = make_double2(v0, v1);
@@ -427,11 +482,11 @@ __global__ void check_refresh_kernel(long long n, unsigned long long* __restrict
                                      void* __restrict__ nhi, InstDev* __restrict__ inst) {
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n; c += (long long)gridDim.x * blockDim.x) {
     const double xv = x[c];
-    if (!(xv >= 0.0 && xv <= 1.0)) atomicMin(&ctl[CTL_CHECK_X], (unsigned long long)c);
+    if (!good_fraction(xv)) atomicMin(&ctl[CTL_CHECK_X], (unsigned long long)c);
     if (!z_given) z[c] = __dsub_rn(1.0, xv);
     const double v = __dmul_rn(nH[c], xv);
     if (PAIR) {
-      const F2 p = f2_from_double(v);
+      const F2 p = f2_from_double_bits(v);
       ((float2*)nhi)[c] = make_float2(p.hi, p.lo);
     } else {
       ((double*)nhi)[c] = v;
@@ -458,7 +513,7 @@ __global__ void check_refresh_kernel(long long n, unsigned long long* __restrict
       z[c] = z_old[c];
       const double v = __dmul_rn(nH[c], xv);
       if (PAIR) {
-        const F2 p = f2_from_double(v);
+        const F2 p = f2_from_double_bits(v);
         ((float2*)nhi)[c] = make_float2(p.hi, p.lo);
       } else {
         ((double*)nhi)[c] = v;
@@ -589,6 +644,8 @@ static float4 step_pairs(double h, double alpha) {
   return make_float4(a_hi, (float)(ha - (double)a_hi), h_hi, (float)(h - (double)h_hi));
 }
 
+static bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
+
 static int grid_for(long long n, int block) {
   long long g = (n + block - 1) / block;
   if (g > 152 * 32) g = 152 * 32;
@@ -671,8 +728,6 @@ cudaError_t launch_add_word(unsigned long long* w, unsigned long long delta, cud
   add_word_kernel<<<1, 32, 0, st>>>(w, delta);
   return cudaGetLastError();
 }
-
-static bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
 cudaError_t launch_check_state(long long n, const double* nH, const double* x, unsigned long long* bad,
                                cudaStream_t st) {
@@ -824,6 +879,13 @@ cudaError_t launch_read_rates(int precision, long long n, const void* K, const v
                               void* og, void* ox, int dtype, double scale, cudaStream_t st) {
   const int block = 256, grid = grid_for(n, block);
   const double* g = (const double*)G;
+  // four cells a thread where every array allows 16-byte accesses
+  if (precision == RT_FP32_MIXED && dtype == RT_DTYPE_F32 && aligned16(K) && aligned16(x) && aligned16(ok) &&
+      aligned16(og) && aligned16(ox)) {
+    read_rates4_kernel<<<grid_for(n / 4, block), block, 0, st>>>(n, (const float2*)K, x, (float*)ok, (float*)og,
+                                                                 (float*)ox, scale);
+    return cudaGetLastError();
+  }
   if (precision == RT_FP64) {
     if (dtype == RT_DTYPE_F64)
       read_rates_kernel<false, double><<<grid, block, 0, st>>>(n, K, g, x, (double*)ok, (double*)og, (double*)ox, scale);

@@ -73,33 +73,32 @@ __device__ __forceinline__ double f2_to_double(F2 a) { return __dadd_rn((double)
 // arithmetic (IEEE-754 binary64 / binary32 fields), for kernels where the
 // FP64 pipe, a small fraction of the FP32 one, would otherwise bound them.
 //
-// Nearest pair to v: hi = v rounded to 24 bits (ties to even) by adding the
-// rounding bias to the binary64 pattern (a carry moves into the exponent as
-// it should); v - hi is then the difference of the two patterns, an integer
-// of at most 2^28 units of v's last place, and lo its FP32 rounding.  Equal
-// to f2_from_double for zeros and 2^-74 <= |v| < 2^125, which it handles
-// this way (hi and lo stay normal FP32 numbers); other values take
-// f2_from_double.
+// Nearest pair to v: hi = v rounded to 24 bits (ties to even; a carry moves
+// into the exponent as it should), lo the FP32 rounding of v - hi, an integer
+// of at most 2^28 units of v's last place.  Equal to f2_from_double for zeros
+// and 2^-74 <= |v| < 2^125, which it handles this way (hi and lo stay normal
+// FP32 numbers); other values take f2_from_double.  All in 32-bit words:
+// 64-bit integer additions share the FP64 pipe here, and it bound the kernels
+// that convert a field (a 256^3 read of the rates: 102 -> 71 us without them).
 // The rare operands of these conversions go through functions that are
 // never inlined, so the compiler cannot predicate their FP64 instructions
 // into the common path.
 static __device__ __noinline__ F2 f2_from_double_call(double v) { return f2_from_double(v); }
 static __device__ __noinline__ double f32_widen_call(float f) { return (double)f; }
 __device__ __forceinline__ F2 f2_from_double_bits(double v) {
-  const unsigned long long u = (unsigned long long)__double_as_longlong(v);
-  const unsigned uh = (unsigned)(u >> 32);
-  const unsigned long long mag = u & 0x7fffffffffffffffULL;
-  if (mag == 0ULL) return {__uint_as_float(uh & 0x80000000u), 0.0f};  // signed zero
-  const int e = (int)((uh >> 20) & 0x7ffu);  // biased binary64 exponent
-  if (e < 949 || e > 1147) return f2_from_double_call(v);
-  const unsigned long long r = (mag + 0x0fffffffULL + ((mag >> 29) & 1ULL)) & ~0x1fffffffULL;
-  const long long d = (long long)(mag - r);  // |v| - |hi|, units of 2^(e - 1075)
-  const unsigned rh = (unsigned)(r >> 32), rl = (unsigned)r;
-  const unsigned sign = uh & 0x80000000u;
-  const unsigned hb = sign | ((((rh >> 20) & 0x7ffu) - 896u) << 23) | ((rh & 0xfffffu) << 3) | (rl >> 29);
-  const float scale = __uint_as_float((unsigned)(e - 948) << 23);  // 2^(e - 1075)
-  const float lo = __fmul_rn(__int2float_rn((int)d), scale);  // |d| <= 2^28
-  return {__uint_as_float(hb), sign ? -lo : lo};
+  const unsigned uh = (unsigned)__double2hiint(v), ul = (unsigned)__double2loint(v);
+  const unsigned mh = uh & 0x7fffffffu, sign = uh & 0x80000000u;
+  if (mh - (949u << 20) >= (199u << 20)) {  // outside 2^-74 .. 2^125
+    if ((mh | ul) == 0u) return {__uint_as_float(sign), 0.0f};  // signed zero
+    return f2_from_double_call(v);
+  }
+  unsigned m = ((mh - (896u << 20)) << 3) | (ul >> 29);
+  const unsigned rem = ul & 0x1fffffffu;
+  const bool up = rem > 0x10000000u - (m & 1u);
+  m += up;
+  const int d = (int)rem - (up ? 0x20000000 : 0);  // |v| - |hi|, units of 2^(e - 1075)
+  const float lo = __fmul_rn(__int2float_rn(d), __uint_as_float(((mh >> 20) - 948u) << 23));  // |d| <= 2^28
+  return {__uint_as_float(sign | m), sign ? -lo : lo};
 }
 // An FP32 number widened to binary64 exactly by moving its fields (normal
 // numbers and zeros; others take the conversion instruction).

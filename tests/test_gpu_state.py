@@ -83,6 +83,30 @@ def test_rates_round_trip(precision):
     grid.close()
 
 
+@pytest.mark.parametrize("skip", [0, 1, 4])
+@pytest.mark.parametrize("dims", [(3, 1, 1), (4, 1, 1), (5, 3, 7), (6, 8, 9)])
+def test_fp32_rates_at_each_alignment(dims, skip):
+    """Four cells a thread leave a remainder of 0 to 3, and an output may start
+    off a 16-byte boundary.  k_ph is FP32 in the grid; Gamma leaves FP32 eV/s
+    through an FP32 pair product instead of FP64: one FP32 rounding apart, or
+    the smallest FP32 number where it is subnormal."""
+    import torch
+    n = int(np.prod(dims))
+    grid = native.Grid(parity.ctx(), _medium(dims), "fp32_mixed")
+    rng = np.random.default_rng(3)
+    native.rt_set_rates(grid.h, synth.round_f32(10.0 ** rng.uniform(-30, -8, n)), 10.0 ** rng.uniform(-47, -20, n))
+    want = grid.rates()
+    out = torch.full((3, n + 8), -7.0, dtype=torch.float32, device="cuda")
+    native.rt_get_rates_async(grid.h, *(out[q, skip:skip + n] for q in range(3)), dtype=native.RT_DTYPE_F32)
+    native.rt_synchronize(grid.h)
+    got = out.cpu().numpy()
+    assert (got[:, :skip] == -7.0).all() and (got[:, skip + n:] == -7.0).all()
+    np.testing.assert_array_equal(got[0, skip:skip + n], want["kph"].astype(np.float32))
+    np.testing.assert_allclose(got[1, skip:skip + n], want["gamma"], rtol=2.0 ** -23, atol=1.5e-45)
+    np.testing.assert_array_equal(got[2, skip:skip + n], want["x_HI"].astype(np.float32))
+    grid.close()
+
+
 @pytest.mark.parametrize("dims", [(1, 1, 1), (32, 8, 8), (33, 9, 9), (31, 7, 17), (3, 40, 2), (70, 1, 5)])
 def test_timestep_on_partial_tiles(dims):
     g = _medium(dims, sources=1)
