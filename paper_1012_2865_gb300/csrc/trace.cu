@@ -160,7 +160,7 @@ __device__ __forceinline__ void acc_switch(LaneAcc& a, unsigned& nseg, int inst,
 }
 
 // A warp's state while it has nothing to trace: the outstanding count last
-// seen, when it was first seen, and how long to sleep (ns; doubles up to 4 us).
+// seen, when it was first seen, and how long to sleep (ns; doubles up to 1 us).
 struct IdleWarp {
   long long seen_out;
   uint64_t seen_ns;
@@ -1276,39 +1276,55 @@ __global__ void __launch_bounds__(kBlock, MinBlocks) trace_kernel(TraceArgs A) {
     //     and no ticket: in practice the lanes whose package ended in this
     //     round; a lane holding a ticket must stay free to take up the record
     //     that the ticket names), the rest to the queue (slots reserved
-    //     together); finished packages leave the outstanding count.
-    //     One atomic per warp carries both: +3 per split, -1 per finished
-    //     package.  Child j = 3 i + k - 1 of the i-th splitting lane goes to
-    //     the j-th free lane when there is one, else to slot base + j - nin.
+    //     together); finished packages leave the outstanding count, and the
+    //     free lanes that get no child take a ticket.  Child j = 3 i + k - 1 of
+    //     the i-th splitting lane goes to the j-th free lane when there is
+    //     one, else to slot base + j - nin.
+    //     One atomic per warp and counter (the count carries +3 per split, -1
+    //     per finished package), all in flight together: a round waits for
+    //     one trip to L2 where one after the other they took up to two, and
+    //     for none of the count where nothing splits (with the shorter sleeps
+    //     below: 128^3 Stroemgren snapshot 0.241 -> 0.232 ms, 24-grid batch 1.785
+    //     -> 1.767 ms, 8 small grids 0.180 -> 0.173 ms).
     Start fresh = NO_START;  // a package starts in this lane now
     const bool split = (ev == EV_SPLIT);
+    const bool done = ev == EV_DONE;
     const unsigned sm = __ballot_sync(kFull, split);
-    const unsigned dm = __ballot_sync(kFull, ev == EV_DONE);
-    if (sm | dm) {
-      const int leader = __ffs(sm | dm) - 1;
+    const unsigned dm = __ballot_sync(kFull, done);
+    const unsigned fm = __ballot_sync(kFull, !split && (!active || done) && ticket < 0);
+    if (sm | dm | fm) {
       const unsigned nsp = __popc(sm);
-      // (not in the finite-speed-of-light kernel, which spills at the
-      // register cap already: there the hand-off code cost more than it saved)
-      const unsigned fm = FSL ? 0u : __ballot_sync(kFull, !split && (!active || ev == EV_DONE) && ticket < 0);
       const unsigned nfree = __popc(fm);
-      const unsigned nin = nfree < 3u * nsp ? nfree : 3u * nsp;  // children placed in this warp
-      const unsigned nq = 3u * nsp - nin;                         // children through the queue
-      unsigned long long base = 0;
-      if (lane == leader) {
-        // The count must include the children before any child is published,
-        // or a consumer could finish a child and see it reach zero: wait for
-        // the atomic's return value; the publishing lanes' fence follows.
-        const long long delta = 3LL * nsp - (long long)__popc(dm);
-        const unsigned long long o = atomicAdd(&A.ctl[CTL_OUTSTANDING], (unsigned long long)delta);
-        asm volatile("" ::"l"(o) : "memory");
-        if (nq) base = atomicAdd(&A.ctl[CTL_TAIL], (unsigned long long)nq);
+      // (no hand-off in the finite-speed-of-light kernel, which spills at the
+      // register cap already: there that code cost more than it saved)
+      const unsigned nin = FSL ? 0u : (nfree < 3u * nsp ? nfree : 3u * nsp);  // children placed in this warp
+      const unsigned nq = 3u * nsp - nin;                                   // children through the queue
+      unsigned long long base = 0, tick = 0;
+      if (lane == 0) {
+        if (nfree > nin) tick = atomicAdd(&A.ctl[CTL_HEAD], (unsigned long long)(nfree - nin));
+        const unsigned long long delta = (unsigned long long)(3LL * nsp - (long long)__popc(dm));
+        if (sm) {
+          // The count must include the children before any child is published,
+          // or a consumer could finish a child and see it reach zero: wait for
+          // the atomic's return value; the publishing lanes' fence follows.
+          if (nq) base = atomicAdd(&A.ctl[CTL_TAIL], (unsigned long long)nq);
+          const unsigned long long o = atomicAdd(&A.ctl[CTL_OUTSTANDING], delta);
+          asm volatile("" ::"l"(o) : "memory");
+        } else if (dm) {
+          atomicAdd(&A.ctl[CTL_OUTSTANDING], delta);  // not waited for
+        }
       }
       __syncwarp();  // orders the leader's atomics before the lanes' fence
-      base = __shfl_sync(kFull, base, leader);
-      if (ev == EV_DONE) {
+      if (done) {
         active = false;
         ev = EV_NONE;
       }
+      if (nfree > nin) {
+        tick = __shfl_sync(kFull, tick, 0);
+        const unsigned q = __popc(fm & lt_mask);
+        if (((fm >> lane) & 1u) && q >= nin) ticket = (long long)(tick + (q - nin));
+      }
+      if (sm) base = __shfl_sync(kFull, base, 0);
       if (!FSL && nin) {
         const unsigned q = __popc(fm & lt_mask);
         const bool recv = ((fm >> lane) & 1u) && q < nin;
@@ -1356,17 +1372,7 @@ __global__ void __launch_bounds__(kBlock, MinBlocks) trace_kernel(TraceArgs A) {
         fresh = START_CHILD;
       }
     }
-    // (2) idle lanes without a ticket take one (one atomic per warp)
-    const bool want = !active && ticket < 0;
-    const unsigned wm = __ballot_sync(kFull, want);
-    if (wm) {
-      const int leader = __ffs(wm) - 1;
-      unsigned long long base = 0;
-      if (lane == leader) base = atomicAdd(&A.ctl[CTL_HEAD], (unsigned long long)__popc(wm));
-      base = __shfl_sync(kFull, base, leader);
-      if (want) ticket = (long long)(base + __popc(wm & lt_mask));
-    }
-    // (3) turn tickets into packages
+    // (2) turn tickets into packages
     uint32_t cell = 0;
     if (!active && ticket >= 0) {
       const unsigned long long tk = (unsigned long long)ticket;
@@ -1396,7 +1402,7 @@ __global__ void __launch_bounds__(kBlock, MinBlocks) trace_kernel(TraceArgs A) {
         active = true;
       }
     }
-    // (4) start the new packages, wherever they came from (one that starts
+    // (3) start the new packages, wherever they came from (one that starts
     //     outside the box is finished at the next (1))
     __syncwarp();
     if (fresh != NO_START) {
@@ -1414,7 +1420,7 @@ __global__ void __launch_bounds__(kBlock, MinBlocks) trace_kernel(TraceArgs A) {
         ev = EV_DONE;
       }
     }
-    // (5) a warp with nothing to trace checks for the end of the trace
+    // (4) a warp with nothing to trace checks for the end of the trace
     const unsigned am = __ballot_sync(kFull, active);
     if (am == 0) {
       long long outst = 0;
@@ -1435,7 +1441,9 @@ __global__ void __launch_bounds__(kBlock, MinBlocks) trace_kernel(TraceArgs A) {
           idle.seen_out = outst;
           idle.seen_ns = now;
         }
-        idle.backoff = backoff < 4096 ? 2 * backoff : 4096;
+        // (a longer sleep shows as latency where a trace has few packages,
+        // up to a level of the ray tree each; 512 ns was no faster)
+        idle.backoff = backoff < 1024 ? 2 * backoff : 1024;
       }
       __syncwarp();
       __nanosleep(backoff);
@@ -1445,7 +1453,7 @@ __global__ void __launch_bounds__(kBlock, MinBlocks) trace_kernel(TraceArgs A) {
       idle.backoff = 256;
       idle.seen_out = -1;  // the no-progress clock runs over one idle stretch only
     }
-    // (6) trace a few segments
+    // (5) trace a few segments
     if (active && ev == EV_NONE) {
       w.begin_visit();
       for (int it = 0; it < A.segs_per_iter; ++it) {
@@ -1457,7 +1465,7 @@ __global__ void __launch_bounds__(kBlock, MinBlocks) trace_kernel(TraceArgs A) {
     // the warp-wide steps.  (Without this barrier the same kernel ran
     // 7-11 % slower on every workload measured.)
     __syncwarp();
-    // (6b) the decisions that the segments left, for all lanes together: a
+    // (5b) the decisions that the segments left, for all lanes together: a
     //      lane's last segment (split, exit, halt, termination) runs here once
     //      per visit instead of inside the loop whenever one lane needs it
     //      (with the rates interleaved: 24 sources in an ionised 128^3 grid 9.67 ->
@@ -1477,7 +1485,7 @@ __global__ void __launch_bounds__(kBlock, MinBlocks) trace_kernel(TraceArgs A) {
       if (active) ev = w.end_visit(A, acc, ev);
     }
     __syncwarp();
-    // (7) halted packages go to the output store (one atomic per warp);
+    // (6) halted packages go to the output store (one atomic per warp);
     //     from here on they are finished packages
     if (FSL) {
       const unsigned hm = __ballot_sync(kFull, ev == EV_HALT);
