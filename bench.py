@@ -202,14 +202,17 @@ def trace_roofline(precision, segments, pushed, kernel_ms, gamma, red, peaks, pe
     Gamma reduction where photons carry energy above the threshold; per queue
     record one write and one read -- over the kernel's event-timed duration,
     against the measured copy bandwidth.
-    L2 reductions: one k_ph reduction per segment (and one Gamma reduction
-    where photons heat) over the same duration, against the L2-resident
+    L2 reductions: one per segment on the FP32-mixed path, which adds k_ph and
+    Gamma with one two-word reduction (L2 takes those at the rate of single
+    ones), and on the FP64 path one for k_ph and one for Gamma where photons
+    heat, over the same duration, against the L2-resident single-word
     reduction rate the probe measured in this run (`red`, from red_peak; the
     per-package residual deposits and the queue's atomics, a few per cent,
     are left out, so the fraction is a lower bound)."""
     red_b = 8 if precision == "fp64" else 4
-    nred = 2 if gamma else 1
-    alg = segments * (8 + red_b * nred) + pushed * 2 * REC_BYTES[precision]
+    words = 2 if gamma else 1
+    nred = words if precision == "fp64" else 1
+    alg = segments * (8 + red_b * words) + pushed * 2 * REC_BYTES[precision]
     s = kernel_ms / 1e3
     achieved = alg / s / 1e9
     hbm = peaks.get("hbm_gbs", 6800.0)

@@ -515,8 +515,10 @@ __device__ __forceinline__ double retrace_tau64(const TraceArgs& A, uint32_t src
 // either comparison or whose two nearest planes lie within 2^-20 of each
 // other.  Source constants sit in registers; what only a package's end needs
 // sits in shared memory.  With the decisions in full at every segment the
-// trace of the 128^3 Stroemgren snapshot took 0.41 ms, now 0.30 ms; 24 sources in an
-// ionised 128^3 grid 13.2 -> 9.6 ms; 1000 in a clumpy 256^3 grid 3.9 -> 3.3 ms.
+// trace of the 128^3 Stroemgren snapshot took 0.41 instead of 0.30 ms, 24 sources
+// in an ionised 128^3 grid 13.2 instead of 9.6 ms, 1000 in a clumpy 256^3 grid 3.9
+// instead of 3.3 ms; with the figures given at the steps below they take
+// 0.23, 6.05 and 2.49 ms.
 //
 // Each decision that shapes the ray tree -- which cell plane is crossed next,
 // whether the package splits, whether it terminates -- is taken from the
