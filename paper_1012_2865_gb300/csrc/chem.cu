@@ -77,9 +77,8 @@ __device__ __forceinline__ bool is_neutral(double x, double z) {
 // One cell, FP32-mixed path: FP32 solution + one double-float Newton
 // correction per substep (see chem_mixed_kernel).  x, z and n arrive and
 // leave in FP64 (converted through their bit fields, off the FP64 pipe); in
-// between, the smaller of the two fractions is carried as a double-float
-// pair s and the larger only as its FP32 complement until a substep needs it
-// as a pair.  ha and h2 are h alpha_B and h as pairs.  Returns
+// between, only the smaller of the two fractions is carried, as a double-float
+// pair s.  ha and h2 are h alpha_B and h as pairs.  Returns
 // n_HI = n_H x_HI as a pair.
 __device__ __forceinline__ F2 chem_cell_mixed(double& x, double& z, double n, float kc, F2 ha, F2 h2, int nsub) {
   const F2 n2 = f2_from_double_bits(n);

@@ -36,7 +36,6 @@ __device__ __forceinline__ float f2_diff(F2 a, F2 b) {
   const F2 d = two_sum(a.hi, -b.hi);
   return __fadd_rn(d.hi, __fadd_rn(d.lo, __fsub_rn(a.lo, b.lo)));
 }
-__device__ __forceinline__ bool f2_less(F2 a, F2 b) { return a.hi < b.hi || (a.hi == b.hi && a.lo < b.lo); }
 __device__ __forceinline__ bool f2_eq(F2 a, F2 b) { return a.hi == b.hi && a.lo == b.lo; }
 // 1 / (n.hi + n.lo) as a pair: the approximate reciprocal (2^-23), one Newton
 // step in FP32, one for the low part (|n| in the normal range's middle, as
@@ -67,9 +66,8 @@ __device__ __forceinline__ F2 f2_from_double(double v) {
   const float hi = __double2float_rn(v);
   return {hi, __double2float_rn(__dsub_rn(v, (double)hi))};
 }
-__device__ __forceinline__ double f2_to_double(F2 a) { return __dadd_rn((double)a.hi, (double)a.lo); }
 
-// The same two conversions with the format changes done in integer
+// That conversion and the one back with the format changes done in integer
 // arithmetic (IEEE-754 binary64 / binary32 fields), for kernels where the
 // FP64 pipe, a small fraction of the FP32 one, would otherwise bound them.
 //
@@ -139,13 +137,6 @@ __device__ __forceinline__ double f64_wide(float f) {
   const unsigned b = __float_as_uint(f);
   const unsigned hi = (b & 0x80000000u) | ((((b >> 23) & 0xffu) + 896u) << 20) | ((b & 0x7fffffu) >> 3);
   return (b & 0x7f800000u) ? __hiloint2double((int)hi, (int)(b << 29)) : 0.0;
-}
-__device__ __forceinline__ float f2_to_float(F2 a) { return __fadd_rn(a.hi, a.lo); }
-// a + b rounded to FP32: f2_to_float(f2_add(a, b)) without the final
-// renormalisation (the same value)
-__device__ __forceinline__ float f2_sum_float(F2 a, F2 b) {
-  const F2 s = two_sum(a.hi, b.hi);
-  return __fadd_rn(s.hi, __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo)));
 }
 
 }  // namespace rtg
