@@ -21,16 +21,20 @@ __device__ __noinline__ double2 chem_substep_fp64(double x, double z, double a, 
 
 // One cell, FP64 path.  The FP64 pipe bounds this kernel, and the closed form
 // of a substep (below) takes two quotients and a square root on it.  Instead
-// the smaller fraction is guessed in FP32 and corrected twice by Newton's
-// method, the residual of the implicit equation in FP64 and the step in FP32
-// (the derivative at the root is -sqrt(D) or sqrt(D)): the first leaves
-// ~1e-13, the second the rounding of its residual,
+// the fraction that is the smaller one after the substep is guessed in FP32
+// and corrected twice by Newton's method, the residual of the implicit
+// equation in FP64 and the step in FP32 (the derivative at the root is
+// -sqrt(D) or sqrt(D)): the first leaves ~1e-13, the second the rounding of
+// its residual,
 //   x-form: (a (1 - x')^2 + x) - b x',   z-form: (a z' + b) z' - (z + hk),
-// whose terms are the size of the result's own.  8 to 10 FP64 operations a
-// substep instead of ~45: 128^3 cells, 10 substeps, 1410 -> 440 us.  Against
-// the recursion in 113 bits over 10 substeps the mean error is 1.5e-16 in x_HI
-// and 1.7e-16 in x_HII, the largest 2.1e-15 and 3.2e-15; the closed form's
-// 1.8e-16, 1.9e-16, 3.7e-15 and 3.9e-15.
+// whose terms are the size of the result's own.  (The guess decides which
+// fraction that is: where a substep takes a cell past 1/2, the other one as
+// one minus the corrected one would only be good to 2^-53 of 1.)  8 to 10 FP64
+// operations a substep instead of ~45: 128^3 cells, 10 substeps, 1410 -> 440
+// us.  Against the recursion in 113 bits the mean error over 10 substeps is
+// 1.5e-16 in x_HI and 1.7e-16 in x_HII, the largest 2.1e-15 and 3.5e-15; the
+// closed form's 1.8e-16, 1.9e-16, 3.6e-15 and 3.7e-15.  The largest of one
+// substep: 6.2e-16 and 4.7e-16, the closed form's 5.8e-16 and 5.1e-16.
 __device__ __forceinline__ void chem_cell_fp64(double& x, double& z, double n, double kc, double h, int nsub,
                                                double alpha) {
   const double a = __dmul_rn(__dmul_rn(h, alpha), n);
@@ -41,17 +45,17 @@ __device__ __forceinline__ void chem_cell_fp64(double& x, double& z, double n, d
   const float af = f32_chop(a), bf = f32_chop(b), hkf = f32_chop(hk);
   for (int i = 0; i < nsub; ++i) {
     const float xf = f32_chop(x), wf = f32_chop(z) + hkf;
-    const bool xform = xf < 0.5f;
-    const float num = xform ? af + xf : wf;
-    if (!fits || !(num >= 1e-22f)) {
+    const float D = fmaf(4.0f * af, wf, bf * bf);
+    const float rs = rsqrtf(D), sq = D * rs;
+    const float gx = __fdividef(2.0f * (af + xf), 2.0f * af + bf + sq);
+    const bool xform = gx < 0.5f;
+    if (!fits || !((xform ? af + xf : wf) >= 1e-22f)) {
       const double2 v = chem_substep_fp64(x, z, a, b, hk);
       x = v.x;
       z = v.y;
       continue;
     }
-    const float D = fmaf(4.0f * af, wf, bf * bf);
-    const float rs = rsqrtf(D);
-    const float g0 = __fdividef(2.0f * num, (xform ? 2.0f * af + bf : bf) + D * rs);
+    const float g0 = xform ? gx : __fdividef(2.0f * wf, bf + sq);
     double v = f64_wide(g0);
     if (xform) {
       v = __dadd_rn(v, f64_wide(rs * f32_chop(__fma_rn(__fma_rn(a, v, -tab), v, __dadd_rn(a, x)))));

@@ -149,3 +149,45 @@ def test_fp64_update_over_its_whole_range(batched):
     if batched:
         b.close()
     grid.close()
+
+
+def _fp64_update(dims, n_H, x_HI, x_HII, k, dt_s, nsub, batched):
+    g = _medium(dims)
+    g.update(n_H=n_H, x_HI=x_HI, x_HII=x_HII)
+    grid = native.Grid(parity.ctx(), g, "fp64")
+    native.rt_set_rates(grid.h, k, np.zeros(k.size))
+    if batched:
+        b = native.Batch(parity.ctx())
+        b.add(grid)
+        b.chem(dt_s, nsub, synth.ALPHA_B)
+        b.close()
+    else:
+        grid.chem(dt_s, nsub, synth.ALPHA_B)
+    x, z = grid.rates()["x_HI"], grid.x_HII()
+    grid.close()
+    return x, z
+
+
+@pytest.mark.parametrize("batched", [False, True])
+@pytest.mark.parametrize("nsub", [1, 2, 3])
+def test_fp64_update_across_one_half(nsub, batched):
+    """Few substeps over which the other fraction becomes the smaller one:
+    neutral cells that are ionised, ionised cells that recombine.  Both keep
+    five units of 2^-53 a substep on either side, relative."""
+    import oracle
+    dims = (16, 16, 16)
+    n = int(np.prod(dims))
+    rng = np.random.default_rng(12)
+    h = synth.MYR_S / nsub
+    ionise = np.arange(n) % 2 == 0
+    small = np.where(rng.random(n) < 0.1, 0.0, 10.0 ** rng.uniform(-16, -0.31, n))
+    x = np.where(ionise, 1.0 - small, small)
+    z = np.where(ionise, small, 1.0 - small)
+    a = 10.0 ** np.where(ionise, rng.uniform(-3, 2, n), rng.uniform(0, 7, n))  # h alpha_B n_H
+    hk = np.where(ionise, 10.0 ** rng.uniform(0, 17, n), 0.0)
+    n_H = a / (h * synth.ALPHA_B)
+    got = _fp64_update(dims, n_H, x, z, hk / h, synth.MYR_S, nsub, batched)
+    want = oracle.chem(n_H, x, z, hk / h, synth.MYR_S, nsub, synth.ALPHA_B)
+    assert ((x > 0.5) != (want[0] > 0.5)).mean() > 0.5
+    for q in range(2):
+        np.testing.assert_allclose(got[q], want[q], rtol=2 * nsub * 5 * 2.0 ** -53, atol=0)
