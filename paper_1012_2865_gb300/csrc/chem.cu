@@ -49,13 +49,15 @@ __device__ __forceinline__ void chem_cell_fp64(double& x, double& z, double n, d
     const float rs = rsqrtf(D), sq = D * rs;
     const float gx = __fdividef(2.0f * (af + xf), 2.0f * af + bf + sq);
     const bool xform = gx < 0.5f;
-    if (!fits || !((xform ? af + xf : wf) >= 1e-22f)) {
+    const float g0 = xform ? gx : __fdividef(2.0f * wf, bf + sq);
+    // the corrections are FP32 numbers: the second one, 1e-13 of the result and
+    // needed to 1e-3, stays above their range's end from 1e-22 on
+    if (!fits || !(g0 >= 1e-22f)) {
       const double2 v = chem_substep_fp64(x, z, a, b, hk);
       x = v.x;
       z = v.y;
       continue;
     }
-    const float g0 = xform ? gx : __fdividef(2.0f * wf, bf + sq);
     double v = f64_wide(g0);
     if (xform) {
       v = __dadd_rn(v, f64_wide(rs * f32_chop(__fma_rn(__fma_rn(a, v, -tab), v, __dadd_rn(a, x)))));

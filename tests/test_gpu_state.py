@@ -191,3 +191,25 @@ def test_fp64_update_across_one_half(nsub, batched):
     assert ((x > 0.5) != (want[0] > 0.5)).mean() > 0.5
     for q in range(2):
         np.testing.assert_allclose(got[q], want[q], rtol=2 * nsub * 5 * 2.0 ** -53, atol=0)
+
+
+@pytest.mark.parametrize("nsub", [1, 2, 10])
+def test_fp64_update_of_tiny_fractions(nsub):
+    """Results down to 1e-60, where corrections held in FP32 would vanish:
+    irradiated gas without recombination (no hydrogen, or next to none) and
+    nearly neutral gas in the dark."""
+    import oracle
+    dims = (16, 16, 16)
+    n = int(np.prod(dims))
+    rng = np.random.default_rng(13)
+    h = synth.MYR_S / nsub
+    lit = np.arange(n) % 2 == 0
+    small = 10.0 ** rng.uniform(-40, -10, n)
+    x, z = np.where(lit, small, 1.0 - small), np.where(lit, 1.0 - small, small)
+    hk = np.where(lit, 10.0 ** rng.uniform(-2, 17.5, n), 0.0)
+    n_H = np.where(lit, np.where(rng.random(n) < 0.5, 0.0, 10.0 ** rng.uniform(-60, -20, n)),
+                   10.0 ** rng.uniform(-3, 4, n))
+    got = _fp64_update(dims, n_H, x, z, hk / h, synth.MYR_S, nsub, False)
+    want = oracle.chem(n_H, x, z, hk / h, synth.MYR_S, nsub, synth.ALPHA_B)
+    for q in range(2):
+        np.testing.assert_allclose(got[q], want[q], rtol=2 * nsub * 5 * 2.0 ** -53, atol=0)
