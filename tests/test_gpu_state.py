@@ -213,3 +213,31 @@ def test_fp64_update_of_tiny_fractions(nsub):
     want = oracle.chem(n_H, x, z, hk / h, synth.MYR_S, nsub, synth.ALPHA_B)
     for q in range(2):
         np.testing.assert_allclose(got[q], want[q], rtol=2 * nsub * 5 * 2.0 ** -53, atol=0)
+
+
+@pytest.mark.parametrize("nsub", [1, 3])
+def test_fp64_update_of_unusual_states(nsub):
+    """Both fractions as given, also where they do not add up to 1 (each
+    rounded to FP32; apart by up to a tenth; x_HII not a number), and rates
+    that are negative or not numbers: as the closed form has them."""
+    import oracle
+    dims = (16, 16, 16)
+    n = int(np.prod(dims))
+    rng = np.random.default_rng(14)
+    h = synth.MYR_S / nsub
+    kind = np.arange(n) % 4
+    x = rng.uniform(0.01, 0.99, n)
+    z = 1.0 - x
+    x = np.where(kind == 0, synth.round_f32(x), x)
+    z = np.where(kind == 0, synth.round_f32(z), np.where(kind == 1, z * rng.uniform(0.9, 1.1, n), z))
+    a = 10.0 ** rng.uniform(-2, 2, n)
+    hk = 10.0 ** rng.uniform(-3, 3, n)
+    negative = kind == 2
+    hk[negative] = rng.uniform(-0.3, 0.0, negative.sum())
+    a[negative] = 10.0 ** rng.uniform(-4, -2, negative.sum())  # keeps the root real
+    z[3], z[7], hk[11], hk[15] = np.nan, np.inf, np.nan, -np.inf
+    n_H = a / (h * synth.ALPHA_B)
+    got = _fp64_update(dims, n_H, x, z, hk / h, synth.MYR_S, nsub, False)
+    want = oracle.chem(n_H, x, z, hk / h, synth.MYR_S, nsub, synth.ALPHA_B)
+    for q in range(2):
+        np.testing.assert_allclose(got[q], want[q], rtol=2 * nsub * 5 * 2.0 ** -53, atol=0)
