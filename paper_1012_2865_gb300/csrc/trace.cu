@@ -811,6 +811,14 @@ struct Walk32 {
     const float4 sa = __ldg(&S.sabs32);
     q = fmaf(hi, 4.1f * kBandT, 1e-30f) +
         4.1f * fmaxf(sa.x * a0.iv.hi, fmaxf(sa.y * a1.iv.hi, sa.z * a2.iv.hi));
+    // step() compares tau + sk q with tau_near, 2^-12 below the termination.
+    // Beside its own boundaries (sk q) a package's error comes from the pair
+    // products (2^-37 of tau; 2^-22 where n_HI is plain FP32), from the sums
+    // (2^-18 at most over the 24,600 planes of a 4096^3 grid), and from its
+    // ancestors, which clip dense cells over lengths that are hardly known:
+    // where those leave more than half of the 2^-12, every segment takes the
+    // full test.
+    if (!(tau_err <= A.tau_term32 * (1.0f / 8192.0f))) q = 1e30f;
     return true;
   }
   __device__ __forceinline__ static float exit_of(const Axis<EXACT>& a, float d, float dim) {

@@ -47,3 +47,29 @@ def test_short_and_long_axes(dims, cells):
     g = _grid(dims, cells, 0.0)
     _, b, r = parity.run_gpu(g, "fp32_mixed")
     parity.assert_trace_parity(g, b, r, parity.run_oracle(g), "fp32_mixed")
+
+
+@pytest.mark.parametrize("seed", range(6))
+def test_termination_after_a_clipped_dense_cell(seed):
+    """A level-6 ray that clips 2e-10 cell lengths off a cell dense enough to
+    take most of its optical depth there: what FP32 pairs know of that length
+    (about 1e-12) leaves an error that only the bound its children inherit
+    covers, and they terminate in thin gas, where it is cells wide."""
+    import oracle
+    rng = np.random.default_rng(seed)
+    dims, dx = (48, 48, 48), 2.0 ** 60
+    n = oracle.pix2vec(6, np.arange(4 ** 6))
+    n = n[np.all((n > 0.45) & (n < 0.7), axis=1)]
+    n = n[rng.integers(len(n))]
+    s = rng.uniform(2.0, 4.0, 3)
+    i = np.ceil(s[0] + 20.0 * n[0])
+    t = (i - s[0]) / n[0]                      # between the splits at 13.8 and 27.7
+    j = np.ceil(s[1] + t * n[1])
+    s[1] = j - (t + 2e-10) * n[1]              # plane j follows plane i at once
+    cell = int(i) + 48 * (int(j) - 1 + 48 * int(s[2] + t * n[2]))
+    f_term, thin = 0.9, 1e-4
+    depth = np.full(48 ** 3, thin)             # optical depth per cell length
+    depth[cell] = (-np.log(f_term) - 37.0 * thin) / 2e-10
+    g = synth._grid(dims, 48 * dx, depth / (synth.SIGMA_HI * dx), 1.0, [s * dx], [1e49], [20.0], [synth.SIGMA_HI])
+    _, b, r = parity.run_gpu(g, "fp32_mixed", f_term=f_term)
+    parity.assert_trace_parity(g, b, r, parity.run_oracle(g, f_term=f_term), "fp32_mixed", exact_segments=True)
