@@ -278,14 +278,15 @@ __global__ void convert_kernel(long long n, const ST* __restrict__ src, double* 
 // as an FP32 pair, rounded (the FP64 pipe is a small fraction of the FP32 one).
 // Small results (an optically thick cell's) would lose the product's low part
 // below the FP32 range and are formed 2^64 times larger; results below the
-// FP32 normal range go through FP64, out of line so that its instructions are
-// not predicated into every cell.
+// FP32 normal range, infinities and values that are not numbers go through
+// FP64, out of line so that its instructions are not predicated into every
+// cell.
 __device__ __noinline__ float scale64(float v, double scale) { return (float)((double)v * scale); }
 __device__ __forceinline__ float scale32(float v, double scale, float sh, float sl) {
   float p = __fmul_rn(v, sh), up = 1.0f;
-  if (fabsf(p) < 1e-30f) {
+  if (!(fabsf(p) >= 1e-30f && fabsf(p) <= 3e38f)) {
     if (v == 0.0f) return 0.0f;
-    if (fabsf(p) < 2.4e-38f || sh < 1e-20f) return scale64(v, scale);
+    if (!(fabsf(p) >= 2.4e-38f && fabsf(p) <= 3e38f) || sh < 1e-20f) return scale64(v, scale);
     v *= 18446744073709551616.0f;  // 2^64
     p = __fmul_rn(v, sh);
     up = 5.4210108624275222e-20f;  // 2^-64

@@ -241,3 +241,27 @@ def test_fp64_update_of_unusual_states(nsub):
     want = oracle.chem(n_H, x, z, hk / h, synth.MYR_S, nsub, synth.ALPHA_B)
     for q in range(2):
         np.testing.assert_allclose(got[q], want[q], rtol=2 * nsub * 5 * 2.0 ** -53, atol=0)
+
+
+@pytest.mark.parametrize("skip", [0, 1])
+def test_rates_without_a_number_are_read_as_they_are(skip):
+    """Infinities, values beyond FP32 and what is not a number, through both
+    forms of the FP32 read."""
+    import torch
+    dims = (4, 3, 5)
+    n = int(np.prod(dims))
+    grid = native.Grid(parity.ctx(), _medium(dims), "fp32_mixed")
+    gam = np.full(n, 1e-25)
+    gam[1:8] = np.inf, -np.inf, np.nan, 1e60, -1e60, 3e26, -1e-25
+    k = np.full(n, 1e-12)
+    k[1:4] = np.inf, np.nan, 1e300
+    native.rt_set_rates(grid.h, k, gam)
+    want = grid.rates()
+    assert np.isinf(want["gamma"][[1, 2, 4, 5]]).all() and np.isnan(want["gamma"][3])
+    out = torch.zeros((2, n + 4), dtype=torch.float32, device="cuda")
+    native.rt_get_rates_async(grid.h, *(out[q, skip:skip + n] for q in range(2)), dtype=native.RT_DTYPE_F32)
+    native.rt_synchronize(grid.h)
+    got = out.cpu().numpy()[:, skip:skip + n]
+    np.testing.assert_array_equal(got[0], want["kph"].astype(np.float32))
+    np.testing.assert_allclose(got[1], want["gamma"], rtol=2.0 ** -23)
+    grid.close()
