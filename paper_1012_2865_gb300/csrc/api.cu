@@ -353,6 +353,20 @@ static int upload(void* dst, const void* src, size_t bytes, int mem_kind, cudaSt
   return RT_OK;
 }
 
+// Whether kernels of `device` may take a caller's device array of `elem`-byte
+// elements where it lies: on an element's boundary, and in memory of that GPU
+// or mapped for every one.  (Copies take the others, or refuse them.)
+static bool in_place(const void* p, size_t elem, int device) {
+  if ((uintptr_t)p % elem != 0) return false;
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeManaged || (a.type == cudaMemoryTypeHost && a.devicePointer == p) ||
+         (a.type == cudaMemoryTypeDevice && a.device == device);
+}
+
 int rt_create_grid(rt_ctx* ctx, const rt_grid_desc* d, void* stream, rt_grid** out) {
   if (!ctx || !d || !out) return fail(RT_ERR_INVALID_ARG, "rt_create_grid: NULL argument");
   if (d->nx < 1 || d->ny < 1 || d->nz < 1) return fail(RT_ERR_INVALID_ARG, "rt_create_grid: dims must be >= 1");
@@ -1025,8 +1039,8 @@ int rt_set_state(rt_grid* g, const double* n_H, const double* x_HI, const double
   const long long ncell = g->ncell;
   const size_t n8 = (size_t)ncell * 8;
   cudaStream_t st = g->stream;
-  // The new state is checked where it lies on the device (a host state is
-  // staged there first) and replaces the grid's in the next kernel, unless a
+  // The new state is checked where it lies on the device (what kernels cannot
+  // read there is staged first) and replaces the grid's in the next kernel, unless a
   // cell failed (an invalid call leaves the grid unchanged); then the caller
   // learns the verdict.  (Staging device arrays too, in memory allocated for
   // the call, and copying them after the verdict took 360 us for a 128^3 state
@@ -1034,15 +1048,20 @@ int rt_set_state(rt_grid* g, const double* n_H, const double* x_HI, const double
   const double *sn = n_H, *sx = x_HI, *sz = x_HII;
   double* stage = nullptr;
   int rc = RT_OK;
-  if (mem_kind == RT_MEM_HOST) {
-    const int nf = (n_H ? 1 : 0) + 1 + (x_HII ? 1 : 0);
+  const double** src[3] = {&sn, &sx, &sz};
+  bool put[3];
+  int nf = 0;
+  for (int f = 0; f < 3; ++f) {
+    put[f] = *src[f] && (mem_kind == RT_MEM_HOST || !in_place(*src[f], sizeof(double), g->ctx->device));
+    nf += put[f];
+  }
+  if (nf) {
     CUDA_TRY(cudaMallocAsync((void**)&stage, nf * n8, st));
     double* d = stage;
-    const double** dst[3] = {&sn, &sx, &sz};
     for (int f = 0; f < 3 && !rc; ++f) {
-      if (!*dst[f]) continue;
-      rc = upload(d, *dst[f], n8, mem_kind, st);
-      *dst[f] = d;
+      if (!put[f]) continue;
+      rc = upload(d, *src[f], n8, mem_kind, st);
+      *src[f] = d;
       d += ncell;
     }
   }
@@ -1145,7 +1164,19 @@ int rt_get_rates_async(rt_grid* g, void* kph, void* gamma, void* x_HI, int dtype
   const long long n = g->ncell;
   cudaStream_t st = g->stream;
   if (mem_kind == RT_MEM_DEVICE) {
-    LAUNCH_TRY(launch_read_rates(g->precision, n, g->K, g->G, g->xHI, kph, gamma, x_HI, dtype, gamma_scale(g), st));
+    // fields of the caller's type go to buffers that kernels cannot write as
+    // copies (k_ph of a mixed grid: every second word)
+    const bool mixed = g->precision == RT_FP32_MIXED, f64 = dtype == RT_DTYPE_F64;
+    const size_t eb = f64 ? 8 : 4;
+    const void* same[3] = {mixed != f64 ? g->K : nullptr, f64 ? g->G : nullptr, f64 ? g->xHI : nullptr};
+    for (int f = 0; f < 3; ++f) {
+      if (!dst[f] || !same[f] || in_place(dst[f], eb, g->ctx->device)) continue;
+      if (f == 0 && mixed) CUDA_TRY(cudaMemcpy2DAsync(dst[f], eb, same[f], 8, eb, (size_t)n, cudaMemcpyDeviceToDevice, st));
+      else CUDA_TRY(cudaMemcpyAsync(dst[f], same[f], (size_t)n * eb, cudaMemcpyDeviceToDevice, st));
+      dst[f] = nullptr;
+    }
+    if (dst[0] || dst[1] || dst[2])
+      LAUNCH_TRY(launch_read_rates(g->precision, n, g->K, g->G, g->xHI, dst[0], dst[1], dst[2], dtype, gamma_scale(g), st));
     return RT_OK;
   }
   int rc = ensure_async(g, false, true);

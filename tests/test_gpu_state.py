@@ -265,3 +265,48 @@ def test_rates_without_a_number_are_read_as_they_are(skip):
     np.testing.assert_array_equal(got[0], want["kph"].astype(np.float32))
     np.testing.assert_allclose(got[1], want["gamma"], rtol=2.0 ** -23)
     grid.close()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32_mixed"])
+def test_device_arrays_off_an_element_boundary(precision):
+    """Through the C ABI a device array may start at any byte: what kernels
+    cannot read or write there is copied."""
+    import torch
+    dims = (5, 4, 3)
+    n = int(np.prod(dims))
+    grid = native.Grid(parity.ctx(), _medium(dims), precision)
+    want = _medium(dims, seed=21)
+
+    def put(a):
+        t = torch.zeros(8 * n + 8, dtype=torch.uint8, device="cuda")
+        t[4:4 + 8 * n] = torch.tensor(np.frombuffer(np.asarray(a, dtype=np.float64).tobytes(), dtype=np.uint8).copy())
+        return t
+
+    keep = [put(want["n_H"]), put(want["x_HI"])]
+    native.check(native.lib().rt_set_state(grid.h, keep[0].data_ptr() + 4, keep[1].data_ptr() + 4, None,
+                                           native.RT_MEM_DEVICE))
+    bad = put(np.full(n, 2.0))
+    with pytest.raises(native.RtError, match=r"x_HI\[0\]"):
+        native.check(native.lib().rt_set_state(grid.h, None, bad.data_ptr() + 4, None, native.RT_MEM_DEVICE))
+    rng = np.random.default_rng(3)
+    k, gam = synth.round_f32(10.0 ** rng.uniform(-20, -8, n)), 10.0 ** rng.uniform(-30, -20, n)
+    native.rt_set_rates(grid.h, k, gam)
+
+    def read(field, dtype, off):  # one field into a buffer `off` bytes off
+        size = 8 if dtype == native.RT_DTYPE_F64 else 4
+        t = torch.full((size * n + 16,), 7, dtype=torch.uint8, device="cuda")
+        p = [None, None, None]
+        p[field] = t.data_ptr() + off
+        native.check(native.lib().rt_get_rates_async(grid.h, *p, dtype, native.RT_MEM_DEVICE))
+        native.rt_synchronize(grid.h)
+        b = t.cpu().numpy()
+        assert (b[:off] == 7).all() and (b[off + size * n:] == 7).all()
+        return np.frombuffer(b[off:off + size * n].tobytes(), dtype=np.float64 if size == 8 else np.float32)
+
+    np.testing.assert_array_equal(read(2, native.RT_DTYPE_F64, 4), want["x_HI"])
+    if precision == "fp64":
+        np.testing.assert_array_equal(read(0, native.RT_DTYPE_F64, 1), k)
+        np.testing.assert_array_equal(read(1, native.RT_DTYPE_F64, 4), gam)
+    else:
+        np.testing.assert_array_equal(read(0, native.RT_DTYPE_F32, 2), k)
+    grid.close()
