@@ -559,7 +559,7 @@ __global__ void check_refresh_kernel(long long n, unsigned long long* __restrict
 // rounding), taken in FP32 where that proves it.
 struct StepArgs {
   double sdx, tau_front;
-  float sdx32;         // 0 where FP32 cannot hold it
+  float sdx32;         // 0 where FP32 cannot hold it or its products
   float hi32, lo32;    // above hi32 in FP32 proves a front cell, below lo32 proves none (inf, -1: never)
   float eps, alpha, dt_max, unit;
   float dt_max_units;  // dt_max / unit
@@ -571,9 +571,13 @@ __device__ __noinline__ bool front_fp64(double nh, double x, double sdx, double 
 __device__ __forceinline__ float cell_timestep(double nh64, double x64, float k, const StepArgs& p) {
   const float nh = f2_from_double_bits(nh64).hi, x = f2_from_double_bits(x64).hi;
   const float rate = fabsf(k + nh * (1.0f - x) * p.alpha);
-  const float t = p.sdx32 * nh * x;  // within 2^-22 of sdx n_HI unless it underflows
+  // within 2^-21 of sdx n_HI where that comes near tau_front: sdx and sdx n_H
+  // are below 1e25 and tau_front above 1e-12, so n_H and x are normal there
+  // (beyond, not a number: neither side is proven)
+  const float t1 = p.sdx32 * nh;
+  const float t = t1 < 1e25f ? t1 * x : __int_as_float(0x7fffffff);
   bool front = t > p.hi32;
-  if (!(front && t < 3e38f) && !(t < p.lo32)) front = front_fp64(nh64, x64, p.sdx, p.tau_front);
+  if (!front && !(t < p.lo32)) front = front_fp64(nh64, x64, p.sdx, p.tau_front);
   float dt = p.dt_max;
   if (front && rate > 0.0f) {
     dt = fminf(p.dt_max, p.eps / rate);
@@ -660,11 +664,15 @@ cudaError_t launch_timestep(int nx, int ny, int nz, const double* nH, const doub
                             double sdx, double tau_front, float eps, float alpha, float dt_max, float unit,
                             unsigned int* out, unsigned long long* done, cudaStream_t st) {
   StepArgs p = {sdx, tau_front, 0.0f, INFINITY, -1.0f, eps, alpha, dt_max, unit, dt_max / unit};
-  if (sdx > 1e-30 && sdx < 1e30) {
+  if (sdx > 1e-30 && sdx < 1e25) {
     const float tau32 = (float)tau_front;
     p.sdx32 = (float)sdx;
-    p.hi32 = tau32 * (1.0f + 1e-6f);
-    if (tau32 > 1e-30f) p.lo32 = tau32 * (1.0f - 1e-6f);
+    if (tau32 > 1e-12f) {
+      p.hi32 = tau32 * (1.0f + 1e-6f);
+      p.lo32 = tau32 * (1.0f - 1e-6f);
+    } else if (tau_front == 0.0) {
+      p.hi32 = 0.0f;
+    }
   }
   const long long tiles = (long long)((nx + kTileX - 1) / kTileX) * ((ny + kTileY - 1) / kTileY) *
                           ((nz + kTileZ - 1) / kTileZ);

@@ -310,3 +310,22 @@ def test_device_arrays_off_an_element_boundary(precision):
     else:
         np.testing.assert_array_equal(read(0, native.RT_DTYPE_F32, 2), k)
     grid.close()
+
+
+@pytest.mark.parametrize("sdx,n_H,x,tau", [(7.0, 0.03, 0.2, None), (1e5, 1e25, 3e-40, None), (3.0, 1e37, 2e-42, None),
+                                           (1e28, 1e-39, 0.3, None), (1e28, 1e-39, 0.3, 1e-20), (1e-28, 1e30, 0.5, None),
+                                           (1e-20, 1e-25, 0.5, 1e-13), (1e29, 1e35, 1e-60, 1e3), (5.0, 1e-3, 1e-9, 0.0),
+                                           (5.0, 1e-3, 0.0, 0.0), (2.0, 0.0, 0.5, 0.1)])
+def test_front_cells_are_the_fp64_ones(sdx, n_H, x, tau):
+    """One cell on either side of the threshold, from 1e-13 to 1e-3 of it (or at
+    a threshold of its own), also where FP32 holds a factor to a few bits."""
+    g = synth._grid((1, 1, 1), 1.0, 1.0, x, [[0.5, 0.5, 0.5]], [1e48], [13.6], [synth.SIGMA_HI])
+    g["n_H"] = np.full(1, n_H)
+    grid = native.Grid(parity.ctx(), g, "fp32_mixed")
+    native.rt_set_rates(grid.h, np.full(1, 1e-10), np.zeros(1))
+    depth = np.float64(sdx) * n_H * x
+    steps = np.concatenate([s * 10.0 ** np.arange(-13, -2.9, 0.125) for s in (-1.0, 1.0)])
+    for t in ([float(depth * (1.0 + d)) for d in steps] if tau is None else [tau]):
+        got = native.rt_timestep(grid.h, sigma_front=sdx, tau_front=t, dt_max=1e20)
+        assert (got < 1e19) == bool(depth > t), (t, got)  # 0.05 / rate in a front cell
+    grid.close()
