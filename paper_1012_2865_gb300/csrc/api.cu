@@ -44,7 +44,8 @@ cudaError_t launch_commit_state(int precision, long long n, unsigned long long* 
                                double* xHII, void* nhi, cudaStream_t st);
 cudaError_t launch_timestep(int nx, int ny, int nz, const double* nH, const double* xHI, const void* K, int fp64_rates,
                             double sdx, double tau_front, float eps, float alpha, float dt_max, float unit,
-                            unsigned int* out, unsigned long long* done, cudaStream_t st);
+                            unsigned int* out, unsigned long long* done, float* field, cudaStream_t st);
+bool timestep_two_passes(int nx, int ny, int nz);
 cudaError_t launch_check_state(long long n, const double* nH, const double* x, unsigned long long* bad,
                                cudaStream_t st);
 cudaError_t launch_check_density(long long n, const double* a, unsigned long long* bad, cudaStream_t st);
@@ -252,6 +253,7 @@ struct rt_grid {
   double* up_stage = nullptr;                // 3 * ncell doubles: n_H, x_HI, x_HII
   double* xHI_alt = nullptr;                 // alternate state buffers: an upload without n_H goes
   double* xHII_alt = nullptr;                // into them and they swap with xHI, xHII on commit
+  float* step_field = nullptr;               // ncell cell timesteps (grids that rt_timestep takes in two passes)
   char* dn_stage = nullptr;                  // 3 * ncell * 8 bytes: k_ph, Gamma, x_HI
   std::string set_err;                       // message of a rejected asynchronous state
   ~rt_grid() {
@@ -263,7 +265,7 @@ struct rt_grid {
     if (up) cudaStreamDestroy(up);
     if (dn) cudaStreamDestroy(dn);
     cudaFree(nH); cudaFree(xHI); cudaFree(xHII); cudaFree(nhi); cudaFree(K); cudaFree(G);
-    cudaFree(inst_dev); cudaFree(src_dev);
+    cudaFree(inst_dev); cudaFree(src_dev); cudaFree(step_field);
     for (int t = 0; t < 2; ++t) {
       if (nhe[t] != nhe64[t]) cudaFree(nhe[t]);
       cudaFree(nhe64[t]); cudaFree(Khe[t]); cudaFree(Ghe[t]);
@@ -1410,9 +1412,12 @@ int rt_timestep(rt_grid* g, double eps_ion, double alpha_B, double sigma_front, 
   // finite dt_max: values in units of dt_max (cells outside the front hold 1)
   const bool finite = isfinite(dt_max) && dt_max < 3.0e38;
   const float dmax = finite ? (float)dt_max : 3.0e38f;
+  if (!g->step_field && timestep_two_passes(g->nx, g->ny, g->nz))
+    CUDA_TRY(cudaMalloc((void**)&g->step_field, (size_t)g->ncell * sizeof(float)));
   LAUNCH_TRY(launch_timestep(g->nx, g->ny, g->nz, g->nH, g->xHI, g->K, g->precision == RT_FP64, sigma_front * g->dx,
                              tau_front, (float)eps_ion, (float)alpha_B, dmax, finite ? dmax : 1.0f, out,
-                             g->ts.ctl + kWordsStep + 1, st));
+                             g->ts.ctl + kWordsStep + 1, g->step_field, st));
+  if (g->step_field) g_launches.fetch_add(1);
   CUDA_TRY(cudaMemcpyAsync(h, out + 1, sizeof *h, cudaMemcpyDeviceToHost, st));
   CUDA_TRY(cudaStreamSynchronize(st));
   float v;

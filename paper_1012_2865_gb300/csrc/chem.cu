@@ -586,11 +586,26 @@ __device__ __forceinline__ float cell_timestep(double nh64, double x64, float k,
   return p.dt_max_units;
 }
 
+// A block's minimum into the grid's: atomicMin on the bit patterns, which order
+// like the positive floats; the block that finishes last moves the minimum to
+// out[1] and resets the running one.
+__device__ __forceinline__ void timestep_finish(float best, unsigned int* out, unsigned long long* done) {
+  for (int o = 16; o > 0; o >>= 1) best = fminf(best, __shfl_xor_sync(0xffffffffu, best, o));
+  if ((threadIdx.x & 31) == 0) atomicMin(&out[0], __float_as_uint(best));
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    if (atomicAdd(done, 1ULL) == (unsigned long long)gridDim.x - 1ULL) {
+      __threadfence();
+      out[1] = atomicExch(&out[0], 0x7f800000u);
+      *done = 0ULL;
+    }
+  }
+}
+
 // Steps 1-3 in one pass over tiles: the per-cell timestep of a tile and its
 // halo in shared memory, the 3^3 Gaussian (exp(-|d|^2/2), renormalised over
-// neighbours inside the grid), and its minimum over the grid (atomicMin on the
-// bit patterns, which order like the positive floats).  The block that
-// finishes last moves the minimum to out[1] and resets the running one.
+// neighbours inside the grid), and its minimum over the grid.
 // Bound by its issue slots (the per-cell timestep of 1.7 cells a cell, mostly).
 // The weights are products over the axes, so a plane's sum is three sums of
 // rows and passes on to the planes beside it; the cells outside hold 0 and the
@@ -645,24 +660,59 @@ __global__ void __launch_bounds__(256) timestep_kernel(int nx, int ny, int nz, c
       }
     }
   }
-  for (int o = 16; o > 0; o >>= 1) best = fminf(best, __shfl_xor_sync(0xffffffffu, best, o));
-  if ((threadIdx.x & 31) == 0) atomicMin(&out[0], __float_as_uint(best));
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    if (atomicAdd(done, 1ULL) == (unsigned long long)gridDim.x - 1ULL) {
-      __threadfence();
-      out[1] = atomicExch(&out[0], 0x7f800000u);
-      *done = 0ULL;
-    }
+  timestep_finish(best, out, done);
+}
+
+// The same in two passes over a field in memory, for grids that fill the tiles
+// badly (see launch_timestep).
+template <typename KT>
+__global__ void __launch_bounds__(256) cell_timestep_kernel(long long n, const double* __restrict__ nH,
+                                                            const double* __restrict__ xHI, const KT* __restrict__ K,
+                                                            int kstride, StepArgs p, float* __restrict__ field) {
+  for (long long c = blockIdx.x * 256LL + threadIdx.x; c < n; c += gridDim.x * 256LL)
+    field[c] = cell_timestep(nH[c], xHI[c], (float)K[c * kstride], p);
+}
+__global__ void __launch_bounds__(256) filter_min_kernel(int nx, int ny, int nz, const float* __restrict__ field,
+                                                         unsigned int* __restrict__ out,
+                                                         unsigned long long* __restrict__ done) {
+  const float w = 0.60653066f;  // e^-1/2
+  const long long n = (long long)nx * ny * nz;
+  float best = __int_as_float(0x7f800000);
+  for (long long c = blockIdx.x * 256LL + threadIdx.x; c < n; c += gridDim.x * 256LL) {
+    const int x = (int)(c % nx), y = (int)((c / nx) % ny), z = (int)(c / ((long long)nx * ny));
+    const auto row = [&](int j, int k) {
+      if (j < 0 || j >= ny || k < 0 || k >= nz) return 0.0f;
+      const float* f = field + (x + (long long)nx * (j + (long long)ny * k));
+      return fmaf(w, (x > 0 ? f[-1] : 0.0f) + (x < nx - 1 ? f[1] : 0.0f), f[0]);
+    };
+    const auto plane = [&](int k) { return fmaf(w, row(y - 1, k) + row(y + 1, k), row(y, k)); };
+    const float cx = (float)((x > 0) + (x < nx - 1)), cy = (float)((y > 0) + (y < ny - 1)),
+                cz = (float)((z > 0) + (z < nz - 1));
+    const float wx = fmaf(w, cx, 1.0f), wxy = fmaf(w, cy * wx, wx);
+    best = fminf(best, fmaf(w, plane(z - 1) + plane(z + 1), plane(z)) / fmaf(w, cz * wxy, wxy));
   }
+  timestep_finish(best, out, done);
+}
+
+// Whether rt_timestep takes the two passes (and so needs a field of nx ny nz
+// floats): where the tiles hold more than 2.5 times the grid's cells, as those
+// of a grid of a few cells across do.  Bound by the loads of the 27 neighbours,
+// the passes take 30 us + 15 ps a cell whatever the shape, the tiles 10 ps a
+// cell that they hold: 12x300x300 (2.7 times) 51 in tiles and 41 us in two passes,
+// 2x1024x1024 (16 times) 349 and 64 us, 1x1x20000000 (256 times) 19500 and 290 us;
+// 16x256x256 (2 times) 40 and 40 us, 40x300x300 (1.6 times) 80 and 91 us, 256^3 199 and
+// 348 us.  (Two passes over a field allocated in each call: 150, 177 and 559 us
+// for the first three.)
+bool timestep_two_passes(int nx, int ny, int nz) {
+  const auto tiles = [](int d, int t) { return (double)((d + t - 1) / t) * t / d; };
+  return tiles(nx, kTileX) * tiles(ny, kTileY) * tiles(nz, kTileZ) > 2.5;
 }
 
 // The minimum (bits of a float) into out[1]; out[0] holds +inf between calls,
-// *done 0.
+// *done 0; field: null, or what timestep_two_passes asks for.
 cudaError_t launch_timestep(int nx, int ny, int nz, const double* nH, const double* xHI, const void* K, int fp64_rates,
                             double sdx, double tau_front, float eps, float alpha, float dt_max, float unit,
-                            unsigned int* out, unsigned long long* done, cudaStream_t st) {
+                            unsigned int* out, unsigned long long* done, float* field, cudaStream_t st) {
   StepArgs p = {sdx, tau_front, 0.0f, INFINITY, -1.0f, eps, alpha, dt_max, unit, dt_max / unit};
   if (sdx > 1e-30 && sdx < 1e25) {
     const float tau32 = (float)tau_front;
@@ -673,6 +723,16 @@ cudaError_t launch_timestep(int nx, int ny, int nz, const double* nH, const doub
     } else if (tau_front == 0.0) {
       p.hi32 = 0.0f;
     }
+  }
+  if (field) {
+    const long long n = (long long)nx * ny * nz;
+    const int g = (int)(n < 152 * 8 * 256 ? (n + 255) / 256 : 152 * 8);
+    if (fp64_rates)
+      cell_timestep_kernel<double><<<g, 256, 0, st>>>(n, nH, xHI, (const double*)K, 1, p, field);
+    else
+      cell_timestep_kernel<float><<<g, 256, 0, st>>>(n, nH, xHI, (const float*)K, 2, p, field);
+    filter_min_kernel<<<g, 256, 0, st>>>(nx, ny, nz, field, out, done);
+    return cudaGetLastError();
   }
   const long long tiles = (long long)((nx + kTileX - 1) / kTileX) * ((ny + kTileY - 1) / kTileY) *
                           ((nz + kTileZ - 1) / kTileZ);

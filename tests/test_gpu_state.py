@@ -329,3 +329,38 @@ def test_front_cells_are_the_fp64_ones(sdx, n_H, x, tau):
         got = native.rt_timestep(grid.h, sigma_front=sdx, tau_front=t, dt_max=1e20)
         assert (got < 1e19) == bool(depth > t), (t, got)  # 0.05 / rate in a front cell
     grid.close()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32_mixed"])
+@pytest.mark.parametrize("dims", [(12, 16, 8), (13, 16, 8), (1, 1, 300), (1, 300, 1), (300, 1, 1), (2, 3, 200),
+                                  (4, 4, 64), (3, 1, 90), (257, 2, 3)])
+def test_timestep_of_thin_grids(precision, dims):
+    """Grids that fill the tiles badly take two passes over a field: both forms
+    against the oracle on either side of the rule."""
+    g = _medium(dims, sources=1)
+    grid, _, r = parity.run_gpu(g, precision)
+    for kw in (dict(dt_max=1e16, tau_front=0.02), dict(dt_max=1e16, tau_front=0.0)):
+        want = timestep.rt_timestep(tuple(dims), g["box_len_cm"] / dims[0], g["n_H"], r["x_HI"],
+                                    np.asarray(r["kph"], dtype=np.float64), **kw)
+        assert native.rt_timestep(grid.h, **kw) == pytest.approx(want, rel=1e-5)
+    grid.close()
+
+
+def test_timestep_takes_the_time_of_the_cells():
+    """A column of cells is no slower than the same number in a cube by more
+    than its neighbours' loads (five times allows for a slow call)."""
+    import time
+    best = []
+    for dims in ((160, 160, 160), (1, 1, 4096000)):
+        grid = native.Grid(parity.ctx(), synth._grid(dims, 1e21, 1e-3, 0.5, [[0, 0, 0]], [1e48], [13.6],
+                                                     [synth.SIGMA_HI]), "fp32_mixed")
+        n = int(np.prod(dims))
+        native.rt_set_rates(grid.h, np.full(n, 1e-12), np.zeros(n))
+        times = []
+        for _ in range(8):
+            t = time.perf_counter()
+            native.rt_timestep(grid.h, dt_max=1e16)
+            times.append(time.perf_counter() - t)
+        best.append(min(times))
+        grid.close()
+    assert best[1] < 5 * best[0], best
