@@ -73,3 +73,27 @@ def test_termination_after_a_clipped_dense_cell(seed):
     g = synth._grid(dims, 48 * dx, depth / (synth.SIGMA_HI * dx), 1.0, [s * dx], [1e49], [20.0], [synth.SIGMA_HI])
     _, b, r = parity.run_gpu(g, "fp32_mixed", f_term=f_term)
     parity.assert_trace_parity(g, b, r, parity.run_oracle(g, f_term=f_term), "fp32_mixed", exact_segments=True)
+
+
+def test_diagonal_ties_need_no_fallback():
+    """Sources on the lattice in a launch that holds others too, and in the
+    allocation-free trace: the ties of their 45-degree rays are exact there as
+    well, so each source takes the FP64 fallbacks it takes by itself."""
+    import torch
+    from paper_1012_2865_gb300 import native
+    dims, alone = (16, 11, 7), 0
+    lattice = [(4.5, 7.5, 2.5), (8.5, 5.5, 3.5), (3.5, 2.5, 1.5), (3.0625, 9.9375, 6.5), (8.0, 5.0, 3.0)]
+    for cells in (lattice, BESIDE):
+        alone += parity.run_gpu(_grid(dims, cells, 0.0), "fp32_mixed")[1]["fallbacks"]
+    _, b, _ = parity.run_gpu(_grid(dims, lattice + BESIDE, 0.0), "fp32_mixed")
+    assert b["fallbacks"] == alone
+    g = _grid(dims, lattice, 0.0)
+    _, b, _ = parity.run_gpu(g, "fp32_mixed")
+    dev = lambda a, t: torch.tensor(a, dtype=t, device="cuda")
+    n = int(np.prod(dims))
+    out = torch.zeros((2, n), dtype=torch.float32, device="cuda")
+    na = native.rt_trace_noalloc(dims, g["box_len_cm"], dev(g["n_H"] * g["x_HI"], torch.float32),
+                                 dev(g["n_H"], torch.float64), dev(g["x_HI"], torch.float64), out[0], out[1],
+                                 g["pos_cm"], g["ndot"], g["e_ph_eV"], g["sigma_cm2"],
+                                 native.trace_params(**synth.DEFAULT_PARAMS))
+    assert na["fallbacks"] == b["fallbacks"]
