@@ -347,13 +347,17 @@ __global__ void read_rates4_kernel(long long n, const float2* __restrict__ kg, c
   }
 }
 
-// The caller's k_ph and Gamma (times scale) into an FP32-mixed grid.
+// The caller's k_ph and Gamma (times scale), each where it is given, into an
+// FP32-mixed grid.
 template <typename ST>
 __global__ void write_rates_kernel(long long n, const ST* __restrict__ k, const ST* __restrict__ g,
                                    float2* __restrict__ kg, double scale) {
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n;
-       c += (long long)gridDim.x * blockDim.x)
-    kg[c] = make_float2((float)k[c], (float)((double)g[c] * scale));
+       c += (long long)gridDim.x * blockDim.x) {
+    if (k && g) kg[c] = make_float2((float)k[c], (float)((double)g[c] * scale));
+    else if (k) kg[c].x = (float)k[c];
+    else kg[c].y = (float)((double)g[c] * scale);
+  }
 }
 
 __global__ void complement_kernel(long long n, const double* __restrict__ x, double* __restrict__ out) {
