@@ -364,3 +364,22 @@ def test_timestep_takes_the_time_of_the_cells():
         best.append(min(times))
         grid.close()
     assert best[1] < 5 * best[0], best
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32_mixed"])
+def test_host_reads_in_pieces(precision):
+    """Fields longer than the read-back buffer (32 MB) by an odd remainder."""
+    dims = (9000001, 1, 1)
+    n = dims[0]
+    grid = native.Grid(parity.ctx(), synth._grid(dims, 1e21, 1e-3, np.linspace(0.0, 1.0, n), [[0, 0, 0]], [1e48],
+                                                 [13.6], [synth.SIGMA_HI]), precision)
+    k = synth.round_f32(1e-12 * np.arange(1, n + 1))
+    native.rt_set_rates(grid.h, k, k * 1e-13)
+    for dtype, tol in ((native.RT_DTYPE_F64, 0.0 if precision == "fp64" else 2.0 ** -23), (native.RT_DTYPE_F32, 2.0 ** -22)):
+        r = grid.rates(dtype)
+        np.testing.assert_array_equal(r["kph"], k.astype(r["kph"].dtype))
+        np.testing.assert_allclose(r["gamma"], k * 1e-13, rtol=tol)
+        np.testing.assert_array_equal(r["x_HI"], np.linspace(0.0, 1.0, n).astype(r["x_HI"].dtype))
+        np.testing.assert_array_equal(native.rt_get_ionised(grid.h, n, dtype),
+                                      (1.0 - np.linspace(0.0, 1.0, n)).astype(r["x_HI"].dtype))
+    grid.close()
