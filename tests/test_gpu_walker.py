@@ -97,3 +97,20 @@ def test_diagonal_ties_need_no_fallback():
                                  g["pos_cm"], g["ndot"], g["e_ph_eV"], g["sigma_cm2"],
                                  native.trace_params(**synth.DEFAULT_PARAMS))
     assert na["fallbacks"] == b["fallbacks"]
+
+
+def test_lengths_along_a_diagonal_in_the_general_form():
+    """Unsplit rays through next to nothing: k_ph is the path length per cell,
+    also along the 45-degree rays of lattice sources, whose ties the general
+    form (an off-lattice source is there too) meets with two pairs for one
+    distance.  An FP32 unit of a radius of 40 is 4e-6 cells."""
+    dims, dx = (64, 64, 64), 2.0 ** 60
+    rng = np.random.default_rng(5)
+    cells = [(x + 0.5, y + 0.5, z + 0.5) for x, y, z in rng.integers(2, 20, (7, 3))] + [(50.3, 50.7, 3.1)]
+    g = synth._grid(dims, 64 * dx, 1e-9 / (synth.SIGMA_HI * dx), 1.0, np.asarray(cells) * dx, np.full(8, 1e49),
+                    np.full(8, 20.0), np.full(8, synth.SIGMA_HI))
+    o = parity.run_oracle(g, level0=2, max_level=2)
+    _, b, r = parity.run_gpu(g, "fp32_mixed", level0=2, max_level=2)
+    np.testing.assert_array_equal(b["counts"], o["counts"])
+    length = o["kph"][o["kph"] > 0].mean()
+    np.testing.assert_allclose(r["kph"], o["kph"], rtol=1e-6, atol=1e-6 * length)
