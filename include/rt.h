@@ -256,9 +256,9 @@ int rt_chem_update(rt_grid* grid, double dt_s, int nsub, double alpha_B);
 /* Replace the gas state of every cell (Sec. 2.2): n_H (may be NULL to keep
  * it), x_HI, and x_HII (NULL for 1 - x_HI), in memory mem_kind, same checks
  * as rt_create_grid; refreshes the absorber density.  The new state is
- * staged and checked on the device: the call returns once the check is done
- * (the caller's arrays may then be reused) and leaves the state unchanged
- * when it fails. */
+ * checked on the device, where device arrays are read in place and host arrays
+ * staged: the call returns once it has replaced the grid's (the caller's
+ * arrays may then be reused) and leaves that unchanged when the check fails. */
 int rt_set_state(rt_grid* grid, const double* n_H, const double* x_HI, const double* x_HII,
                  int mem_kind);
 

@@ -1049,7 +1049,7 @@ int rt_set_state(rt_grid* g, const double* n_H, const double* x_HI, const double
   // cell failed (an invalid call leaves the grid unchanged); then the caller
   // learns the verdict.  (Staging device arrays too, in memory allocated for
   // the call, and copying them after the verdict took 360 us for a 128^3 state
-  // and 250 us for a 32^3 one, now 52 and 36 us.)
+  // and 250 us for a 32^3 one, now 51 and 30 us.)
   const double *sn = n_H, *sx = x_HI, *sz = x_HII;
   double* stage = nullptr;
   int rc = RT_OK;

@@ -187,7 +187,8 @@ __global__ void chem_kernel(long long ncell, const double* __restrict__ nH, doub
 // residual: 128^3 cells, 10 substeps, the whole call 102 -> 70 us.  Over 10
 // substeps the error against 113 bits is 4.2e-13 at most and 6.0e-15 on average
 // in x_HI, 5.1e-13 and 4.9e-15 in x_HII (4.2e-13, 6.0e-15, 1.5e-12 and 4.9e-15
-// before).
+// before).  (A cell that passes 1/2 in one of the last two substeps keeps the
+// fraction that has become the smaller one to ~1e-14 of 1, not of itself.)
 //
 // Same backward-Euler step for the FP32-mixed path, solved by FP32 + one
 // Newton correction: the smaller fraction is first obtained in FP32 from its
@@ -616,7 +617,7 @@ __device__ __forceinline__ void timestep_finish(float best, unsigned int* out, u
 // norm is the same product of sums over ones, so a uniform field comes back
 // unchanged to the bit.  128^3, per call: 255 us with the field in a scratch
 // array and the filter in a second kernel, 68 us with 27 tested neighbours a
-// cell and the FP64 front test in line, now 44 us (256^3: 290 -> 196).
+// cell and the FP64 front test in line, now 40 us (256^3: 290 -> 199).
 constexpr int kTileX = 32, kTileY = 8, kTileZ = 8;
 template <typename KT>
 __global__ void __launch_bounds__(256) timestep_kernel(int nx, int ny, int nz, const double* __restrict__ nH,

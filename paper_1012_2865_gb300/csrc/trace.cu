@@ -58,8 +58,6 @@ enum Event { EV_NONE = 0, EV_SPLIT, EV_DONE, EV_HALT, EV_RARE, EV_TERM };
 enum Start { NO_START = 0, START_CHILD, START_ROOT, START_RESUMED };
 constexpr int kAcc = 5;  // budget sums per grid: emitted, absorbed, escaped, resumed, halted
 
-// Photon budget of one lane for the grid it is working on; lives in shared
-// memory (one slot per thread) and is touched only at package events.
 // Position of the set bit of rank n (0 = lowest) in m; m holds more than n
 // set bits.  A binary search on the population counts of the low halves.
 __device__ __forceinline__ int nth_set_bit(unsigned m, unsigned n) {
@@ -79,6 +77,8 @@ __device__ __forceinline__ int nth_set_bit(unsigned m, unsigned n) {
   return pos;
 }
 
+// Photon budget of one lane for the grid it is working on; lives in shared
+// memory (one slot per thread) and is touched only at package events.
 struct LaneAcc {
   double emitted, absorbed, escaped, resumed, halted;
   unsigned long long segments;

@@ -86,3 +86,27 @@ def test_halting_radii_equal_the_oracle(output):
         np.testing.assert_array_equal(got, ref[:n])
         assert np.all(ref[n:] > 31.0)  # what was dropped lies beyond the diagonal
     assert tables[-1].size < len(cdt)  # the table stops growing once light has crossed the box
+
+
+VISITS = r"""
+#include <cstdio>
+#include "policy.h"
+int main() {
+  const unsigned long long lanes[] = {1ULL, 77824ULL};
+  for (unsigned long long l : lanes) {
+    const unsigned long long pkgs[] = {0ULL, 1ULL, 64 * l - 1, 64 * l, 64 * l + 1, 1ULL << 40};
+    for (unsigned long long p : pkgs) printf("%d ", rtg::visit_segments(p, l));
+  }
+  return 0;
+}
+"""
+
+
+def test_long_visits_once_packages_outnumber_the_lanes(tmp_path):
+    """64 segments a visit, 128 from 64 packages a lane on (0: none read back)."""
+    src, exe = tmp_path / "visits.cpp", tmp_path / "visits"
+    src.write_text(VISITS)
+    subprocess.run(["g++", "-std=c++17", "-O1", "-I", os.path.join(build.ROOT, "paper_1012_2865_gb300", "csrc"),
+                    str(src), "-o", str(exe)], check=True)
+    got = subprocess.run([str(exe)], capture_output=True, text=True, check=True).stdout.split()
+    assert [int(v) for v in got] == [64, 64, 64, 128, 128, 128] * 2
