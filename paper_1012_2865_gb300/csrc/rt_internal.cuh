@@ -69,7 +69,7 @@ enum FlightMode {
 struct __align__(16) SourceDev {
   // FP32 view (mixed path), one 16-byte load each
   float4 k32;     // sdx, w, rw, heat (see the FP64 fields)
-  float4 s32;     // position as FP32 pair, high part; .w = 1 if exact32
+  float4 s32;     // position as FP32 pair, high part; .w = 45-degree ties (fill_position32)
   float4 slo32;   // low part (s - s32); .w = sdx - k32.x
   float4 sabs32;  // 2^-46 |s| where the pair does not hold s exactly, else 0; .w = p0
   float4 sb32;    // s - sa as FP32 pairs (sb32, sblo32), sa the integer nearest s
@@ -97,7 +97,13 @@ struct __align__(16) SourceDev {
 // at least 1/16 apart.
 inline bool exact_in_f32(double v) { return v == ldexp(floor(ldexp(v, 4)), -4) && fabs(v) <= 4096.0; }
 
-// The FP32 view of a source's position from S.s (and S.exact32).
+// The FP32 view of a source's position from S.s (and S.exact32), and which of its
+// 45-degree rays (equal cosines in x and y) meet x and y planes at exactly equal
+// distances: those of equal signs (1) where s_x - s_y is an integer, those of
+// opposite signs (2) where s_x + s_y is.  The distances' numerators are then the
+// same real number, so FP64 rounds them and the quotients alike; where they are
+// not equal they lie a cell apart, which is more than 2^-20 of them on axes of
+// up to 2^19 cells.
 inline void fill_position32(SourceDev& S, int nx, int ny, int nz, double p0) {
   int exact = 1;
   float hi[3], lo[3], ab[3], bh[3], bl[3];
@@ -113,7 +119,10 @@ inline void fill_position32(SourceDev& S, int nx, int ny, int nz, double p0) {
     exact &= exact_in_f32(S.s[a]) ? 1 : 0;
   }
   S.exact32 = exact && nx <= 4096 && ny <= 4096 && nz <= 4096;
-  S.s32 = make_float4(hi[0], hi[1], hi[2], S.exact32 ? 1.0f : 0.0f);
+  const double b0 = S.s[0] - S.sa[0], b1 = S.s[1] - S.sa[1];  // exact, in [-1/2, 1/2]
+  const bool halves = fabs(b0) == 0.5 && fabs(b1) == 0.5, short_axes = nx <= 1 << 19 && ny <= 1 << 19;
+  const int ties = !short_axes ? 0 : (halves || b0 == b1 ? 1 : 0) + (halves || b0 == -b1 ? 2 : 0);
+  S.s32 = make_float4(hi[0], hi[1], hi[2], (float)ties);
   S.slo32 = make_float4(lo[0], lo[1], lo[2], (float)(S.sdx - (double)(float)S.sdx));
   S.sabs32 = make_float4(ab[0], ab[1], ab[2], (float)p0);
   S.sb32 = make_float4(bh[0], bh[1], bh[2], 0.0f);

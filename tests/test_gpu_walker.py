@@ -114,3 +114,26 @@ def test_lengths_along_a_diagonal_in_the_general_form():
     np.testing.assert_array_equal(b["counts"], o["counts"])
     length = o["kph"][o["kph"] > 0].mean()
     np.testing.assert_allclose(r["kph"], o["kph"], rtol=1e-6, atol=1e-6 * length)
+
+
+T3 = 16.0 / 3.0
+
+
+@pytest.mark.parametrize("xlo", [0.9, 0.0])
+@pytest.mark.parametrize("cells,exact", [
+    ([(T3, T3, 2.1), (T3, T3, 6.9)], True), ([(8.3, 10.3, 3.3)], True), ([(8.3, 5.7, 3.3), (9.7, 4.3, 0.2)], False),
+    ([(0.7, 0.3, 5.1)], True), ([(8.3, 8.7, 2.0)], True), ([(8.3, 4.3, 3.3), (1.0 / 3.0, 4.0 / 3.0, 3.0)], False),
+    ([(8.3, 4.3 + 1e-13, 3.3), (9.7, 4.3 - 1e-14, 2.2)], False), ([(2.5, 9.25, 3.1), (2.5, 9.5, 3.1)], True)],
+    ids=["thirds", "equal", "opposite", "opposite-exact", "opposite-exact-2", "rounded", "near", "lattice-xy"])
+def test_ties_off_the_lattice(cells, exact, xlo):
+    """45-degree rays of sources whose x and y lie equally far from planes: where
+    that holds exactly the ties need no fallback, and where the positions'
+    rounding sets the planes apart by 1e-16 to 1e-13, FP64 decides."""
+    g = _grid((16, 11, 7), cells, xlo)
+    _, b, r = parity.run_gpu(g, "fp32_mixed")
+    parity.assert_trace_parity(g, b, r, parity.run_oracle(g), "fp32_mixed")
+    s = np.asarray(g["pos_cm"]) / (g["box_len_cm"] / 16)  # as the library has them
+    frac = s - np.rint(s)
+    tied = (np.abs(frac[:, 0]) == np.abs(frac[:, 1])).all()
+    if exact and tied:
+        assert b["fallbacks"] == 0
