@@ -91,10 +91,12 @@ struct LaneAcc {
   float Pstart, tau0, tau_err, lim;
   int steps, mask;
   float cover;  // covering factor of the last segment (where traced with one)
-  // 88 bytes = 22 banks: the 8-byte accesses of a half-warp to one field
+  double n[3];  // the direction in FP64, once a decision has needed it (level and pix it is of)
+  uint32_t n_level, n_pix;
+  // 120 bytes = 30 banks: the 8-byte accesses of a half-warp to one field
   // fall on 16 different bank pairs (a 64-byte stride puts them on two)
 };
-static_assert(sizeof(LaneAcc) == 88, "conflict-free stride of the per-lane sums");
+static_assert(sizeof(LaneAcc) == 120, "conflict-free stride of the per-lane sums");
 
 // A block's budget sums per grid for the first kBlkGrids grids of the
 // launch: its rows of TraceArgs.blk (global memory, kBlkRow words per grid)
@@ -571,17 +573,29 @@ __device__ __forceinline__ int dir_pair(const TraceArgs& A, int level, uint32_t 
 
 // Exact (FP64) crossing decision for cell (c0, c1, c2) of package (level,
 // pix) of source src: bit 3 = split, bits 0-2 = axes that reach the next
-// plane first, bit 6 = the crossing lies beyond the halting radius rlim
-// (+inf without a finite speed of light).  Inlined where it is used once: as a
-// call it cost the kernel's caller-saved registers (28 spilled words).
-__device__ __forceinline__ int decide64(const TraceArgs& A, uint32_t src, int level, uint32_t pix, int c0, int c1,
-                                        int c2, double rlim) {
+// plane first, among those of `near` (bits 0-2; the pairs prove the others
+// later), bit 6 = the crossing lies beyond the halting radius rlim (+inf
+// without a finite speed of light).  Inlined where it is used once: as a call it
+// cost the kernel's caller-saved registers (28 spilled words).  The FP64
+// direction is kept with the lane's sums: a ray whose planes nearly tie at every
+// step (a source at x = 5.3, y = 60.3) asks for it as often, and with it formed
+// and three quotients taken each time its trace took 0.27 ms in a neutral 128^3
+// box and 0.95 in an ionised one, now 0.235 and 0.83.
+__device__ __forceinline__ int decide64(const TraceArgs& A, LaneAcc& acc, uint32_t src, int level, uint32_t pix, int c0,
+                                        int c1, int c2, int near, double rlim) {
   const SourceDev& S = A.src[src];
-  double n[3];
-  pix2vec64(level, pix, n);
-  const double u0 = next_t64(c0, S.s[0], n[0]);
-  const double u1 = next_t64(c1, S.s[1], n[1]);
-  const double u2 = next_t64(c2, S.s[2], n[2]);
+  if (acc.n_level != (uint32_t)level || acc.n_pix != pix) {
+    double v[3];
+    pix2vec64(level, pix, v);
+    acc.n[0] = v[0]; acc.n[1] = v[1]; acc.n[2] = v[2];
+    acc.n_level = (uint32_t)level;
+    acc.n_pix = pix;
+  }
+  const double n[3] = {acc.n[0], acc.n[1], acc.n[2]};
+  const double inf = __longlong_as_double(0x7ff0000000000000LL);
+  const double u0 = near & 1 ? next_t64(c0, S.s[0], n[0]) : inf;
+  const double u1 = near & 2 ? next_t64(c1, S.s[1], n[1]) : inf;
+  const double u2 = near & 4 ? next_t64(c2, S.s[2], n[2]) : inf;
   const double rn = fmin(u0, fmin(u1, u2));
   int out = 0;
   if (level < A.max_level && rn > A.rsplit[level]) out |= 8;
@@ -956,7 +970,7 @@ struct Walk32 {
   // leaves the box; rn receives the crossing distance.  Orders that the pairs
   // cannot prove are re-taken in FP64 (decide64) and counted in fb.
   template <bool FSL>
-  __device__ __forceinline__ int decide(const TraceArgs& A, F2& rn, unsigned& fb) const {
+  __device__ __forceinline__ int decide(const TraceArgs& A, LaneAcc& acc, F2& rn, unsigned& fb) const {
     const SourceDev& S = A.src[src];
     int imin = 0;
     rn = a0.t;
@@ -968,10 +982,11 @@ struct Walk32 {
     const float emin = imin == 0 ? b0 : (imin == 1 ? b1 : b2);
     bool m0 = imin == 0, m1 = imin == 1, m2 = imin == 2;
     bool unsure = false;
+    int near = 1 << imin;  // the axes among which the pairs leave the first plane open
     const bool xy_tie = diag_exact();  // planes this close are an exact tie then (see step)
-    if (!m0 && f2_diff(a0.t, rn) <= b0 + emin) { if (imin == 1 && xy_tie) m0 = true; else unsure = true; }
-    if (!m1 && f2_diff(a1.t, rn) <= b1 + emin) { if (imin == 0 && xy_tie) m1 = true; else unsure = true; }
-    if (!m2 && f2_diff(a2.t, rn) <= b2 + emin) unsure = true;
+    if (!m0 && f2_diff(a0.t, rn) <= b0 + emin) { near |= 1; if (imin == 1 && xy_tie) m0 = true; else unsure = true; }
+    if (!m1 && f2_diff(a1.t, rn) <= b1 + emin) { near |= 2; if (imin == 0 && xy_tie) m1 = true; else unsure = true; }
+    if (!m2 && f2_diff(a2.t, rn) <= b2 + emin) { near |= 4; unsure = true; }
     const int l = lvl();
     bool split = false, halt = false;
     if (l < A.max_level) {
@@ -990,7 +1005,7 @@ struct Walk32 {
     if (unsure) {
       const double rlim64 = !FSL ? __longlong_as_double(0x7ff0000000000000LL)
                                  : ((int)age < A.n_ages ? A.rlim64[age] : 0.0);
-      const int d64 = decide64(A, src, l, pix, c0, c1, c2, rlim64);
+      const int d64 = decide64(A, acc, src, l, pix, c0, c1, c2, near, rlim64);
       split = (d64 & 8) != 0;
       halt = (d64 & 64) != 0;
       m0 = (d64 & 1) != 0;
@@ -1146,7 +1161,7 @@ struct Walk32 {
     lim = acc.lim;
     F2 rn;
     unsigned fb = 0;
-    const int m = decide<FSL>(A, rn, fb);
+    const int m = decide<FSL>(A, acc, rn, fb);
     acc.fallbacks += fb;
     if (m & 8) return EV_SPLIT;
     const bool halt = FSL && (m & 64);  // Step 3j: the segment ends at rlim
@@ -1290,6 +1305,7 @@ __global__ void __launch_bounds__(kBlock, MinBlocks) trace_kernel(TraceArgs A) {
   acc.emitted = acc.absorbed = acc.escaped = acc.resumed = acc.halted = 0.0;
   acc.segments = acc.fallbacks = acc.fallbacks_tau = 0;
   acc.inst = -1;
+  acc.n_level = 0xffffffffu;
   if ((threadIdx.x & 31) == 0) sh_idle[threadIdx.x >> 5] = IdleWarp{-1, 0, 256u};
   if (threadIdx.x == 0) sh_epoch = (uint32_t)A.ctl[CTL_EPOCH];
   __syncthreads();

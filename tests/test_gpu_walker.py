@@ -137,3 +137,14 @@ def test_ties_off_the_lattice(cells, exact, xlo):
     tied = (np.abs(frac[:, 0]) == np.abs(frac[:, 1])).all()
     if exact and tied:
         assert b["fallbacks"] == 0
+
+
+def test_near_ties_of_many_packages():
+    """Planes that nearly tie at every step, along each pair of axes, for
+    packages of several levels and sources in one warp: the direction kept for
+    such decisions is the package's own."""
+    cells = [(5.3, 12.3, 3.3), (5.3 + 1e-14, 9.3, 2.7), (1.1, 8.1, 4.1), (8.1, 1.1 + 2e-15, 4.1), (2.7, 9.3, 4.7)]
+    g = _grid((16, 16, 9), cells, 0.0)
+    _, b, r = parity.run_gpu(g, "fp32_mixed", phi_c=3.0)
+    parity.assert_trace_parity(g, b, r, parity.run_oracle(g, phi_c=3.0), "fp32_mixed")
+    assert b["fallbacks"] > 500
